@@ -39,16 +39,16 @@ __device__ __forceinline__ Band band_of(int32_t score, int32_t ie, int32_t je, c
     return q;
 }
 
-// Traceback sort key of a pair of class cls (class-major): pairs whose
-// one-lane slab exceeds small_slab_words first, then the rest, each by
-// falling chunk window (~9 % and ~4 % buckets).  A warp sweeps the widest
-// window of its pairs at every chunk, so pairs of one task should share the
-// width: sorted by it, a task of the 1M-pair batch of 100 x 200 pairs
-// sweeps 1.07x the cells of its pairs' own windows, against 1.24x sorted by
-// rows x width.  Also the one-lane slab words (need) and chunk window (wc)
-// the launch sizing uses.  score <= 0: no alignment (width 0, need 0).
-__device__ __forceinline__ void tb_cost_key(int cls, int32_t score, int32_t ie, int32_t je, int32_t small_slab_words,
-                                            const Scoring &sc, int32_t &key, int32_t &need32, int32_t &wc, bool &big)
+// Traceback sort key of a pair of class cls (class-major): pairs whose chunk
+// window is wider than kTbWide first, then the rest, each by falling chunk
+// window (~9 % and ~4 % buckets).  A warp sweeps the widest window of its
+// pairs at every chunk, so pairs of one task should share the width: sorted
+// by it, a task of the 1M-pair batch of 100 x 200 pairs sweeps 1.07x the
+// cells of its pairs' own windows, against 1.24x sorted by rows x width.
+// Also the one-lane slab words (need) and chunk window (wc) the launch sizing
+// uses.  score <= 0: no alignment (width 0, need 0).
+__device__ __forceinline__ void tb_cost_key(int cls, int32_t score, int32_t ie, int32_t je, const Scoring &sc,
+                                            int32_t &key, int32_t &need32, int32_t &wc, bool &big)
 {
     int64_t need = 0;
     wc = 0;
@@ -59,9 +59,9 @@ __device__ __forceinline__ void tb_cost_key(int cls, int32_t score, int32_t ie, 
         wc = w;
     }
     const float lw = __log2f((float)(wc > 1 ? wc : 1));
-    big = need > small_slab_words;
+    big = wc > kTbWide;
     if (big) {
-        const int cb = min(63, max(0, (int)(8.f * lw) - 32));
+        const int cb = min(63, max(0, (int)(8.f * lw) - 64));
         key = cls * N_NBUCKET + (63 - cb);
     } else {
         const int cb = min(191, max(0, (int)(16.f * lw)));

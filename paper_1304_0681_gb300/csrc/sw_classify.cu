@@ -19,10 +19,12 @@ __global__ void k_classify(PairSet ps, int64_t n_reads, int64_t n_pairs, Scoring
     // at the end: a batch has few classes, and a global atomic per key group
     // would send every warp to the same few addresses
     __shared__ int32_t s_count[N_CLASS], s_max_n[N_CLASS], s_max_m[N_CLASS];
+    __shared__ unsigned long long s_sum_n[N_CLASS];
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         s_count[c] = 0;
         s_max_n[c] = 0;
         s_max_m[c] = 0;
+        s_sum_n[c] = 0;
     }
     __syncthreads();
     // warp-strided so that every lane of a warp takes part in the key groups
@@ -72,11 +74,13 @@ __global__ void k_classify(PairSet ps, int64_t n_reads, int64_t n_pairs, Scoring
         if (key >= 0) {
             const unsigned mx_n = __reduce_max_sync(g.mask, (unsigned)n);
             const unsigned mx_m = __reduce_max_sync(g.mask, (unsigned)m);
+            const unsigned sm_n = __reduce_add_sync(g.mask, (unsigned)n);  // 32 windows of under 2^20 bases
             if (g.rank == 0) {
                 atomicAdd(&hist[key], g.size);
                 atomicAdd(&s_count[cls], g.size);
                 atomicMax(&s_max_n[cls], (int32_t)mx_n);
                 atomicMax(&s_max_m[cls], (int32_t)mx_m);
+                atomicAdd(&s_sum_n[cls], (unsigned long long)sm_n);
             }
         }
     }
@@ -86,6 +90,7 @@ __global__ void k_classify(PairSet ps, int64_t n_reads, int64_t n_pairs, Scoring
             atomicAdd(&info->count[c], s_count[c]);
             atomicMax(&info->max_n[c], s_max_n[c]);
             atomicMax(&info->max_m[c], s_max_m[c]);
+            atomicAdd(&info->sum_n[c], s_sum_n[c]);
         }
 }
 

@@ -9,9 +9,10 @@
 //   k_plan_score  per class the lanes per pair and rows per lane (the cost
 //                 model of score_plan_of), the class's place in the sorted
 //                 order, its score variant (compiled rows x arithmetic
-//                 mode), and the chunk-boundary scratch of classes whose
-//                 reads need several row chunks;
-//   k_plan_tb     per class and part (pairs with big slabs, the rest) the
+//                 mode), the chunk-boundary scratch of classes whose
+//                 reads need several row chunks, and which classes keep row
+//                 checkpoints for the traceback;
+//   k_plan_tb     per class and part (pairs with wide windows, the rest) the
 //                 traceback kernel, its lanes per pair and slab sizes
 //                 (tb_part_shape), and per traceback variant the size of a
 //                 warp's scratch slot and how many warps fit the budget.
@@ -27,10 +28,10 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_score(const ClassInfo *__
                                                              DevScorePlan *__restrict__ out,
                                                              int32_t *__restrict__ status)
 {
-    __shared__ int32_t s_var[N_CLASS], s_cnt[N_CLASS], s_bnd[N_CLASS], s_lanes[N_CLASS];
+    __shared__ int32_t s_var[N_CLASS], s_cnt[N_CLASS], s_bnd[N_CLASS], s_lanes[N_CLASS], s_ck[N_CLASS];
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = info->count[c];
-        int32_t var = -1, bnd = 0, lanes = 1;
+        int32_t var = -1, bnd = 0, lanes = 1, ck = 0;
         if (cnt > 0) {
             const int mode = c / N_MCLASS;
             const int32_t mm = info->max_m[c], mn = info->max_n[c];
@@ -57,11 +58,13 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_score(const ClassInfo *__
             // per group: two buffers x longest window x (H, F) x 4 bytes
             bnd = chunks > 1 ? 16 * mn : 0;
             var = ri * N_MODES + mode;
+            if (pp.ck_bytes > 0 && mode != MODE_I32) ck = ck_block_rows(rows);
         }
         s_var[c] = var;
         s_cnt[c] = cnt;
         s_bnd[c] = bnd;
         s_lanes[c] = lanes;
+        s_ck[c] = ck;
         out->cls_count[c] = cnt;
         out->cls_lanes[c] = lanes;
         out->cls_bnd_bytes[c] = bnd;
@@ -94,6 +97,24 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_score(const ClassInfo *__
                 run += s_cnt[c];
             }
         }
+    }
+    // checkpoints: blocks are doubled until the most they may take fits the
+    // pool (a block of the whole read needs none)
+    {
+        const int64_t limit = min(pp.ck_bytes / 16, (int64_t)0xFFFFFFF0u);
+        int64_t used = 0;
+        int shift = 0;
+        for (;; ++shift) {
+            used = 0;
+            for (int c = lane; c < N_CLASS; c += 32)
+                if (s_ck[c])
+                    used += ck_class_units(s_cnt[c], (int64_t)info->sum_n[c], info->max_m[c], info->max_n[c],
+                                           s_lanes[c], s_ck[c] << shift);
+            for (int d = 16; d; d >>= 1) used += __shfl_xor_sync(0xffffffffu, used, d);
+            if (used <= limit) break;  // at the latest when no read is longer than its block
+        }
+        for (int c = lane; c < N_CLASS; c += 32) out->cls_ck[c] = s_ck[c] << shift;
+        if (lane == 0) out->ck_units = (used + 15) & ~(int64_t)15;  // 256-byte alignment
     }
     int nb = 0;
     int32_t n_v[N_SCORE_VARIANTS];
@@ -141,6 +162,12 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_tb(const ClassInfo *__res
 {
     __shared__ int64_t s_slot[N_TB_PARTS];
     __shared__ int8_t s_pv[N_TB_PARTS];  // each part's variant (-1: none)
+    __shared__ int32_t s_n16;            // pairs of the 16-bit classes
+    if (threadIdx.x == 0) s_n16 = 0;
+    __syncthreads();
+    if (threadIdx.x < N_CLASS && threadIdx.x >= N_MCLASS && info->count[threadIdx.x] > 0)
+        atomicAdd(&s_n16, info->count[threadIdx.x]);
+    __syncthreads();
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = info->count[c];
         const int32_t big = ti->n_big[c];
@@ -156,14 +183,18 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_tb(const ClassInfo *__res
             int64_t slot = 0;
             if (t.count > 0) {
                 const int64_t need = ti->max_need[c] > 1 ? ti->max_need[c] : 1;
-                // a part too small to give a task (64 / T pairs) to a quarter
-                // of the warps of a launch spreads each pair over more lanes
-                // (at most 8): the tasks then finish sooner, which is what a
-                // small batch waits for
-                int min_lanes = 1;
-                while (min_lanes < 8 && (int64_t)t.count * min_lanes < (int64_t)pp.tb_warps[0] * 16) min_lanes *= 2;
-                slot = tb_part_shape(c / N_MCLASS, pp.allow16 != 0, info->max_m[c], need, ti->max_wcap[part][c],
-                                     part, pp.small_slab_words, t, min_lanes);
+                // a batch too small to give a task (64 / T pairs) to a
+                // quarter of the warps of a launch spreads each two pairs
+                // over more lanes, and so does a small part of long reads
+                // (its tasks are many blocks one after another): the tasks
+                // then finish sooner, which is what the call waits for
+                int lanes = part == 0 ? 8 : 1;  // wide windows: see kTbWide
+                const int64_t enough = (int64_t)pp.tb_warps[0] * 16;
+                while (lanes < 8 && ((int64_t)s_n16 * lanes < enough ||
+                                     (info->max_m[c] > 512 && (int64_t)t.count * lanes < enough)))
+                    lanes *= 2;
+                slot = tb_part_shape(c / N_MCLASS, pp.allow16 != 0, sp->cls_ck[c], info->max_m[c], need,
+                                     ti->max_wcap[part][c], part, pp.sc, lanes, t);
             }
             out->part[2 * c + part] = t;
             s_slot[2 * c + part] = slot;
@@ -172,113 +203,49 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_tb(const ClassInfo *__res
     }
     __syncthreads();
     // the first warp finishes: each variant's part list (longest reads
-    // first, big-slab part first), its slot and pool sizes, and the split
+    // first, wide part first), its slot size, and the split
     if (threadIdx.x >= 32) return;
     const int lane = threadIdx.x;
     const unsigned lt = (1u << lane) - 1u;
-    const int PAIRS_OF[N_TB16_VARIANTS] = {64, 32, 16, 8, 4, 2};
-    int32_t n_v[N_TB_VARIANTS];
-    int64_t slot_v[N_TB_VARIANTS], bnd_v[N_TB_VARIANTS], need_v[N_TB_VARIANTS];
+    const int64_t ck_words = 4 * sp->ck_units;
+    const int64_t total = pp.tb_bytes / 4 - ck_words;
     int64_t split16 = 0, split32 = 0;
     for (int v = 0; v < N_TB_VARIANTS; ++v) {
         int32_t n = 0;
-        int64_t slot = 0, bnd = 0, need = 0;
+        int64_t slot = 0;
         for (int q0 = N_TB_PARTS - 1; q0 >= 0; q0 -= 32) {
-            // parts 2c (big) and 2c + 1 of class c, classes descending
+            // parts 2c (wide) and 2c + 1 of class c, classes descending
             const int qi = q0 - lane;
             const int q = qi >= 0 ? (qi ^ 1) : -1;
             const bool hit = q >= 0 && s_pv[q] == v;
-            const TbPartPlan *t = hit ? &out->part[q] : nullptr;
             const unsigned m = __ballot_sync(0xffffffffu, hit);
             if (hit) {
                 out->var_part[v][n + __popc(m & lt)] = (int16_t)q;
                 slot = max(slot, s_slot[q]);
-                if (v < N_TB16_VARIANTS) {
-                    bnd = max(bnd, t->bnd_ints);
-                    need += (int64_t)((t->count + PAIRS_OF[v] - 1) / PAIRS_OF[v]) * 32 * t->slab_words;
-                    split16 += t->count;
-                } else {
-                    split32 += t->count;
-                }
+                (v < N_TB16_VARIANTS ? split16 : split32) += out->part[q].count;
             }
             n += __popc(m);
         }
-        for (int d = 16; d; d >>= 1) {
-            slot = max(slot, __shfl_xor_sync(0xffffffffu, slot, d));
-            bnd = max(bnd, __shfl_xor_sync(0xffffffffu, bnd, d));
-            need += __shfl_xor_sync(0xffffffffu, need, d);
+        for (int d = 16; d; d >>= 1) slot = max(slot, __shfl_xor_sync(0xffffffffu, slot, d));
+        if (lane == 0) {
+            // a slot per warp, as many warps as fit (the launches run one
+            // after another, each with everything the checkpoints leave)
+            const int64_t words = (slot + 63) & ~(int64_t)63;  // 256-byte alignment
+            const int64_t w = n ? min((int64_t)pp.tb_warps[v], total / max(words, (int64_t)1)) : 0;
+            if (n && w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's slot does not fit the scratch
+            out->var_n[v] = n;
+            out->var_slot_words[v] = words;
+            out->var_slot_offset[v] = ck_words;
+            out->var_warps[v] = (int32_t)w;
         }
-        n_v[v] = n;
-        slot_v[v] = slot;
-        bnd_v[v] = bnd;
-        need_v[v] = need;
     }
     for (int d = 16; d; d >>= 1) {
         split16 += __shfl_xor_sync(0xffffffffu, split16, d);
         split32 += __shfl_xor_sync(0xffffffffu, split32, d);
     }
-    if (lane != 0) return;
-    out->split[0] = split16;
-    out->split[1] = split32;
-    // the launches run one after another, each with the whole budget
-    const int64_t total = pp.tb_bytes / 4;
-    auto r64 = [](int64_t x) { return (x + 63) & ~(int64_t)63; };  // 256-byte alignment
-    for (int v = 0; v < N_TB_VARIANTS; ++v) {
-        out->var_n[v] = n_v[v];
-        out->var_slot_offset[v] = 0;
-        out->var_bnd_words[v] = 0;
-        out->var_warps[v] = 0;
-        out->var_run_warps[v] = 0;
-        out->var_slot_words[v] = 0;
-        if (!n_v[v]) continue;
-        if (v >= N_TB16_VARIANTS) {
-            // int32 kernels: a slot per warp, as many warps as fit
-            const int64_t words = r64(slot_v[v]);
-            const int64_t w = min((int64_t)pp.tb_warps[v], total / max(words, (int64_t)1));
-            if (w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's slot does not fit the scratch
-            out->var_slot_words[v] = words;
-            out->var_warps[v] = (int32_t)w;
-            continue;
-        }
-        // 16-bit kernel: boundary rows of the warps that take part, full
-        // slots, then the pool; tiles go to the pool (walked later at full
-        // occupancy) or are swept and walked by warps that hold a full slot
-        int64_t tile = 0;
-        for (int i = 0; i < n_v[v]; ++i) tile = max(tile, 32 * out->part[out->var_part[v][i]].slab_words);
-        const int64_t bnd = r64(bnd_v[v]), need = need_v[v];
-        tile = r64(tile);
-        if (bnd + tile > total) {
-            atomicOr(status, ST_UNSUPPORTED);  // not even one warp's row and slot fit the scratch
-            continue;
-        }
-        // as many warps as fit take part (each with a boundary row), at
-        // least one of them with a full slot
-        const int64_t run = bnd ? min((int64_t)pp.tb_warps[v], (total - tile) / bnd) : (int64_t)pp.tb_warps[v];
-        const int64_t avail = total - run * bnd;  // >= tile
-        // T >= 4: a task has at most 16 walks, cheap next to its sweep, so
-        // every running warp gets a slot if it can and the pool takes the
-        // rest; T <= 2: 32 or 64 walks per task run best in the separate walk
-        // kernel, so the pool comes first (half the space when it cannot
-        // hold every task)
-        int64_t slots;
-        if (v >= 2) slots = max((int64_t)1, min(run, avail / tile));
-        else if (need + tile <= avail) slots = max((int64_t)1, min(run, (avail - need) / tile));
-        else slots = max((int64_t)1, min(run, (avail / 2) / tile));
-        out->var_bnd_words[v] = bnd;
-        out->var_slot_words[v] = tile;
-        out->var_slot_offset[v] = run * bnd;
-        out->var_run_warps[v] = (int32_t)run;
-        out->var_warps[v] = (int32_t)slots;
-        int64_t pool = out->var_slot_offset[v] + slots * tile;
-        for (int i = 0; i < n_v[v]; ++i) {
-            TbPartPlan &t = out->part[out->var_part[v][i]];
-            const int64_t tw = r64(32 * t.slab_words);
-            const int64_t tasks = (t.count + PAIRS_OF[v] - 1) / PAIRS_OF[v];
-            const int64_t fit = min(tasks, (total - pool) / tw);
-            t.pool_tasks = (int32_t)fit;
-            t.pool_offset = pool;
-            pool += fit * tw;
-        }
+    if (lane == 0) {
+        out->split[0] = split16;
+        out->split[1] = split32;
     }
 }
 

@@ -2,11 +2,13 @@
 //
 // The paper's Stage E, task iii returns the alignment itself, not only its
 // score; downstream, long runs of deletions in it mark splice junctions.
-// The score pass keeps no traceback.  This pass recomputes the DP exactly
-// (int32, unfloored E and F) over a region that provably holds every optimal
-// alignment ending at the end cell (i_end, j_end), and walks back through it.
+// The score pass keeps no traceback bits.  This pass recomputes the DP exactly
+// over a region that provably holds every optimal alignment ending at the end
+// cell (i_end, j_end), and walks back through it: the 16-bit kernel (further
+// down) block by block from the score pass's row checkpoints, the int32
+// kernel over the whole read's band.
 //
-// The region.  Any alignment with this score that ends on read row i_end
+// The band of the int32 kernel.  Any alignment with this score that ends on read row i_end
 // holds at most i_end+1 aligned read bases, each worth at most `match`, and
 // with o <= e <= 0 one gap run is the cheapest way to spend gap bases, so
 //   deletions  D <= (match (i_end+1) + o - score) / (-e) + 1
@@ -29,10 +31,10 @@
 // the end cell, writes the runs reversed into the pair's CSR slot and
 // reverses them in place.
 //
-// Scheduling.  The score pass's epilogue gives every pair a cost key (rows x
-// window), a counting sort orders each length class by cost so a warp's
-// groups sweep similar windows, and pairs whose slab exceeds the small slab
-// of the main part form a part of their own with larger slabs.  A device
+// Scheduling.  The score pass's epilogue gives every pair a cost key (its
+// chunk window), a counting sort orders each length class by it so a warp's
+// groups sweep similar windows, and pairs with wide windows form a part of
+// their own with larger slabs.  A device
 // planner (sw_devplan.cu) sizes every part and assigns it to one of the
 // persistent launches below; each warp of a launch owns one scratch slot,
 // sized for the largest part of its launch.
@@ -425,25 +427,44 @@ __global__ void __launch_bounds__(128) k_traceback(const TracebackLaunch L)
 }
 
 // ---------------------------------------------------------------------------
-// 16x2 traceback.  One lane owns two pairs, A in the low and B in the high
-// half of every register, so each DPX instruction recomputes two cells.  It
-// serves the classes whose score bound keeps every value below 32768
-// (match x min(m, n) <= 32000, match - o <= 127).  A lane stores two 32-bit
-// words per window offset (rows 0-3 and rows 4-7; pair A in bits 0-15, pair
-// B in bits 16-31), and its words of four consecutive offsets share one
-// 32-byte sector: uint2 [((chunk x WCAP4 + t / 4) x 32 + lane) x 4 + t % 4].
-// The warp's stores fill each sector over four steps, and a walk moving
-// left along a chunk reads one sector per four offsets.
+// 16x2 traceback, one block of rows at a time.  It serves the classes whose
+// score bound keeps every value below 32768 (match x min(m, n) <= 32000,
+// match - o <= 127).  A group of T lanes owns two pairs, A in the low and B
+// in the high half of every register, so each DPX instruction recomputes two
+// cells.
 //
-// Per cell four bits record which equalities fail (1 = not equal):
+// Blocks.  The score pass kept H and F of every column for the rows that end
+// a block of 40 to 64 read rows (the checkpoints).  A pair's path is at
+// (i, j) with the exact value v of its state; the block of row i is swept
+// from the checkpoint above it (row i0 - 1, or the matrix edge) down to row
+// i over the columns the path can use, the walk goes back through the block
+// until it crosses row i0 or ends, and the next block starts from there.
+//
+// The columns.  A path that enters the block below checkpoint column j' with
+// value h gains at most match per row, and its d = j - j' - (i - i0 + 1)
+// deletions cost at least -o - (d - 1) e, so it can reach v only if
+//   h + match (i - i0 + 1) + o + (d - 1) e >= v.
+// D is the largest such d over the checkpoint's columns (and over paths that
+// start inside the block, h = 0); the insertions are bounded likewise by the
+// largest h.  Row r of the block then needs columns j - (i - r) - D ..
+// j - (i - r) + I only: cells on optimal paths keep their exact values, all
+// others can only come out lower, so every comparison of the walk comes out
+// as in the full matrix.  From the path's side, the rows below r gain at most
+// match each, so no more than (score - v + match (i - r) + o) / -e + 1
+// deletions lie below row r, which narrows the last rows' windows.  The whole
+// read's band is as wide as the loss of the whole read allows; a block's is
+// as wide as its own loss.  Sweeping the 2M uneven pairs of 75 to 800 bases
+// by whole-read bands took 45 ms, plus 7.5 ms for walks in kernels of their
+// own.
+//
+// Sweep.  Lane k of a group holds 8 rows of a chunk of 8T rows on a one-step
+// wavefront.  A lane stores two 32-bit words per window offset (rows 0-3 and
+// rows 4-7; pair A in bits 0-15, pair B in bits 16-31), and its words of four
+// consecutive offsets share one 32-byte sector: uint2
+// [((chunk x S4 + t / 4) x 32 + lane) x 4 + t % 4].  Per cell four bits record
+// which equalities fail (1 = not equal):
 //   bit 0  H != H(i-1,j-1) + s    bit 1  H != E
 //   bit 2  E != H(i,j-1) + o      bit 3  F != H(i-1,j) + o
-// so the walk takes the diagonal where bit 0 is clear, else E where bit 1
-// is clear, else F, and a gap run opens where bit 2 (3) is clear -- the same
-// preferences as the int32 kernel.  Whether H is 0 is not stored: the walk
-// carries the exact value of its current state, starting from the score,
-// and stops where H reaches 0.
-//
 // Each bit is min(x, 1) per half of a difference x that is non-negative in
 // both halves (a maximum minus one of its operands), so the differences and
 // the packing of the bits are integer multiply-adds on the FMA pipe, next to
@@ -451,18 +472,30 @@ __global__ void __launch_bounds__(128) k_traceback(const TracebackLaunch L)
 // instructions when s - o >= 0 for every substitution (FMA_ADD), else the
 // diagonal add and its difference move to the ALU pipe.
 //
-// Each pair keeps its own chunk windows (the clamped band boxes); both pairs
-// of a lane step through window offset t together and the warp steps to its
-// widest window.  Offsets past a pair's own window are computed as well:
-// they lie right of its box and hold values no larger than the full
-// matrix's (past the window end they see an all-(s = o) table, so nothing
-// grows there), which changes no cell the walk reads.  Boundary rows hold
-// (H | F << 16) per pair and offset, read by the next chunk at its own shift.
+// Each pair keeps its own chunk windows; both pairs of a lane step through
+// window offset t together and the warp steps to its widest window.  Offsets
+// past a pair's own window are computed as well: they lie right of its box
+// and hold values no larger than the full matrix's (past the window end they
+// see an all-(s = o) table, so nothing grows there), which changes no cell
+// the walk reads.  Boundary rows between chunks hold (H | F << 16) per pair
+// and offset and are updated in place; the block's checkpoint columns are
+// copied into the same row first.  Windows start at multiples of four
+// columns, so a boundary row is read four offsets at a time, one group of
+// four steps before it is used: a step takes the SM's 16 warps about 560
+// cycles to issue, an L2 load under this traffic longer.  The rows (and the
+// tiles) bypass the L1, which they would overflow; reads, windows and
+// checkpoints then stay in it.
 //
-// A warp sweeps one task (2G pairs) into the tile of its scratch slot and
-// then walks the task's pairs, one thread per pair, while the other warps of
-// the SM keep sweeping: the walk is a chain of dependent loads, mostly from
-// the L2 the sweep just wrote to.
+// Walk.  The path takes the diagonal where bit 0 is clear, else E where bit 1
+// is clear, else F, and a gap run opens where bit 2 (3) is clear.  Whether H
+// is 0 is not stored: the walk carries the exact value of its state, starting
+// from the score, and stops where H reaches 0.  Where the read and window
+// bases are equal the diagonal always holds (H(i,j) <= H(i-1,j-1) + match:
+// dropping the last aligned pair of an alignment that ends at (i,j) leaves
+// one that reaches (i-1,j-1) with the same gap), so the walk skips runs of
+// equal bases 16 at a time and reads the tile at mismatches and gaps only.
+// A lane with two pairs to walk (T = 1) takes a step of each per iteration,
+// their loads in flight together.
 
 __device__ __forceinline__ uint32_t mad_u32(uint32_t a, uint32_t b, uint32_t c)
 {
@@ -480,35 +513,6 @@ __device__ __forceinline__ uint32_t min_u16x2(uint32_t a, uint32_t b)
 
 __device__ __forceinline__ uint32_t splat16(int32_t x) { return ((uint32_t)(uint16_t)(int16_t)x) * 0x10001u; }
 
-// Streams the window bases of one pair, one column per call; past the
-// window end it yields table index 4 (all s = o).
-struct WinStream {
-    uint32_t ww, wn;
-    int64_t apos, aend;
-    __device__ void start(const uint32_t *__restrict__ wins, int64_t a0, int64_t end)
-    {
-        apos = a0;
-        aend = end;
-        ww = wn = 0;
-        if (a0 < end) {
-            const int64_t a1 = (a0 & ~(int64_t)15) + 16;
-            ww = load_bases(wins, a0, (int)lmin(a1 - a0, end - a0));
-            wn = a1 < end ? load_bases(wins, a1, (int)lmin(16, end - a1)) : 0u;
-        }
-    }
-    __device__ __forceinline__ uint32_t next(const uint32_t *__restrict__ wins)
-    {
-        const uint32_t idx = apos < aend ? (ww & 3u) : 4u;
-        ww >>= 2;
-        if (((++apos) & 15) == 0) {
-            ww = wn;
-            const int64_t a2 = apos + 16;
-            wn = a2 < aend ? load_bases(wins, a2, (int)lmin(16, aend - a2)) : 0u;
-        }
-        return idx;
-    }
-};
-
 // Selector nibbles of one row for pair A (bytes 0-1) and pair B (bytes 2-3):
 // the row's base picks its byte of the column table and the high byte
 // replicates its sign; a row without a base takes the sign of byte 0 (0 or
@@ -520,235 +524,64 @@ __device__ __forceinline__ uint32_t sel16(uint32_t xa, uint32_t xb)
     return a | (b << 8);
 }
 
-// Tile geometry of a 16-bit traceback launch: T lanes per group (two pairs),
-// G = 32 / T groups and 2G pairs per task.  Word (chunk c, step t, lane)
-// of a task's tile: uint2 [((c * S4 + t / 4) * 32 + lane) * 4 + t % 4],
-// S4 = ceil((WCAP + T - 1) / 4) groups of four steps per chunk; lane k of a
-// group computes window offset t - k at step t.
-__device__ __forceinline__ int64_t tb16_word(int c, int t, int lane, int S4)
+// Bases pos - 15 .. pos of a packed buffer, base pos in the top two bits
+// (before the buffer's start: zeros).
+__device__ __forceinline__ uint32_t bases_back(const uint32_t *__restrict__ buf, int64_t pos)
 {
-    return ((((int64_t)c * S4 + (t >> 2)) * 32 + lane) << 2) + (t & 3);
+    const int64_t w = pos >> 4;
+    const uint32_t hi = __ldg(buf + w);
+    const uint32_t lo = ((pos & 15) != 15 && w > 0) ? __ldg(buf + w - 1) : 0u;
+    return __funnelshift_rc(lo, hi, 2 * (int)(pos & 15) + 2);
 }
 
-// Collects a CIGAR as the walk emits it (its last run first) and writes it
-// forward into the pair's slot.  The first LB runs emitted -- the whole CIGAR
-// in the common case -- stay in a per-thread buffer and are stored at the
-// end; runs past those are parked at the end of the slot and moved down in
-// batches of loads before stores.  No run is read back from global memory
-// unless the CIGAR has more than LB runs.
-struct FwdCigar {
-    static constexpr int LB = 16;
-    uint32_t *out;
-    int64_t cap;
-    int32_t n;
-    uint32_t op;
-    int32_t len;
-    bool overflow;
-    uint32_t buf[LB];
-    __device__ void push(uint32_t o, int32_t l)
-    {
-        if (l <= 0) return;
-        if (len > 0 && o == op) {
-            len += l;
-            return;
-        }
-        flush();
-        op = o;
-        len = l;
-    }
-    __device__ void flush()
-    {
-        if (len > 0) {
-            const uint32_t run = ((uint32_t)len << 4) | op;
-            if (n >= cap) overflow = true;
-            else if (n < LB) buf[n] = run;
-            else out[cap - 1 - (n - LB)] = run;
-            ++n;
-        }
-        len = 0;
-    }
-    // run e (in emission order) goes to position n - 1 - e
-    __device__ void finish()
-    {
-        if (overflow) return;
-        const int32_t parked = n - LB;
-        if (parked > 0) {
-            const int64_t src = cap - n + LB;  // > 0: every source lies above its target
-            for (int32_t k = 0; k < parked; k += 4) {
-                uint32_t v[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (k + u < parked) v[u] = out[src + k + u];
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (k + u < parked) out[k + u] = v[u];
-            }
-        }
-        const int32_t nb = n < LB ? n : LB;
-        for (int32_t e = 0; e < nb; ++e) out[n - 1 - e] = buf[e];
-    }
+// The pairs of a warp's task, one entry per pair: path position (i, j), the
+// exact value v of its state st (0 H, 1 E, 2 F, -1 no more to do), the
+// current block's first row i0 and band limits D and I, and the CIGAR so far
+// (cn runs written below the slot's end out, then a run of len x op).
+template <int PAIRS>
+struct TaskPairs {
+    int64_t rs[PAIRS], ws[PAIRS], out[PAIRS];
+    uint32_t ck[PAIRS];
+    int32_t ck_row[PAIRS];
+    int32_t p[PAIRS], n[PAIRS], S[PAIRS], cap[PAIRS];
+    int32_t i[PAIRS], j[PAIRS], v[PAIRS], st[PAIRS];
+    int32_t i0[PAIRS], D[PAIRS], I[PAIRS];
+    int32_t cn[PAIRS], op[PAIRS], len[PAIRS];
 };
 
-// Walk back from a pair's end cell through the tile of its task (group g,
-// 16-bit half `half`), carrying the exact value of the current state (the
-// tile does not record where H is 0), and write its CIGAR.  A walk keeps the
-// sector of four steps it read last, and the 16-base words of read and
-// window that hold its current row and column.  SAME_KERNEL: the tile was
-// written by this warp in this launch (ordered by __syncwarp) and is read
-// through L2 (ld.global.cg), since the slot is reused by the warp's next
-// task; else it was written by an earlier launch and is read through the
-// read-only cache, where walks of neighbouring groups share 128-byte lines.
-// The walk's CIGAR writer is a separate object (its run buffer is indexed,
-// so it lives in local memory, while the walk's own state stays in
-// registers).
-template <int T, bool SAME_KERNEL>
-struct Walk16 {
-    const uint2 *tile;
-    TbPair qq;
-    int32_t p, i, jj, v;
-    int g, hs, S4, state, cc, clo, chi;
-    int64_t gkey, rkey, wkey, it, limit;
-    uint4 ga, gb;
-    uint32_t rw, ww;
-    bool ok;
+// num / d for d >= 1 (the common gap extension of 1 needs no division).
+__device__ __forceinline__ int32_t div_by(int32_t num, int32_t d) { return d == 1 ? num : num / d; }
 
-    // false when there is nothing to walk (no alignment: 0 runs written)
-    __device__ __forceinline__ bool begin(const TbParams &P, FwdCigar &cg, const uint2 *__restrict__ tile_,
-                                          int32_t p_, int g_, int half, int WCAP, int64_t lane_chunks)
-    {
-        constexpr int rc = T * TB_ROWS;
-        tile = tile_;
-        p = p_;
-        g = g_;
-        hs = 16 * half;
-        S4 = (WCAP + T - 1 + 3) >> 2;
-        qq = tb_pair(P, p, nullptr);
-        // the sweep skipped (and reported) pairs that overrun the tile
-        if ((qq.rows + rc - 1) / rc > lane_chunks || min(qq.W, rc + (qq.b - qq.a)) > WCAP) qq.score = 0;
-        if (qq.score <= 0) {
-            P.cig_n[p] = 0;
-            return false;
-        }
-        const int64_t off = P.cig_off[p];
-        cg.out = P.cig_ops + off;
-        cg.cap = P.cig_off[p + 1] - off;
-        cg.n = 0;
-        cg.op = 0u;
-        cg.len = 0;
-        cg.overflow = false;
-        cg.push(4u, qq.m - 1 - qq.ie);  // trailing soft clip
-        i = qq.ie;
-        jj = qq.W - 1;
-        v = qq.score;  // value of the current state at (i, jj)
-        state = 0;
-        cc = i / rc;
-        chunk_window(qq, cc, rc, clo, chi);
-        gkey = rkey = wkey = -1;
-        ga = gb = make_uint4(0u, 0u, 0u, 0u);
-        rw = ww = 0u;
-        ok = false;
-        // every step moves, or switches into a gap state before moving
-        limit = 2 * ((int64_t)qq.rows + qq.W) + 4;
-        it = 0;
-        return true;
-    }
+// Most deletions an alignment part can hold that may lose `num` more than
+// the opening of one gap (num < 0: none); -ge = nge = 0: no limit.
+__device__ __forceinline__ int32_t max_del(int32_t num, int32_t nge)
+{
+    if (nge == 0) return 1 << 24;
+    return num < 0 ? 0 : div_by(num, nge) + 1;
+}
 
-    // one step; false when the walk is over (done, or inconsistent)
-    __device__ __forceinline__ bool step(const TbParams &P, FwdCigar &cg)
-    {
-        constexpr int rc = T * TB_ROWS;
-        if (it++ >= limit) return false;
-        if (state == 0 && v == 0) {
-            ok = true;
-            return false;
-        }
-        if (i < 0 || jj < 0 || v < 0) return false;
-        if (i < cc * rc) {
-            cc = i / rc;
-            chunk_window(qq, cc, rc, clo, chi);
-        }
-        if (jj < clo || jj > chi) return false;  // left the band: inconsistent
-        const int kk = (i - cc * rc) >> 3, r = i & 7;
-        const int t = (jj - clo) + kk;
-        const int64_t sector = ((int64_t)cc * S4 + (t >> 2)) * 32 + g * T + kk;
-        if (sector != gkey) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(tile + (sector << 2));
-            if (SAME_KERNEL) {  // written by this warp in this launch: through L2
-                ga = __ldcg(src);
-                gb = __ldcg(src + 1);
-            } else {            // written by an earlier launch: the read-only path
-                ga = __ldg(src);
-                gb = __ldg(src + 1);
-            }
-            gkey = sector;
-        }
-        const int sl = t & 3;
-        const uint32_t wlo = sl == 0 ? ga.x : sl == 1 ? ga.z : sl == 2 ? gb.x : gb.z;
-        const uint32_t whi = sl == 0 ? ga.y : sl == 1 ? ga.w : sl == 2 ? gb.y : gb.w;
-        const uint32_t code = ((r < 4 ? wlo : whi) >> (hs + 4 * (r & 3))) & 0xFu;
-        if (state == 0) {
-            if (!(code & 1u)) {
-                // diagonal: H(i-1, j-1) = H(i, j) - s(r_i, w_j)
-                const int64_t rpos = qq.rs + i, wpos = qq.ws + qq.jlo + jj;
-                if ((rpos >> 4) != rkey) {
-                    rkey = rpos >> 4;
-                    rw = __ldg(P.ps.reads + rkey);
-                }
-                if ((wpos >> 4) != wkey) {
-                    wkey = wpos >> 4;
-                    ww = __ldg(P.ps.wins + wkey);
-                }
-                const uint32_t ri = (rw >> (2 * (rpos & 15))) & 3u;
-                const uint32_t wj = (ww >> (2 * (wpos & 15))) & 3u;
-                v -= ri == wj ? P.sc.ma : P.sc.mi;
-                cg.push(0u, 1);
-                --i;
-                --jj;
-            } else {
-                state = (code & 2u) ? 2 : 1;
-            }
-        } else if (state == 1) {
-            cg.push(2u, 1);
-            if (!(code & 4u)) {
-                v -= P.sc.go;  // E(i,j) = H(i,j-1) + o
-                state = 0;
-            } else {
-                v -= P.sc.ge;  // E(i,j) = E(i,j-1) + e
-            }
-            --jj;
-        } else {
-            cg.push(1u, 1);
-            if (!(code & 8u)) {
-                v -= P.sc.go;  // F(i,j) = H(i-1,j) + o
-                state = 0;
-            } else {
-                v -= P.sc.ge;
-            }
-            --i;
-        }
-        return true;
-    }
+// First window column (a multiple of 4) of the rows from r0 on of a block
+// entered at (i, j) with value v: D deletions at most, and no more than the
+// rows below r0 can pay for.
+__device__ __forceinline__ int32_t block_lo(int32_t i, int32_t j, int32_t v, int32_t D, int32_t S, int32_t r0,
+                                            const Scoring &sc)
+{
+    const int32_t back = i - r0;
+    const int32_t d = min(D, max_del(S - v + sc.ma * back + sc.go, -sc.ge));
+    return max(0, j - back - d) & ~3;
+}
 
-    __device__ __forceinline__ void end(const TbParams &P, FwdCigar &cg, int32_t *status)
-    {
-        if (!ok) atomicOr(status, ST_INTERNAL);
-        cg.push(4u, i + 1);  // leading soft clip
-        cg.flush();
-        if (cg.overflow) {
-            P.cig_n[p] = -1;
-            atomicOr(status, ST_CAPACITY);
-        } else {
-            cg.finish();
-            P.cig_n[p] = cg.n;
-        }
-    }
-};
+__device__ __forceinline__ uint32_t quad_at(const uint4 &q, int s)
+{
+    return s == 0 ? q.x : s == 1 ? q.y : s == 2 ? q.z : q.w;
+}
 
 template <int T, bool FMA_ADD>
 __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
 {
     constexpr int G = 32 / T;       // groups per warp, two pairs each
     constexpr int PAIRS = 2 * G;    // pairs per task
+    constexpr int rc = T * TB_ROWS; // rows per chunk
     const TbParams &P = L.P;
     // s_tab[w] byte x = s(x, w) - o; s_tab[4] = 0 (s = o, past a window end)
     __shared__ uint32_t s_tab[8];
@@ -767,361 +600,557 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
     // input already found invalid (an unsupported size means some pairs were
     // not scored, so the traceback order is incomplete): do nothing
     if (*(volatile const int32_t *)L.status & (ST_BAD_INPUT | ST_UNSUPPORTED)) return;
-    // the warp's boundary row, and its full slot for tasks it also walks
-    if (warp_global >= dp.var_run_warps[v]) return;
-    uint32_t *const bnd = L.slab + warp_global * dp.var_bnd_words[v];
-    const bool has_slot = warp_global < dp.var_warps[v];
-    uint2 *const own = (uint2 *)(L.slab + dp.var_slot_offset[v] + warp_global * dp.var_slot_words[v]);
-    const int32_t go = P.sc.go, ge = P.sc.ge;
-    const uint32_t GE2 = splat16(ge), GO2 = splat16(go);
+    if (warp_global >= dp.var_warps[v]) return;  // no scratch slot
+    uint32_t *const slot = L.slab + dp.var_slot_offset[v] + warp_global * dp.var_slot_words[v];
+    const uint32_t GE2 = splat16(P.sc.ge), GO2 = splat16(P.sc.go);
     const uint32_t one = (uint32_t)L.one;
     const uint32_t m1 = 0u - one, two = one + one, four = two + two, eight = four + four;
     const uint32_t mul1 = eight + eight, mul2 = mul1 * mul1, mul3 = mul2 * mul1;  // 16, 256, 4096
     const uint32_t ONES = 0x00010001u;
 
-    constexpr int rc = T * TB_ROWS;
-    // The part's and phase's values live in shared memory, one record per
-    // warp, read where they are used (held in registers across the sweep
-    // they would crowd out the sweep's own).
+    __shared__ TaskPairs<PAIRS> s_task[4];  // 128 threads: 4 warps
+    TaskPairs<PAIRS> &tp = s_task[threadIdx.x >> 5];
+    // The part's values live in shared memory, one record per warp, read
+    // where they are used (held in registers across the sweep they would
+    // crowd out the sweep's own).
     struct PartCtx {
         const int32_t *order;
-        int32_t *ctr;        // the phase's work counter
-        uint32_t *pool;      // the part's first pooled tile
-        int64_t n_items, lo, hi, tile_words, lane_chunks;
-        int32_t wcap, s4, pi, phase;
+        int32_t *ctr;
+        uint4 *bnd;
+        int64_t lane_chunks;
+        int32_t n_items, wcap, s4, block_rows, pi;
     };
-    __shared__ PartCtx s_pc[4];  // 128 threads: 4 warps
+    __shared__ PartCtx s_pc[4];
     volatile PartCtx *const pc = &s_pc[threadIdx.x >> 5];
     if (lane == 0) pc->pi = 0;
     __syncwarp();
     for (; pc->pi < dp.var_n[v]; __syncwarp(), pc->pi = pc->pi + (lane == 0 ? 1 : 0), __syncwarp()) {
-    // tasks 0 .. pool_tasks-1 keep their tiles (32 lanes x slab words) in the
-    // pool for k_tb16_walk; the rest are swept into the warp's own slot and
-    // walked at once.  The boundary row is updated in place: (H | F << 16) of
-    // pair x at offset j in word (j * G + g) * 2 + x.
     if (lane == 0) {
-        const TbPartPlan &tp = dp.part[dp.var_part[v][pc->pi]];
-        const int32_t s4 = (tp.wcap + T - 1 + 3) >> 2;
-        pc->order = L.order + tp.start;
-        pc->pool = L.slab + tp.pool_offset;
-        pc->n_items = tp.count;
-        pc->tile_words = (32 * tp.slab_words + 63) & ~(int64_t)63;
-        pc->lane_chunks = tp.slab_words / (8 * (int64_t)max(s4, 1));
-        pc->wcap = tp.wcap;
+        const TbPartPlan &pp = dp.part[dp.var_part[v][pc->pi]];
+        const int32_t s4 = (pp.wcap + T - 1 + 3) >> 2;
+        pc->order = L.order + pp.start;
+        pc->ctr = L.work_counter + 2 * pp.cls + pp.part;
+        pc->bnd = (uint4 *)(slot + ((32 * pp.slab_words + 63) & ~(int64_t)63));
+        pc->lane_chunks = pp.slab_words / (8 * (int64_t)max(s4, 1));
+        pc->n_items = pp.count;
+        pc->wcap = pp.wcap;
         pc->s4 = s4;
-        pc->phase = 0;
+        pc->block_rows = pp.block_rows;
     }
     __syncwarp();
 
-    for (; pc->phase < 2; __syncwarp(), pc->phase = pc->phase + (lane == 0 ? 1 : 0), __syncwarp()) {
-    if (pc->phase == 1 && !has_slot) break;
-    if (lane == 0) {
-        const TbPartPlan &tp = dp.part[dp.var_part[v][pc->pi]];
-        const int64_t n_pool = min((int64_t)tp.count, (int64_t)tp.pool_tasks * PAIRS);
-        const bool ph = pc->phase != 0;
-        pc->ctr = L.work_counter + (ph ? CTR_TB_OWN - CTR_TB : 0) + 2 * tp.cls + tp.part;
-        pc->lo = ph ? n_pool : 0;
-        pc->hi = ph ? (int64_t)tp.count : n_pool;
-    }
-    __syncwarp();
-    const bool own_task = pc->phase != 0;
     for (;;) {
-        int bb = 0;
-        if (lane == 0) bb = atomicAdd(pc->ctr, PAIRS);
-        bb = __shfl_sync(FULLMASK, bb, 0);
-        const int64_t base = pc->lo + bb;
-        if (base >= pc->hi) break;
-        uint2 *const slab = own_task ? own : (uint2 *)(pc->pool + (int64_t)(bb / PAIRS) * pc->tile_words);
-        const int WCAP = pc->wcap;
-        const int64_t lane_chunks = pc->lane_chunks;
-        TbPair q[2];
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const int64_t item = base + 2 * g + x;
-            const int32_t p = item < pc->n_items ? pc->order[item] : -1;
-            q[x] = tb_pair(P, p, k == 0 ? L.status : nullptr);
-            const bool over = (q[x].rows + rc - 1) / rc > lane_chunks || min(q[x].W, rc + (q[x].b - q[x].a)) > WCAP;
-            if (q[x].score > 0 && over) {
-                // the launch was sized from the class maxima; never overrun
-                if (k == 0) atomicOr(L.status, ST_INTERNAL);
-                q[x].score = 0;
-                q[x].rows = 0;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(pc->ctr, PAIRS);
+        base = __shfl_sync(FULLMASK, base, 0);
+        if (base >= pc->n_items) break;
+        for (int wi = lane; wi < PAIRS; wi += 32) {
+            const int32_t p = base + wi < pc->n_items ? pc->order[base + wi] : -1;
+            const TbPair q = tb_pair(P, p, L.status);
+            tp.p[wi] = p;
+            tp.rs[wi] = q.rs;
+            tp.ws[wi] = q.ws;
+            tp.n[wi] = q.n;
+            tp.S[wi] = tp.v[wi] = q.score;
+            tp.i[wi] = q.ie;
+            tp.j[wi] = q.je;
+            tp.st[wi] = q.score > 0 ? 0 : -1;
+            tp.cn[wi] = 0;
+            tp.op[wi] = 4;  // trailing soft clip
+            tp.len[wi] = q.m - 1 - q.ie;
+            tp.ck[wi] = 0;
+            tp.ck_row[wi] = 0;
+            const int64_t o0 = p >= 0 ? P.cig_off[p] : 0, o1 = p >= 0 ? P.cig_off[p + 1] : 0;
+            tp.out[wi] = o1;
+            tp.cap[wi] = (int32_t)lmin(o1 - o0, INT32_MAX);
+            if (p >= 0 && q.score <= 0) P.cig_n[p] = 0;
+            if (q.score > 0 && pc->block_rows) {
+                const uint2 c = P.ck_pos[p];
+                tp.ck[wi] = c.x;
+                tp.ck_row[wi] = (int32_t)c.y;
             }
         }
-        const int32_t rows_l = max(q[0].score > 0 ? q[0].rows : 0, q[1].score > 0 ? q[1].rows : 0);
-        const int32_t rows_w = __reduce_max_sync(FULLMASK, (unsigned)rows_l);
-        const int chunks = (rows_w + rc - 1) / rc;
+        __syncwarp();
 
-        int prev_lo[2] = {0, 0};
-        int prev_width = 0;  // offsets the previous chunk's last lanes wrote
-        for (int c = 0; c < chunks; ++c) {
-            int lo[2], hi[2];
-#pragma unroll
+        for (;;) {
+            // the next block of every pair that is not done: its first row
+            // and band limits
+            bool any = false, any_top = false;
+            int rows_l = 0;
+#pragma unroll 1
             for (int x = 0; x < 2; ++x) {
-                lo[x] = 0;
-                hi[x] = -1;
-                if (q[x].score > 0 && c * rc < q[x].rows) chunk_window(q[x], c, rc, lo[x], hi[x]);
+                const int wi = 2 * g + x;
+                const bool act = tp.st[wi] >= 0;
+                const int32_t i = tp.i[wi], j = tp.j[wi], vv = tp.v[wi], S = tp.S[wi];
+                const int32_t br = pc->block_rows, ma = P.sc.ma, go = P.sc.go, nge = -P.sc.ge;
+                const int32_t blk = act && br ? i / br : 0;
+                const int32_t i0 = blk * br;
+                const int32_t nrow = act ? i - i0 + 1 : 0;
+                const int32_t gain = ma * nrow - vv;
+                int32_t D = max_del(gain + go, nge), M = 0;
+                if (act && i0 > 0) {
+                    const int32_t dcap = max_del(gain + go + min(S, ma * i0), nge);
+                    const int32_t jmin = max(0, j - nrow - dcap);
+                    const uint4 *row = P.ck_pool + tp.ck[wi] + (int64_t)(blk - 1) * (tp.ck_row[wi] >> 1);
+                    const int sh = 16 * (tp.ck_row[wi] & 1);
+#pragma unroll 4
+                    for (int u = (j >> 1) - k; u >= (jmin >> 1); u -= T) {
+                        const uint4 q = __ldg(row + u);
+                        const int32_t h0 = (int32_t)((q.x >> sh) & 0xFFFFu), h1 = (int32_t)((q.z >> sh) & 0xFFFFu);
+                        M = max(M, max(h0, h1));
+                        const int32_t d = j - 2 * u - nrow;
+                        if (d >= 1 && (d - 1) * nge <= gain + go + h0) D = max(D, d);
+                        if (d >= 2 && (d - 2) * nge <= gain + go + h1) D = max(D, d - 1);
+                    }
+                }
+#pragma unroll
+                for (int o = 1; o < T; o <<= 1) {
+                    D = max(D, __shfl_xor_sync(FULLMASK, D, o));
+                    M = max(M, __shfl_xor_sync(FULLMASK, M, o));
+                }
+                const int32_t inum = i0 > 0 ? gain + M : gain + go + nge;
+                __syncwarp();
+                if (act && k == 0) {
+                    tp.i0[wi] = i0;
+                    tp.D[wi] = D;
+                    tp.I[wi] = inum < 0 ? 0 : inum / (ma + nge);
+                    if ((nrow + rc - 1) / rc > pc->lane_chunks) {  // never overrun the tile
+                        atomicOr(L.status, ST_INTERNAL);
+                        P.cig_n[tp.p[wi]] = 0;
+                        tp.st[wi] = -1;
+                    }
+                }
+                __syncwarp();
+                if (tp.st[wi] >= 0) {
+                    any = true;
+                    any_top |= i0 > 0;
+                    rows_l = max(rows_l, nrow);
+                }
             }
-            const int width = __reduce_max_sync(FULLMASK, (unsigned)max(max(hi[0] - lo[0] + 1, hi[1] - lo[1] + 1), 0));
-            const int steps = width + T - 1;
-            const int i0 = c * rc + k * TB_ROWS;
-            uint32_t sel[TB_ROWS];
-            {
-                uint32_t codes[2];
+            if (!__any_sync(FULLMASK, any)) break;
+            any_top = __any_sync(FULLMASK, any_top);
+            const int chunks = ((int)__reduce_max_sync(FULLMASK, (unsigned)rows_l) + rc - 1) / rc;
+
+            int prev_lo[2] = {0, 0};
+            int prev_groups = 0;  // groups of four offsets of the boundary row that hold values
+            for (int c = 0; c < chunks; ++c) {
+                int lo[2], hi[2], rem[2];
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    codes[x] = 0x44444444u;  // 4 bits per row, 4 = no base
-                    const int cnt = min(TB_ROWS, q[x].rows - i0);
-                    if (q[x].score > 0 && cnt > 0) {
-                        const uint32_t w = load_bases(P.ps.reads, q[x].rs + i0, cnt);
-#pragma unroll
-                        for (int r = 0; r < TB_ROWS; ++r)
-                            if (r < cnt) codes[x] = (codes[x] & ~(0xFu << (4 * r))) | (((w >> (2 * r)) & 3u) << (4 * r));
+                    const int wi = 2 * g + x;
+                    lo[x] = 0;
+                    hi[x] = -1;
+                    rem[x] = 0;
+                    const int32_t i = tp.i[wi], j = tp.j[wi], r0 = tp.i0[wi] + c * rc;
+                    if (tp.st[wi] >= 0 && r0 <= i) {
+                        lo[x] = block_lo(i, j, tp.v[wi], tp.D[wi], tp.S[wi], r0, P.sc);
+                        hi[x] = min(j, j - (i - min(r0 + rc - 1, i)) + tp.I[wi]);
+                        if (hi[x] - lo[x] >= pc->wcap) {  // never overrun the tile or the boundary row
+                            if (k == 0) atomicOr(L.status, ST_INTERNAL);
+                            hi[x] = lo[x] + pc->wcap - 1;
+                        }
+                        rem[x] = tp.n[wi] - lo[x];  // window columns from lo on
                     }
                 }
-#pragma unroll
-                for (int r = 0; r < TB_ROWS; ++r) sel[r] = sel16((codes[0] >> (4 * r)) & 0xFu, (codes[1] >> (4 * r)) & 0xFu);
-            }
-            uint32_t E[TB_ROWS], Hp[TB_ROWS];
-#pragma unroll
-            for (int r = 0; r < TB_ROWS; ++r) {
-                E[r] = 0u;
-                Hp[r] = 0u;
-            }
-            // one boundary row, updated in place: the first lane reads offset
-            // j (two steps ahead, at j + shift, shift >= 0) at step j - 2, the
-            // last lane overwrites it at step j + T - 1
-            const uint32_t *bin = (c > 0 && k == 0) ? bnd : nullptr;
-            uint32_t *bout = (c + 1 < chunks && k == T - 1) ? bnd : nullptr;
-            // a pair's window moves right by shift >= 0 from chunk to chunk; a
-            // pair without rows in this chunk reads the row at shift 0 (its
-            // values are never used)
-            int shift[2];
-#pragma unroll
-            for (int x = 0; x < 2; ++x) shift[x] = hi[x] >= lo[x] ? max(lo[x] - prev_lo[x], 0) : 0;
-            auto bload = [&](int x, int j) -> uint32_t {
-                return (bin && j >= 0 && j < prev_width) ? bin[((int64_t)j * G + g) * 2 + x] : 0u;
-            };
-            // the row above, two offsets ahead: packed (H | F << 16) per pair
-            uint32_t nb[2], nc[2], dg[2];
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                dg[x] = bload(x, shift[x] - 1);
-                nb[x] = bload(x, shift[x]);
-                nc[x] = bload(x, shift[x] + 1);
-            }
-            uint32_t diag_in = prmt(dg[0], dg[1], 0x5410u);
-            WinStream ws[2];
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                const int64_t a0 = q[x].ws + q[x].jlo + lo[x];
-                ws[x].start(P.ps.wins, a0, q[x].score > 0 ? q[x].ws + q[x].n : a0);
-            }
-            uint32_t out_h = 0u, out_f = 0u;
-            int64_t widx = tb16_word(c, 0, lane, pc->s4);   // tile word of step t
-            int64_t bidx = ((int64_t)(0 - k) * G + g) * 2;  // boundary word of offset t - k
-
-            for (int t = 0; t < steps; ++t) {
-                // the row above: from the lane before (its last step), or the
-                // previous chunk's boundary row for the group's first lane
-                uint32_t up_h = T > 1 ? __shfl_up_sync(FULLMASK, out_h, 1) : 0u;
-                uint32_t up_f = T > 1 ? __shfl_up_sync(FULLMASK, out_f, 1) : 0u;
-                if (k == 0) {
-                    up_h = prmt(nb[0], nb[1], 0x5410u);
-                    up_f = prmt(nb[0], nb[1], 0x7632u);
+                // offsets, in groups of four
+                const int groups =
+                    ((int)__reduce_max_sync(FULLMASK, (unsigned)max(max(hi[0] - lo[0] + 1, hi[1] - lo[1] + 1), 0)) +
+                     3) >> 2;
+                const int steps = 4 * groups + T - 1;
+                uint4 *const bnd = pc->bnd + 2 * g;  // group q of pair x at bnd[2 * G * q + x]
+                if (c == 0 && any_top) {
+                    // the checkpoint's columns from lo - 4 on, as a boundary
+                    // row (zeros for a pair whose block starts at row 0)
 #pragma unroll
                     for (int x = 0; x < 2; ++x) {
-                        nb[x] = nc[x];
-                        nc[x] = bload(x, t + 2 + shift[x]);
+                        const int wi = 2 * g + x;
+                        const bool top = hi[x] >= lo[x] && tp.i0[wi] > 0;
+                        const int32_t n = tp.n[wi];
+                        const int sh = 16 * (tp.ck_row[wi] & 1);
+                        const uint4 *row = P.ck_pool + tp.ck[wi] +
+                                           (int64_t)(top ? tp.i0[wi] / pc->block_rows - 1 : 0) * (tp.ck_row[wi] >> 1);
+                        auto hf = [&](uint32_t h, uint32_t f) { return ((h >> sh) & 0xFFFFu) | ((f >> sh) << 16); };
+                        prev_lo[x] = lo[x] - 4;
+#pragma unroll 4
+                        for (int q = k; q <= groups; q += T) {
+                            const int col = lo[x] - 4 + 4 * q;
+                            uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                            if (top && col >= 0 && col < n) {
+                                const uint4 a = __ldg(row + (col >> 1));
+                                const uint4 b = col + 2 < n ? __ldg(row + (col >> 1) + 1) : w;
+                                w.x = hf(a.x, a.y);
+                                if (col + 1 < n) w.y = hf(a.z, a.w);
+                                w.z = hf(b.x, b.y);
+                                if (col + 3 < n) w.w = hf(b.z, b.w);
+                            }
+                            __stcg(bnd + 2 * G * q + x, w);
+                        }
                     }
+                    prev_groups = groups + 1;
+                    __syncwarp();
                 }
-                const int jl = t - k;  // this lane's window offset
-                if (jl >= 0) {
-                    const uint32_t tA = s_tab[ws[0].next(P.ps.wins)];
-                    const uint32_t tB = s_tab[ws[1].next(P.ps.wins)];
-                    uint32_t d0 = diag_in, hu = up_h, f = up_f;
-                    uint32_t w0 = 0u, w1 = 0u;
+                // one boundary row, updated in place: the first lane reads
+                // group q + shift (shift >= 0, in groups) before the last
+                // lane overwrites group q; a pair without rows in this chunk
+                // reads it at shift 0 (its values are never used)
+                const bool has_in = (c > 0 || any_top) && k == 0;
+                const bool has_out = c + 1 < chunks && k == T - 1;
+                int shift[2];
 #pragma unroll
-                    for (int r = 0; r < TB_ROWS; ++r) {
-                        const uint32_t sp = prmt(tA, tB, sel[r]);  // s - o, both pairs
-                        const uint32_t e = __viaddmax_s16x2(E[r], GE2, Hp[r]);
-                        f = __viaddmax_s16x2(f, GE2, hu);
-                        const uint32_t d = FMA_ADD ? mad_u32(d0, one, sp) : __viaddmax_s16x2(d0, sp, 0x80008000u);
-                        const uint32_t u = __vimax3_s16x2(d, e, f);
-                        const uint32_t h = __viaddmax_s16x2_relu(u, GO2, 0u);
-                        const uint32_t nd = FMA_ADD ? min_u16x2(mad_u32(d, m1, u), ONES) : min_u16x2(u ^ d, ONES);
-                        const uint32_t ne = min_u16x2(mad_u32(e, m1, u), ONES);
-                        const uint32_t nE = min_u16x2(mad_u32(Hp[r], m1, e), ONES);
-                        const uint32_t nF = min_u16x2(mad_u32(hu, m1, f), ONES);
-                        uint32_t code = mad_u32(ne, two, nd);
-                        code = mad_u32(nE, four, code);
-                        code = mad_u32(nF, eight, code);
-                        if (r == 0) w0 = code;
-                        else if (r == 4) w1 = code;
-                        else if (r < 4) w0 = mad_u32(code, r == 1 ? mul1 : r == 2 ? mul2 : mul3, w0);
-                        else w1 = mad_u32(code, r == 5 ? mul1 : r == 6 ? mul2 : mul3, w1);
-                        d0 = Hp[r];
-                        Hp[r] = h;
-                        E[r] = e;
-                        hu = h;
+                for (int x = 0; x < 2; ++x) shift[x] = hi[x] >= lo[x] ? max(lo[x] - prev_lo[x], 0) >> 2 : 0;
+                auto bload = [&](int x, int q) -> uint4 {
+                    return has_in && q >= 0 && q < prev_groups ? __ldcg(bnd + 2 * G * q + x)
+                                                               : make_uint4(0u, 0u, 0u, 0u);
+                };
+                // the row above: packed (H | F << 16) of four offsets per pair
+                const uint32_t dg0 = bload(0, shift[0] - 1).w, dg1 = bload(1, shift[1] - 1).w;
+                uint4 nb[2] = {bload(0, shift[0]), bload(1, shift[1])};
+                // the windows' first bases and the rows' (while those loads
+                // are in flight)
+                uint32_t codes[2], ww[2], wn[2];
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    const int wi = 2 * g + x;
+                    ww[x] = 0u;
+                    wn[x] = rem[x] > 0 ? load_bases(P.ps.wins, tp.ws[wi] + lo[x], min(16, rem[x])) : 0u;
+                    codes[x] = 0x44444444u;  // 4 bits per row, 4 = no base
+                    const int row = tp.i0[wi] + c * rc + k * TB_ROWS;
+                    const int cnt = rem[x] > 0 ? min(TB_ROWS, tp.i[wi] - row + 1) : 0;
+                    if (cnt > 0) {
+                        const uint32_t w = load_bases(P.ps.reads, tp.rs[wi] + row, cnt);
+#pragma unroll
+                        for (int r = 0; r < TB_ROWS; ++r)
+                            if (r < cnt)
+                                codes[x] = (codes[x] & ~(0xFu << (4 * r))) | (((w >> (2 * r)) & 3u) << (4 * r));
                     }
-                    // a lane's four consecutive steps share one 32-byte
-                    // sector; pooled tiles stream out (walked much later),
-                    // own tiles stay in L2 for the walk right after
-                    if (own_task) __stcg(slab + widx, make_uint2(w0, w1));
-                    else __stcs(slab + widx, make_uint2(w0, w1));
-                    out_h = hu;
-                    out_f = f;
-                    if (bout) *(uint2 *)(bout + bidx) = make_uint2(prmt(hu, f, 0x5410u), prmt(hu, f, 0x7632u));
-                    diag_in = up_h;
                 }
-                widx += (t & 3) == 3 ? 32 * 4 - 3 : 1;
-                bidx += 2 * G;
+                uint32_t sel[TB_ROWS];
+#pragma unroll
+                for (int r = 0; r < TB_ROWS; ++r)
+                    sel[r] = sel16((codes[0] >> (4 * r)) & 0xFu, (codes[1] >> (4 * r)) & 0xFu);
+                uint32_t E[TB_ROWS], Hp[TB_ROWS];
+#pragma unroll
+                for (int r = 0; r < TB_ROWS; ++r) {
+                    E[r] = 0u;
+                    Hp[r] = 0u;
+                }
+                uint32_t diag_in = prmt(dg0, dg1, 0x5410u);
+                uint32_t out_h = 0u, out_f = 0u;
+                uint4 *tile = (uint4 *)slot + ((int64_t)c * pc->s4 * 32 + lane) * 2;  // sector of steps t0 .. t0 + 3
+
+                for (int t0 = 0; t0 < steps; t0 += 4) {
+                    uint4 nx[2], ob[2];
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) nx[x] = bload(x, shift[x] + (t0 >> 2) + 1);
+#pragma unroll 1
+                    for (int half = 0; half < 2; ++half) {
+                    uint4 wq;
+#pragma unroll
+                    for (int s = 0; s < 2; ++s) {
+                        const int t = t0 + 2 * half + s;
+                        // the row above: from the lane before (its last
+                        // step), or the boundary row for the group's first
+                        // lane
+                        uint32_t up_h = T > 1 ? __shfl_up_sync(FULLMASK, out_h, 1) : 0u;
+                        uint32_t up_f = T > 1 ? __shfl_up_sync(FULLMASK, out_f, 1) : 0u;
+                        if (k == 0) {
+                            const uint32_t a = quad_at(nb[0], s), b = quad_at(nb[1], s);
+                            up_h = prmt(a, b, 0x5410u);
+                            up_f = prmt(a, b, 0x7632u);
+                        }
+                        const int jl = t - k;  // this lane's window offset
+                        uint32_t w0 = 0u, w1 = 0u;
+                        if (T == 1 || jl >= 0) {
+                            if ((T > 1 || s == 0) && (jl & 15) == 0) {
+                                // the next 16 columns' bases, requested 16 columns before
+#pragma unroll
+                                for (int x = 0; x < 2; ++x) {
+                                    ww[x] = wn[x];
+                                    const int left = rem[x] - jl - 16;
+                                    wn[x] = left > 0 ? load_bases(P.ps.wins, tp.ws[2 * g + x] + lo[x] + jl + 16,
+                                                                  min(16, left))
+                                                     : 0u;
+                                }
+                            }
+                            const uint32_t tA = s_tab[jl < rem[0] ? ww[0] & 3u : 4u];
+                            const uint32_t tB = s_tab[jl < rem[1] ? ww[1] & 3u : 4u];
+                            ww[0] >>= 2;
+                            ww[1] >>= 2;
+                            uint32_t d0 = diag_in, hu = up_h, f = up_f;
+#pragma unroll
+                            for (int r = 0; r < TB_ROWS; ++r) {
+                                const uint32_t sp = prmt(tA, tB, sel[r]);  // s - o, both pairs
+                                const uint32_t e = __viaddmax_s16x2(E[r], GE2, Hp[r]);
+                                f = __viaddmax_s16x2(f, GE2, hu);
+                                const uint32_t d =
+                                    FMA_ADD ? mad_u32(d0, one, sp) : __viaddmax_s16x2(d0, sp, 0x80008000u);
+                                const uint32_t u = __vimax3_s16x2(d, e, f);
+                                const uint32_t h = __viaddmax_s16x2_relu(u, GO2, 0u);
+                                const uint32_t nd =
+                                    FMA_ADD ? min_u16x2(mad_u32(d, m1, u), ONES) : min_u16x2(u ^ d, ONES);
+                                const uint32_t ne = min_u16x2(mad_u32(e, m1, u), ONES);
+                                const uint32_t nE = min_u16x2(mad_u32(Hp[r], m1, e), ONES);
+                                const uint32_t nF = min_u16x2(mad_u32(hu, m1, f), ONES);
+                                uint32_t code = mad_u32(ne, two, nd);
+                                code = mad_u32(nE, four, code);
+                                code = mad_u32(nF, eight, code);
+                                if (r == 0) w0 = code;
+                                else if (r == 4) w1 = code;
+                                else if (r < 4) w0 = mad_u32(code, r == 1 ? mul1 : r == 2 ? mul2 : mul3, w0);
+                                else w1 = mad_u32(code, r == 5 ? mul1 : r == 6 ? mul2 : mul3, w1);
+                                d0 = Hp[r];
+                                Hp[r] = h;
+                                E[r] = e;
+                                hu = h;
+                            }
+                            out_h = hu;
+                            out_f = f;
+                            diag_in = up_h;
+                            const uint32_t o0 = prmt(hu, f, 0x5410u), o1 = prmt(hu, f, 0x7632u);
+                            if (T == 1) {
+                                (s == 0 ? ob[0].z : ob[0].w) = o0;
+                                (s == 0 ? ob[1].z : ob[1].w) = o1;
+                            } else if (has_out) {
+                                uint32_t *const w = (uint32_t *)(bnd + 2 * G * (jl >> 2)) + (jl & 3);
+                                __stcg(w, o0);
+                                __stcg(w + 4, o1);
+                            }
+                        }
+                        (s == 0 ? wq.x : wq.z) = w0;
+                        (s == 0 ? wq.y : wq.w) = w1;
+                    }
+                    __stcg(tile + half, wq);
+                    if (half == 0) {
+#pragma unroll
+                        for (int x = 0; x < 2; ++x) {
+                            nb[x].x = nb[x].z;
+                            nb[x].y = nb[x].w;
+                            ob[x].x = ob[x].z;
+                            ob[x].y = ob[x].w;
+                        }
+                    }
+                    }
+                    tile += 64;
+                    if (T == 1 && has_out) {
+                        __stcg(bnd + 2 * G * (t0 >> 2), ob[0]);
+                        __stcg(bnd + 2 * G * (t0 >> 2) + 1, ob[1]);
+                    }
+                    nb[0] = nx[0];
+                    nb[1] = nx[1];
+                }
+                prev_lo[0] = lo[0];
+                prev_lo[1] = lo[1];
+                prev_groups = groups;
+                __syncwarp();
             }
-            prev_lo[0] = lo[0];
-            prev_lo[1] = lo[1];
-            prev_width = width;
-            __syncwarp();
-        }
-        // a task in the warp's own slot: its walks, one thread per pair,
-        // while the other warps of the SM keep sweeping; then the slot is
-        // free for the next task
-        if (own_task) {
-            for (int wi = lane; wi < PAIRS; wi += 32) {
-                const int64_t item = base + wi;
-                if (item >= pc->n_items) break;
-                Walk16<T, true> w;
-                FwdCigar cg;
-                if (w.begin(P, cg, slab, pc->order[item], wi >> 1, wi & 1, pc->wcap, pc->lane_chunks)) {
-                    while (w.step(P, cg)) {
-                    }
-                    w.end(P, cg, L.status);
+
+            // the walks back through the block: lanes 0 and 1 of a group one
+            // pair each, or with T = 1 a lane both of its pairs
+            constexpr int NW = T == 1 ? 2 : 1;
+            int wst_[NW], wi_[NW], i_[NW], j_[NW], v_[NW], cn_[NW], len_[NW], cl_[NW], lo_[NW];
+            uint32_t op_[NW];
+            bool go_[NW], fin_[NW], ok_[NW];
+            bool more = false;
+#pragma unroll
+            for (int x = 0; x < NW; ++x) {
+                const int wi = 2 * g + (T == 1 ? x : min(k, 1));
+                wi_[x] = wi;
+                wst_[x] = tp.st[wi];
+                i_[x] = tp.i[wi];
+                j_[x] = tp.j[wi];
+                v_[x] = tp.v[wi];
+                cn_[x] = tp.cn[wi];
+                len_[x] = tp.len[wi];
+                op_[x] = (uint32_t)tp.op[wi];
+                cl_[x] = -1;
+                lo_[x] = 0;
+                go_[x] = (T == 1 || k < 2) && wst_[x] >= 0;
+                fin_[x] = false;
+                ok_[x] = true;
+                more |= go_[x];
+            }
+            const int S4 = pc->s4, wcap = pc->wcap;
+            auto push = [&](int x, uint32_t o, int32_t l) {
+                if (o == op_[x]) {
+                    len_[x] += l;
+                    return;
                 }
+                if (len_[x] > 0) {  // runs are parked downwards from the slot's end
+                    if (cn_[x] < tp.cap[wi_[x]])
+                        P.cig_ops[tp.out[wi_[x]] - 1 - cn_[x]] = ((uint32_t)len_[x] << 4) | op_[x];
+                    ++cn_[x];
+                }
+                op_[x] = o;
+                len_[x] = l;
+            };
+            // the walk's end, or its exit from the block
+            auto stopped = [&](int x) {
+                if (wst_[x] == 0 && v_[x] == 0) fin_[x] = true;
+                else if (wst_[x] == 1 || i_[x] >= tp.i0[wi_[x]]) {
+                    if (j_[x] >= 0 && v_[x] >= 0) return false;
+                    ok_[x] = false;
+                }
+                return true;
+            };
+#pragma unroll
+            for (int x = 0; x < NW; ++x)
+                if (go_[x] && stopped(x)) go_[x] = false;
+            while (more) {
+                // equal bases: the diagonal
+                uint32_t diff[NW];
+#pragma unroll
+                for (int x = 0; x < NW; ++x) {
+                    const bool need = go_[x] && wst_[x] == 0;
+                    const int64_t r = need ? tp.rs[wi_[x]] + i_[x] : 0, w = need ? tp.ws[wi_[x]] + j_[x] : 0;
+                    diff[x] = bases_back(P.ps.reads, r) ^ bases_back(P.ps.wins, w);
+                }
+                bool cell[NW];  // a cell of the tile decides the next step
+#pragma unroll
+                for (int x = 0; x < NW; ++x) {
+                    cell[x] = go_[x];
+                    if (go_[x] && wst_[x] == 0) {
+                        const int same = min(__clz((int)diff[x]) >> 1, 16);
+                        const int run = min(same, min(i_[x] - tp.i0[wi_[x]], j_[x]) + 1);
+                        if (run > 0) {
+                            push(x, 0u, run);
+                            i_[x] -= run;
+                            j_[x] -= run;
+                            v_[x] -= run * P.sc.ma;
+                            if (stopped(x)) go_[x] = false;
+                            cell[x] = go_[x] && same < 16;
+                        }
+                    }
+                }
+                uint2 word[NW];
+                int row[NW];
+#pragma unroll
+                for (int x = 0; x < NW; ++x) {
+                    row[x] = 0;
+                    word[x] = make_uint2(0u, 0u);
+                    if (cell[x]) {
+                        const int wi = wi_[x];
+                        const int rel = i_[x] - tp.i0[wi], c = rel / rc;
+                        if (c != cl_[x]) {
+                            cl_[x] = c;
+                            lo_[x] = block_lo(tp.i[wi], tp.j[wi], tp.v[wi], tp.D[wi], tp.S[wi], tp.i0[wi] + c * rc,
+                                              P.sc);
+                        }
+                        const int jl = j_[x] - lo_[x], kk = (rel - c * rc) >> 3, t = jl + kk;
+                        row[x] = rel & 7;
+                        if (jl < 0 || jl >= wcap) {  // left the band: inconsistent
+                            ok_[x] = go_[x] = cell[x] = false;
+                        } else {
+                            const int64_t sector = ((int64_t)c * S4 + (t >> 2)) * 32 + g * T + kk;
+                            word[x] = __ldcg((const uint2 *)slot + 4 * sector + (t & 3));
+                        }
+                    }
+                }
+                more = false;
+#pragma unroll
+                for (int x = 0; x < NW; ++x) {
+                    if (cell[x]) {
+                        const uint32_t code =
+                            ((row[x] < 4 ? word[x].x : word[x].y) >> (16 * (wi_[x] & 1) + 4 * (row[x] & 3))) & 0xFu;
+                        if (wst_[x] == 0 && (code & 1u)) wst_[x] = (code & 2u) ? 2 : 1;
+                        if (wst_[x] == 0) {
+                            v_[x] -= P.sc.mi;  // H(i-1, j-1) = H(i, j) - s
+                            push(x, 0u, 1);
+                            --i_[x];
+                            --j_[x];
+                        } else {
+                            // E(i,j) = H(i,j-1) + o or E(i,j-1) + e, and F
+                            // the same way up
+                            const bool del = wst_[x] == 1;
+                            push(x, del ? 2u : 1u, 1);
+                            if (!(code & (del ? 4u : 8u))) wst_[x] = 0;
+                            v_[x] -= wst_[x] == 0 ? P.sc.go : P.sc.ge;
+                            if (del) --j_[x];
+                            else --i_[x];
+                        }
+                        if (stopped(x)) go_[x] = false;
+                    }
+                    more |= go_[x];
+                }
+            }
+#pragma unroll
+            for (int x = 0; x < NW; ++x) {
+                const int wi = wi_[x];
+                if (tp.st[wi] < 0 || (T > 1 && k >= 2)) continue;
+                if (!fin_[x] && (i_[x] < 0 || !ok_[x])) {  // no zero reached: inconsistent
+                    atomicOr(L.status, ST_INTERNAL);
+                    fin_[x] = true;
+                }
+                if (fin_[x]) {
+                    push(x, 4u, i_[x] + 1);  // leading soft clip
+                    push(x, 5u, 0);
+                    const int32_t cn = cn_[x], cap = tp.cap[wi], p = tp.p[wi];
+                    if (cn > cap) {
+                        P.cig_n[p] = -1;
+                        atomicOr(L.status, ST_CAPACITY);
+                    } else {
+                        // the runs stand in order at the slot's end: move them down
+                        uint32_t *const to = P.cig_ops + P.cig_off[p];
+                        const uint32_t *const from = P.cig_ops + tp.out[wi] - cn;
+                        if (to != from)
+                            for (int32_t q = 0; q < cn; ++q) to[q] = from[q];
+                        P.cig_n[p] = cn;
+                    }
+                    wst_[x] = -1;
+                }
+                tp.st[wi] = wst_[x];
+                tp.i[wi] = i_[x];
+                tp.j[wi] = j_[x];
+                tp.v[wi] = v_[x];
+                tp.cn[wi] = cn_[x];
+                tp.op[wi] = (int32_t)op_[x];
+                tp.len[wi] = len_[x];
             }
             __syncwarp();
         }
     }
-    }  // phases
     }  // parts
 }
 
-// The walks of a 16-bit launch's pooled tasks: one thread per pair, at full
-// occupancy (a walk is a chain of dependent loads from tiles long out of L2,
-// so many walks in flight hide the latency).  Item k of a part lives in task
-// k / 2G of the part's pool, group (k % 2G) / 2, half k % 2.
-template <int T>
-__global__ void __launch_bounds__(256, 4) k_tb16_walk(const TracebackLaunch L)
+// A device-planned launch of traceback variant v: the 16-bit kernel with
+// tb16_variant_lanes(v) lanes per two pairs for v < N_TB16_VARIANTS, else the
+// int32 kernel, tiled or with T lanes per pair.  fma: every substitution
+// score minus gap_open is >= 0, so the 16-bit diagonal add can run on the
+// FMA pipe.
+static const void *tb16_kernel(int lanes, bool fma)
 {
-    constexpr int PAIRS = 2 * (32 / T);
-    const TbParams &P = L.P;
-    const DevTbPlan &dp = *L.dp;
-    const int v = L.variant;
-    if (*(volatile const int32_t *)L.status & (ST_BAD_INPUT | ST_UNSUPPORTED)) return;
-    const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    for (int pi = 0; pi < dp.var_n[v]; ++pi) {
-        const TbPartPlan &tp = dp.part[dp.var_part[v][pi]];
-        const int WCAP = tp.wcap;
-        const int S4 = (WCAP + T - 1 + 3) >> 2;
-        const int64_t lane_chunks = tp.slab_words / (8 * (int64_t)max(S4, 1));
-        const int64_t tile_words = (32 * tp.slab_words + 63) & ~(int64_t)63;
-        const int64_t n_pool = min((int64_t)tp.count, (int64_t)tp.pool_tasks * PAIRS);
-        const int32_t *const order = L.order + tp.start;
-        for (int64_t item = tid; item < n_pool; item += nthreads) {
-            const uint2 *tile = (const uint2 *)(L.slab + tp.pool_offset + (item / PAIRS) * tile_words);
-            const int wi = (int)(item % PAIRS);
-            Walk16<T, false> w;
-            FwdCigar cg;
-            if (w.begin(P, cg, tile, order[item], wi >> 1, wi & 1, WCAP, lane_chunks)) {
-                while (w.step(P, cg)) {
-                }
-                w.end(P, cg, L.status);
-            }
-        }
+    switch (lanes) {
+    case 1: return fma ? (const void *)k_traceback16<1, true> : (const void *)k_traceback16<1, false>;
+    case 2: return fma ? (const void *)k_traceback16<2, true> : (const void *)k_traceback16<2, false>;
+    case 4: return fma ? (const void *)k_traceback16<4, true> : (const void *)k_traceback16<4, false>;
+    default: return fma ? (const void *)k_traceback16<8, true> : (const void *)k_traceback16<8, false>;
     }
 }
 
-// A device-planned launch of traceback variant v: the 16-bit kernel with T =
-// 2^v lanes per pair for v < N_TB16_VARIANTS, else the int32 kernel, tiled or
-// with T lanes per pair.  fma: every substitution score minus gap_open is
-// >= 0, so the 16-bit diagonal add can run on the FMA pipe.
+static const void *tb_kernel(int v, bool fma)
+{
+    if (v >= 0 && v < N_TB16_VARIANTS) return tb16_kernel(tb16_variant_lanes(v), fma);
+    if (v == TB_VAR_TILED) return (const void *)k_traceback<true>;
+    if (v == TB_VAR_GROUPED) return (const void *)k_traceback<false>;
+    return nullptr;
+}
+
 int launch_traceback_variant(int v, bool fma, const TracebackLaunch &L, int blocks, cudaStream_t st)
 {
-    if (!L.dp || blocks < 1) return SW_ERR_INTERNAL;
+    const void *fn = tb_kernel(v, fma);
+    if (!fn || !L.dp || blocks < 1) return SW_ERR_INTERNAL;
     TracebackLaunch V = L;
     V.variant = v;
-    switch (v) {
-#define SWGB_TB16(VV, TT)                                                                          \
-    case VV:                                                                                       \
-        if (fma) k_traceback16<TT, true><<<blocks, 128, 0, st>>>(V);                               \
-        else k_traceback16<TT, false><<<blocks, 128, 0, st>>>(V);                                  \
-        break;
-        SWGB_TB16(0, 1)
-        SWGB_TB16(1, 2)
-        SWGB_TB16(2, 4)
-        SWGB_TB16(3, 8)
-        SWGB_TB16(4, 16)
-        SWGB_TB16(5, 32)
-#undef SWGB_TB16
-    case TB_VAR_TILED: k_traceback<true><<<blocks, 128, 0, st>>>(V); break;
-    case TB_VAR_GROUPED: k_traceback<false><<<blocks, 128, 0, st>>>(V); break;
-    default: return SW_ERR_INTERNAL;
-    }
+    void *args[] = {&V};
+    if (cuda_failed(cudaLaunchKernel(fn, dim3(blocks), dim3(128), args, 0, st))) return SW_ERR_CUDA;
     count_launch();
     return launch_status();
-}
-
-int launch_tb_walk_variant(int v, const TracebackLaunch &L, int blocks, cudaStream_t st)
-{
-    if (!L.dp || blocks < 1) return SW_ERR_INTERNAL;
-    TracebackLaunch V = L;
-    V.variant = v;
-    switch (v) {
-    case 0: k_tb16_walk<1><<<blocks, 256, 0, st>>>(V); break;
-    case 1: k_tb16_walk<2><<<blocks, 256, 0, st>>>(V); break;
-    case 2: k_tb16_walk<4><<<blocks, 256, 0, st>>>(V); break;
-    case 3: k_tb16_walk<8><<<blocks, 256, 0, st>>>(V); break;
-    case 4: k_tb16_walk<16><<<blocks, 256, 0, st>>>(V); break;
-    case 5: k_tb16_walk<32><<<blocks, 256, 0, st>>>(V); break;
-    default: return SW_ERR_INTERNAL;
-    }
-    count_launch();
-    return launch_status();
-}
-
-int tb_walk_variant_blocks(int v, int sm_count, int *blocks)
-{
-    const void *fn = nullptr;
-    switch (v) {
-    case 0: fn = (const void *)k_tb16_walk<1>; break;
-    case 1: fn = (const void *)k_tb16_walk<2>; break;
-    case 2: fn = (const void *)k_tb16_walk<4>; break;
-    case 3: fn = (const void *)k_tb16_walk<8>; break;
-    case 4: fn = (const void *)k_tb16_walk<16>; break;
-    case 5: fn = (const void *)k_tb16_walk<32>; break;
-    default: return SW_ERR_INTERNAL;
-    }
-    int bps = 0;
-    if (cuda_failed(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 256, 0))) return SW_ERR_CUDA;
-    *blocks = std::max(bps, 1) * sm_count;
-    return SW_OK;
 }
 
 // Blocks of a full-occupancy launch of traceback variant v.
 int traceback_variant_blocks(int v, int sm_count, int *blocks)
 {
-    const void *fn = nullptr;
-    switch (v) {
-    case 0: fn = (const void *)k_traceback16<1, true>; break;
-    case 1: fn = (const void *)k_traceback16<2, true>; break;
-    case 2: fn = (const void *)k_traceback16<4, true>; break;
-    case 3: fn = (const void *)k_traceback16<8, true>; break;
-    case 4: fn = (const void *)k_traceback16<16, true>; break;
-    case 5: fn = (const void *)k_traceback16<32, true>; break;
-    case TB_VAR_TILED: fn = (const void *)k_traceback<true>; break;
-    case TB_VAR_GROUPED: fn = (const void *)k_traceback<false>; break;
-    default: return SW_ERR_INTERNAL;
-    }
+    const void *fn = tb_kernel(v, true);
+    if (!fn) return SW_ERR_INTERNAL;
     int bps = 0;
     if (cuda_failed(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 128, 0))) return SW_ERR_CUDA;
     *blocks = std::max(bps, 1) * sm_count;

@@ -31,7 +31,6 @@ void note_cuda_error(cudaError_t e) { g_cuda_error = (int)e; }
 namespace {
 
 constexpr int kThreads = 128;
-constexpr int kSmallSlabWords = 4096;  // per-group slab of a traceback's main part
 constexpr int kMaxDevices = 64;
 constexpr int kAuxStreams = 4;
 constexpr int kHostChunks = 2;                 // sw_batch_align_host pipelines a batch in this many chunks
@@ -41,7 +40,7 @@ constexpr int64_t kHostChunkMin = 65536;       // ... of at least this many pair
 // and the per-warp slots of the traceback.  A warp's slot is sized on the
 // device for its launch's largest part; launches use as many warps as fit.
 constexpr int64_t kScoreBndMin = (int64_t)32 << 20, kScoreBndMax = (int64_t)1 << 30, kScoreBndPerPair = 1024;
-constexpr int64_t kTbMin = (int64_t)64 << 20, kTbPerPair = (int64_t)32 << 10;
+constexpr int64_t kTbMin = (int64_t)256 << 20, kTbPerPair = (int64_t)96 << 10;
 constexpr int64_t kTbCapMax = (int64_t)16 << 30, kTbCapMin = (int64_t)1 << 30;
 constexpr double kTbFreeShare = 0.3;
 
@@ -56,7 +55,6 @@ struct Buffer {
 struct ExecCtx {
     int score_blocks[N_SCORE_VARIANTS] = {};
     int tb_blocks[N_TB_VARIANTS] = {};
-    int walk_blocks[N_TB16_VARIANTS] = {};
     cudaStream_t aux[kAuxStreams] = {};
     cudaEvent_t fork_ev = nullptr;
     cudaEvent_t join_ev[kAuxStreams] = {};
@@ -71,8 +69,6 @@ int exec_ctx_init(ExecCtx &x, int sm_count)
         if ((rc = score_variant_blocks(v, sm_count, &x.score_blocks[v]))) return rc;
     for (int v = 0; v < N_TB_VARIANTS; ++v)
         if ((rc = traceback_variant_blocks(v, sm_count, &x.tb_blocks[v]))) return rc;
-    for (int v = 0; v < N_TB16_VARIANTS; ++v)
-        if ((rc = tb_walk_variant_blocks(v, sm_count, &x.walk_blocks[v]))) return rc;
     for (int k = 0; k < kAuxStreams; ++k) {
         if (cuda_failed(cudaStreamCreateWithFlags(&x.aux[k], cudaStreamNonBlocking))) return SW_ERR_CUDA;
         if (cuda_failed(cudaEventCreateWithFlags(&x.join_ev[k], cudaEventDisableTiming))) return SW_ERR_CUDA;
@@ -271,6 +267,7 @@ bool scoring_ok(const sw_scoring_t *s)
 // traceback slots).
 struct Scratch {
     int32_t *keys, *order, *hist, *bstart, *cursor, *counters, *tb_keys, *tb_order, *expect;
+    uint2 *ck_pos;
     ClassInfo *info;
     TbClassInfo *tbinfo;
     DevScorePlan *splan;
@@ -301,6 +298,7 @@ size_t fixed_layout(int64_t n_pairs, uint8_t *base, Scratch &S)
     S.counters = (int32_t *)take(sizeof(int32_t) * N_COUNTERS);
     S.tb_keys = (int32_t *)take(sizeof(int32_t) * n_pairs);
     S.tb_order = (int32_t *)take(sizeof(int32_t) * n_pairs);
+    S.ck_pos = (uint2 *)take(sizeof(uint2) * n_pairs);
     S.tbinfo = (TbClassInfo *)take(sizeof(TbClassInfo));
     S.expect = (int32_t *)take(sizeof(int32_t) * 3 * N_CLASS);
     S.splan = (DevScorePlan *)take(sizeof(DevScorePlan));
@@ -322,7 +320,7 @@ PlanParams plan_params(const ExecCtx &x, const Scoring &sc, bool allow16, int64_
     for (int v = 0; v < N_TB_VARIANTS; ++v) pp.tb_warps[v] = x.tb_blocks[v] * (kThreads / 32);
     pp.score_bnd_bytes = score_bnd_bytes;
     pp.tb_bytes = tb_bytes;
-    pp.small_slab_words = kSmallSlabWords;
+    pp.ck_bytes = allow16 ? tb_bytes / 4 * 3 : 0;
     pp.allow16 = allow16 ? 1 : 0;
     return pp;
 }
@@ -372,7 +370,9 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
             L.tb_keys = S.tb_keys;
             L.tb_hist = S.hist;
             L.tb_info = S.tbinfo;
-            L.small_slab_words = kSmallSlabWords;
+            L.ck_pool = (uint4 *)S.tb;
+            L.ck_cursor = (uint32_t *)(S.counters + CTR_CK);
+            L.ck_pos = S.ck_pos;
         }
         L.dp = S.splan;
         if ((rc = launch_score_variant(v, L, x.score_blocks[v], x.aux[v % kAuxStreams]))) return rc;
@@ -384,7 +384,8 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
                                       st)))
             return rc;
         if ((rc = launch_plan_tb(S.info, S.tbinfo, S.splan, pp, S.tplan, &S.info->status, st))) return rc;
-        const TbParams P{ps, sc, out_score, out_end, cig->ops, cig->offsets, cig->n_ops, 1, kSmallSlabWords};
+        const TbParams P{ps, sc, out_score, out_end, cig->ops, cig->offsets, cig->n_ops, (const uint4 *)S.tb,
+                         S.ck_pos};
         const bool fma = sc.mi >= sc.go;
         // one after another: each launch has the whole slot budget
         for (int v = 0; v < N_TB_VARIANTS; ++v) {
@@ -396,7 +397,6 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
             B.status = &S.info->status;
             B.dp = S.tplan;
             if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], st))) return rc;
-            if (v < N_TB16_VARIANTS && (rc = launch_tb_walk_variant(v, B, x.walk_blocks[v], st))) return rc;
         }
     }
     if (timing && cuda_failed(cudaEventRecord(x.phase[3], st))) return SW_ERR_CUDA;
@@ -518,48 +518,36 @@ void plan_budgets(const ClassInfo &ci, const PlanParams &pp, bool cigar, int64_t
     bnd_bytes = std::max<int64_t>(nb * (int64_t)align_up(per, 256), 256);
     tb_bytes = 0;
     if (!cigar) return;
-    // per traceback launch: its widest boundary row, tile and slot over the
-    // classes it may serve, and the pool all of its tasks would fill
-    int64_t bnd_v[N_TB_VARIANTS] = {}, slot_v[N_TB_VARIANTS] = {}, pool_v[N_TB_VARIANTS] = {};
+    // the row checkpoints of every class, and per traceback launch the widest
+    // slot over the classes it may serve
+    int64_t slot_v[N_TB_VARIANTS] = {}, ck = 0;
     for (int c = 0; c < N_CLASS; ++c) {
         if (!ci.count[c]) continue;
         const int mode = c / N_MCLASS;
         const int32_t mm = ci.max_m[c], mn = std::max(ci.max_n[c], 1);
         const int64_t chunks = (mm + TB_ROWS - 1) / TB_ROWS;
-        // the widest window, and the widest below each kernel switch
-        const int64_t cand[3] = {mn, std::min<int64_t>(mn, kTiledLaneWords16 / (2 * chunks) / 4 * 4),
-                                 std::min<int64_t>(mn, kTiledLaneWords / chunks)};
+        if (pp.allow16 && mode != MODE_I32)
+            ck += 16 * std::max(ck_class_units(ci.count[c], (int64_t)ci.sum_n[c], mm, mn, 1, 40),
+                                ck_class_units(ci.count[c], (int64_t)ci.sum_n[c], mm, mn, 32, 40));
+        // the widest window, the widest of the narrow part, and the widest
+        // one-lane tile of the int32 kernels
+        const int64_t cand[3] = {mn, std::min<int64_t>(mn, kTbWide), std::min<int64_t>(mn, kTiledLaneWords / chunks)};
         for (int64_t w : cand) {
             if (w < 1) continue;
-            for (int part = 0; part < 2; ++part) {
+            for (int lanes = w > kTbWide ? 8 : 1; lanes <= 8; lanes *= 2) {
                 TbPartPlan t{};
-                const int64_t slot = tb_part_shape(mode, pp.allow16 != 0, mm, chunks * w, (int32_t)w, part,
-                                                   pp.small_slab_words, t);
-                const int v = t.variant;
-                if (v < N_TB16_VARIANTS) {
-                    const int64_t tile = (32 * t.slab_words + 63) & ~(int64_t)63;
-                    const int64_t tasks = (ci.count[c] + 2 * (32 >> v) - 1) / (2 * (32 >> v));
-                    bnd_v[v] = std::max(bnd_v[v], (t.bnd_ints + 63) & ~(int64_t)63);
-                    slot_v[v] = std::max(slot_v[v], tile);
-                    pool_v[v] = std::max(pool_v[v], tasks * tile);  // one candidate per class counts
-                } else {
-                    slot_v[v] = std::max(slot_v[v], (slot + 63) & ~(int64_t)63);
-                }
+                const int64_t slot = tb_part_shape(mode, pp.allow16 != 0, 64, mm, chunks * w, (int32_t)w,
+                                                   w > kTbWide ? 0 : 1, pp.sc, lanes, t);
+                slot_v[t.variant] = std::max(slot_v[t.variant], (slot + 63) & ~(int64_t)63);
             }
         }
     }
     const int64_t cap = kTbCapMax / 4;  // words
-    for (int v = 0; v < N_TB_VARIANTS; ++v) {
-        if (!slot_v[v]) continue;
-        const int64_t w = pp.tb_warps[v];
-        int64_t words;
-        if (v < N_TB16_VARIANTS)
-            words = std::min(w * bnd_v[v], cap) + std::max({std::min(pool_v[v] + slot_v[v], cap),
-                                                            std::min(w * slot_v[v], cap), slot_v[v]});
-        else
-            words = std::max(std::min(w * slot_v[v], cap), 4 * slot_v[v]);
-        tb_bytes = std::max(tb_bytes, 4 * words);
-    }
+    for (int v = 0; v < N_TB_VARIANTS; ++v)
+        if (slot_v[v])
+            tb_bytes = std::max(tb_bytes, 4 * std::max(std::min(pp.tb_warps[v] * slot_v[v], cap), 4 * slot_v[v]));
+    // the planner lets checkpoints take three quarters of the scratch
+    tb_bytes = std::max(tb_bytes + std::min(ck, kTbCapMax), (std::min(ck, kTbCapMax) + 2) / 3 * 4);
 }
 
 int plan_build(sw_plan *pl, DeviceState *ds, cudaStream_t st)

@@ -83,6 +83,7 @@ struct ClassInfo {
     int32_t max_m[N_CLASS];
     int32_t status;
     int32_t pad[3];
+    unsigned long long sum_n[N_CLASS];  // window bases of the class
 };
 
 struct TbClassInfo;
@@ -107,7 +108,12 @@ struct ScoreLaunch {
     int32_t *tb_keys = nullptr;
     int32_t *tb_hist = nullptr;
     TbClassInfo *tb_info = nullptr;
-    int32_t small_slab_words = 0;
+    // row checkpoints for the traceback (classes with cls_ck in the plan):
+    // the pool in 16-byte units, its cursor, and per pair (first unit, units
+    // per row x 2 + half of the word the pair is in)
+    uint4 *ck_pool = nullptr;
+    uint32_t *ck_cursor = nullptr;
+    uint2 *ck_pos = nullptr;
     // device-planned launch (dp != nullptr): the launch serves every class
     // of score variant `variant` in the plan; order is then the whole
     // sorted pair order, work_counter the base of the per-class counters and
@@ -125,15 +131,15 @@ struct TbParams {
     uint32_t *cig_ops;
     const int64_t *cig_off;
     int32_t *cig_n;
-    int32_t lanes;            // T lanes per pair
-    int32_t small_slab_words; // per-group slab of the main launch
+    const uint4 *ck_pool;     // row checkpoints of the score pass
+    const uint2 *ck_pos;
 };
 
 // Per-class facts of the traceback sort, read back to size the slabs.
 struct TbClassInfo {
     int32_t max_need[N_CLASS];  // largest slab (words) a pair of the class needs
-    int32_t n_big[N_CLASS];     // pairs needing more than small_slab_words
-    int32_t max_wcap[2][N_CLASS];  // widest chunk window: [0] big-slab launch, [1] main launch
+    int32_t n_big[N_CLASS];     // pairs with chunk windows wider than kTbWide
+    int32_t max_wcap[2][N_CLASS];  // widest chunk window: [0] the wide part, [1] the rest
 };
 
 // A persistent traceback launch: every part of traceback variant `variant`
@@ -174,11 +180,21 @@ __host__ __device__ inline int score_rows_at(int i)
 // classes (or traceback parts) its variant was given and exits at once when
 // it has none.
 constexpr int N_SCORE_VARIANTS = N_SCORE_ROWS * N_MODES;  // variant = rows index * N_MODES + mode
-constexpr int N_TB16_VARIANTS = 6;                        // 16-bit traceback, T = 1, 2, 4, 8, 16, 32
-constexpr int TB_VAR_TILED = 6;                           // int32 traceback, one lane per pair, warp tiles
-constexpr int TB_VAR_GROUPED = 7;                         // int32 traceback, T lanes per pair
-constexpr int N_TB_VARIANTS = 8;
-constexpr int N_TB_PARTS = 2 * N_CLASS;                   // per class: pairs with big slabs, then the rest
+constexpr int N_TB16_VARIANTS = 5;                        // 16-bit traceback: wide windows, T = 8; the rest, T = 8, 4, 2, 1
+constexpr int TB_VAR_TILED = 5;                           // int32 traceback, one lane per pair, warp tiles
+constexpr int TB_VAR_GROUPED = 6;                         // int32 traceback, T lanes per pair
+constexpr int N_TB_VARIANTS = 7;
+__host__ __device__ inline int tb16_variant_lanes(int v) { return v == 0 ? 8 : 16 >> v; }
+constexpr int N_TB_PARTS = 2 * N_CLASS;                   // per class: the wide part, then the rest
+// Chunk windows wider than this form a part (and launches) of their own: a
+// warp's scratch slot is sized for the widest window of its launch, and a
+// few spliced pairs with windows of thousands of columns would otherwise
+// leave room for a fraction of the warps.  They take 8 lanes per two pairs:
+// over windows this wide the wavefront's extra steps cost little, a warp
+// waits for the widest of 8 pairs rather than of 64, and a task (many blocks
+// one after another) ends 7 times sooner -- the wide pairs of the 2M uneven
+// batch took 33 ms with one or two lanes, most of it in the last few tasks.
+constexpr int kTbWide = 256;
 constexpr int kMaxPlanOverrides = 16;
 constexpr int kPlanThreads = 384;                         // >= N_CLASS
 
@@ -194,8 +210,8 @@ struct PlanParams {
     int32_t score_warps[N_SCORE_VARIANTS];  // warps each score launch runs
     int32_t tb_warps[N_TB_VARIANTS];        // warps each traceback launch runs
     int64_t score_bnd_bytes;                // chunk-boundary scratch of the score launches
-    int64_t tb_bytes;                       // per-warp traceback scratch, shared by the (sequential) launches
-    int32_t small_slab_words;
+    int64_t tb_bytes;                       // traceback scratch: row checkpoints, then the warps' slots
+    int64_t ck_bytes;                       // most of it that row checkpoints may take (0: none)
     int32_t allow16;                        // 16-bit traceback allowed (SW_TB_AUTO)
 };
 
@@ -208,6 +224,8 @@ struct DevScorePlan {
     int32_t cls_count[N_CLASS];
     int32_t cls_lanes[N_CLASS];
     int32_t cls_bnd_bytes[N_CLASS];           // per group; 0 when a read fits one row chunk
+    int32_t cls_ck[N_CLASS];                  // rows between checkpoints (0: none kept)
+    int64_t ck_units;                         // 16-byte units of the pool the checkpoints may take
     int16_t var_cls[N_SCORE_VARIANTS][N_CLASS];  // longest reads first
 };
 
@@ -216,26 +234,49 @@ struct TbPartPlan {
     int32_t lanes, wcap;
     int64_t slab_words, bnd_ints;  // per lane (16-bit), per warp tile (tiled) or per group (grouped)
     int32_t variant;
-    int32_t pool_tasks;            // 16-bit: tasks whose tiles go to the pool (walked by k_tb16_walk)
-    int64_t pool_offset;           // 16-bit: words from the scratch base to the part's first pooled tile
+    int32_t block_rows;            // 16-bit: rows between the class's checkpoints (0: the whole read is one block)
 };
 
-// Traceback scratch of one launch (words from the scratch base; the launches
-// run one after another and each has the whole budget).  16-bit kernel: the
-// boundary rows of the warps that take part, then full per-warp slots for
-// tasks swept and walked by the warp itself, then the pool of tiles that the
-// separate walk kernel reads.  int32 kernels: per-warp slots only.
+// Traceback scratch of one launch: per-warp slots from var_slot_offset on
+// (words; the launches run one after another and each has everything the
+// row checkpoints leave).
 struct DevTbPlan {
     int32_t var_n[N_TB_VARIANTS];
-    int32_t var_warps[N_TB_VARIANTS];     // warps with a full slot (int32 kernels: the others exit)
+    int32_t var_warps[N_TB_VARIANTS];     // warps with a slot (the others exit)
     int64_t var_slot_words[N_TB_VARIANTS];
     int64_t var_slot_offset[N_TB_VARIANTS];
-    int64_t var_bnd_words[N_TB_VARIANTS];  // 16-bit: boundary row words per warp
-    int32_t var_run_warps[N_TB_VARIANTS];  // 16-bit: warps that take part (each with a boundary row)
     int64_t split[2];                     // pairs through the 16-bit and the int32 kernels
     int16_t var_part[N_TB_VARIANTS][N_TB_PARTS];
     TbPartPlan part[N_TB_PARTS];
 };
+
+// Rows between the checkpoints of a score plan with R rows per lane: a
+// multiple of R (checkpoints are bottom rows of lanes) of 40 to 64 rows,
+// doubled as often as the pool's size asks for.  Narrower blocks would have
+// narrower bands (a block's band allows for its own loss) but store more.
+__host__ __device__ inline int ck_block_rows(int R)
+{
+    return R >= 50 ? R : R > 16 ? 2 * R : 64;
+}
+
+// 16-byte units that the checkpoints of a class take at most: a task of
+// `per_warp` pairs stores, per checkpointed row and group of two pairs, its
+// widest window's columns two to a unit, and one more for each lane of a
+// group but the last.  Tasks are consecutive in the order
+// sorted by falling window length in buckets of 32 bases, so a task's widest
+// window is at most its last pair's bucket plus the step to the task before,
+// and the steps add up to the longest window once; the last bucket
+// (everything past its start) is unsorted.
+__host__ __device__ inline int64_t ck_class_units(int64_t cnt, int64_t sum_n, int32_t mm, int32_t mn,
+                                                  int32_t lanes, int32_t block_rows)
+{
+    const int64_t rows = (mm - 1) / block_rows;
+    const int32_t per_warp = 2 * (32 / lanes);
+    const int64_t slots = cnt + per_warp;
+    const int64_t cols = mn > 32 * (N_NBUCKET - 1) ? slots * mn
+                                                   : sum_n + 32 * slots + (int64_t)per_warp * (mn + 32);
+    return rows * (cols / 4 + slots / 2 * lanes + lanes);
+}
 
 // Score-pass arithmetic of a pair (or class) whose scores are at most hmax
 // (match x min(m, n)) under a sw_set_score_mode setting: 16-bit keys up to
@@ -297,63 +338,60 @@ __host__ __device__ inline void score_plan_of(int mode, int32_t m_max, int64_t h
     }
 }
 
-// Traceback launch shape of one part of a class (part 0: pairs whose
-// one-lane slab exceeds small_slab_words, part 1: the rest).  m_max: the
-// class's longest read; max_need: the largest one-lane slab of the class;
-// wcap_in: the part's widest chunk window.  The 16-bit kernel serves every
-// class with a 16-bit score mode unless allow16 is off.  T lanes share a
-// pair: one where a lane's tile (every chunk at the widest window) stays
-// small, else the smallest power of two with the longest read in at most 8
-// (16-bit) or 4 (int32) chunks of 8T rows -- a chunk sweeps its rows' band
-// box, 8T - 1 columns wider than the band, so smaller T wastes fewer cells
-// and larger T keeps fewer pairs per warp waiting (measured on the uneven
-// batch, 16-bit: 4 chunks 57.0 ms, 8 chunks 49.6 ms, 16 chunks 64.5 ms).
-// Also the words one warp's scratch slot needs for this part.
-constexpr int kTbChunks16 = 8, kTbChunks32 = 4;
-constexpr int64_t kTiledLaneWords = 4096, kTiledLaneWords16 = 8192;
-__host__ __device__ inline int64_t tb_part_shape(int mode, bool allow16, int32_t m_max, int64_t max_need,
-                                                 int32_t wcap_in, int part, int32_t small_slab_words, TbPartPlan &t,
-                                                 int min_lanes16 = 1)
+// Traceback launch shape of one part of a class (part 0: chunk windows wider
+// than kTbWide, part 1: the rest).  m_max: the class's longest read;
+// max_need: the largest one-lane slab of the class (int32 kernels); wcap_in:
+// the part's widest chunk window; block_rows: rows between the class's
+// checkpoints (0 or m_max and more: the whole read is one block).  The 16-bit kernel
+// serves every class with a 16-bit score mode unless allow16 is off, with
+// lanes16 lanes per two pairs.  The int32 kernel takes one lane per pair
+// where a lane's tile (every chunk at the widest window) stays small, else
+// the smallest power of two with the longest read in at most 4 chunks of 8T
+// rows.  Also the words one warp's scratch slot needs for this part.
+constexpr int kTbChunks32 = 4;
+constexpr int64_t kTiledLaneWords = 4096;
+__host__ __device__ inline int64_t tb_part_shape(int mode, bool allow16, int32_t block_rows, int32_t m_max,
+                                                 int64_t max_need, int32_t wcap_in, int part, const Scoring &sc,
+                                                 int lanes16, TbPartPlan &t)
 {
     const int64_t chunks = (m_max + TB_ROWS - 1) / TB_ROWS;
     int32_t wcap = wcap_in > 1 ? wcap_in : 1;
-    const int64_t wcap4 = (wcap + 3) / 4 * 4;
-    const bool packed16 = allow16 && mode != MODE_I32;
-    int Tl = 1;
-    while (Tl < 32 && (int64_t)Tl * 8 * (packed16 ? kTbChunks16 : kTbChunks32) < m_max) Tl *= 2;
-    const bool one_lane16 = chunks * wcap4 * 2 <= kTiledLaneWords16;
-    const bool tiled = !packed16 && chunks * wcap <= kTiledLaneWords;
-    int T = (packed16 && one_lane16) || tiled ? 1 : Tl;
-    if (packed16 && T < min_lanes16) T = min_lanes16;
-    t.lanes = T;
-    int64_t slot;
-    if (packed16) {
-        const int64_t chunks_t = (m_max + 8 * T - 1) / (8 * T);
-        wcap += 8 * (T - 1);
+    t.block_rows = 0;
+    if (allow16 && mode != MODE_I32) {
+        const int T = lanes16;
+        const int64_t rows = block_rows && block_rows < m_max ? block_rows : m_max;
+        const int64_t chunks_t = (rows + 8 * T - 1) / (8 * T);
+        // a block entered inside an insertion run does not pay for opening
+        // it, so its band may be a few columns wider than the whole pair's;
+        // windows start at multiples of four columns
+        wcap = (wcap + (sc.ge - sc.go) / (sc.ma - sc.ge) + 2 + 8 * (T - 1) + 3 + 3) / 4 * 4;
         const int64_t s4 = (wcap + T - 1 + 3) / 4;
-        t.slab_words = chunks_t * s4 * 8;                            // per lane
-        t.bnd_ints = chunks_t > 1 ? (int64_t)(32 / T) * 2 * wcap : 0;  // per warp: one row
-        int v = 0;
-        while ((1 << v) < T) ++v;
-        t.variant = v;
-        slot = 32 * t.slab_words + t.bnd_ints;
-    } else if (tiled) {
+        t.lanes = T;
+        t.wcap = wcap;
+        t.block_rows = block_rows;
+        t.slab_words = chunks_t * s4 * 8;                // per lane
+        t.bnd_ints = (int64_t)(32 / T) * 2 * (wcap + 8);  // per warp: one row
+        t.variant = part == 0 ? 0 : T == 8 ? 1 : T == 4 ? 2 : T == 2 ? 3 : 4;
+        return ((32 * t.slab_words + 63) & ~(int64_t)63) + t.bnd_ints;
+    }
+    int T = 1;
+    while (T < 32 && (int64_t)T * 8 * kTbChunks32 < m_max) T *= 2;
+    const bool tiled = chunks * wcap <= kTiledLaneWords;
+    if (tiled) T = 1;
+    t.lanes = T;
+    t.wcap = wcap;
+    if (tiled) {
         t.slab_words = chunks * wcap;                  // per lane
         t.bnd_ints = chunks > 1 ? (int64_t)4 * wcap : 0;
         t.variant = TB_VAR_TILED;
-        slot = 32 * (t.slab_words + t.bnd_ints);
-    } else {
-        const int64_t chunks_t = (m_max + 8 * T - 1) / (8 * T);
-        const int64_t wcap_t = wcap + 8 * (T - 1);
-        const int64_t need = max_need > 1 ? max_need : 1;
-        t.slab_words = T == 1 ? (part == 0 ? need : (need < small_slab_words ? need : small_slab_words))
-                              : chunks_t * wcap_t * T;  // per group
-        t.bnd_ints = chunks_t > 1 ? (int64_t)4 * wcap_t : 0;
-        t.variant = TB_VAR_GROUPED;
-        slot = (int64_t)(32 / T) * (t.slab_words + t.bnd_ints);
+        return 32 * (t.slab_words + t.bnd_ints);
     }
-    t.wcap = wcap;
-    return slot;
+    const int64_t chunks_t = (m_max + 8 * T - 1) / (8 * T);
+    const int64_t wcap_t = wcap + 8 * (T - 1);
+    t.slab_words = T == 1 ? (max_need > 1 ? max_need : 1) : chunks_t * wcap_t * T;  // per group
+    t.bnd_ints = chunks_t > 1 ? (int64_t)4 * wcap_t : 0;
+    t.variant = TB_VAR_GROUPED;
+    return (int64_t)(32 / T) * (t.slab_words + t.bnd_ints);
 }
 
 // score_setting: the sw_set_score_mode value (SW_SCORE_INT32: every pair in
@@ -376,13 +414,10 @@ int launch_score_variant(int v, const ScoreLaunch &L, int blocks, cudaStream_t s
 int score_variant_blocks(int v, int sm_count, int *blocks);
 int launch_traceback_variant(int v, bool fma, const TracebackLaunch &L, int blocks, cudaStream_t st);
 int traceback_variant_blocks(int v, int sm_count, int *blocks);
-// The walks of a 16-bit traceback launch's pooled tasks (v < N_TB16_VARIANTS).
-int launch_tb_walk_variant(int v, const TracebackLaunch &L, int blocks, cudaStream_t st);
-int tb_walk_variant_blocks(int v, int sm_count, int *blocks);
-// Per-class work counters of one batch: score, traceback (pooled tasks),
-// traceback (tasks a warp sweeps and walks itself).
-constexpr int N_COUNTERS = 6 * N_CLASS;
-constexpr int CTR_TB = 2 * N_CLASS, CTR_TB_OWN = 4 * N_CLASS;
+// Work counters of one batch: score (per class), traceback (per part), and
+// the checkpoint pool's cursor.
+constexpr int CTR_TB = N_CLASS, CTR_CK = CTR_TB + N_TB_PARTS;
+constexpr int N_COUNTERS = CTR_CK + 1;
 int launch_scan_scatter(const int32_t *keys, int64_t n_pairs, const int32_t *class_count, int32_t *hist,
                         int32_t *bucket_start, int32_t *cursor, int32_t *order, cudaStream_t st);
 

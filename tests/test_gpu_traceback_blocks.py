@@ -1,0 +1,89 @@
+"""The 16-bit traceback recomputes a read in blocks of 40 to 64 rows from the
+score pass's checkpoints: reads whose length, end row, gaps or start fall on
+and around the block edges, windows on both sides of the wide-window split,
+every number of lanes per two pairs, and several scorings, bit-exact against
+the oracle."""
+import numpy as np
+import pytest
+
+import synth
+from gpu_helpers import assert_parity, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+DEFAULT = (5, -4, -10, -1)
+
+
+def _batch(pairs):
+    reads, wins = zip(*pairs)
+    off = lambda a: np.concatenate([[0], np.cumsum([len(x) for x in a])]).astype(np.int64)  # noqa: E731
+    n = len(reads)
+    return synth.Workload("blocks", np.concatenate(reads), off(reads), np.concatenate(wins), off(wins),
+                          np.arange(n, dtype=np.int64), np.arange(n + 1, dtype=np.int64), np.zeros(n, np.uint8),
+                          np.zeros(n, np.int32))
+
+
+def _edge_pairs(rng, lengths, alphabet=4):
+    """Reads with one gap run that begins, ends or lies across a block edge,
+    flanked by random bases; some with their first rows unrelated."""
+    out = []
+    base = lambda n: rng.integers(0, alphabet, n).astype(np.uint8)  # noqa: E731
+    for m in lengths:
+        for at in sorted({1, m // 2} | {e + d for e in (40, 50, 64, 100, 128) for d in (-1, 0, 1) if 0 < e + d < m - 1}):
+            read = base(m)
+            for gap in (0, 1, 7, -1, -6, 40, 300):
+                if gap >= 0:   # window bases the read lacks
+                    win = np.concatenate([read[:at], base(gap), read[at:]])
+                else:          # read bases the window lacks
+                    win = np.concatenate([read[:at], read[min(m, at - gap):]])
+                if rng.random() < 0.3:
+                    win = np.concatenate([base(at), win[at:]])   # the alignment starts inside the read
+                out.append((read, np.concatenate([base(rng.integers(0, 30)), win, base(rng.integers(0, 30))])))
+    return out
+
+
+@pytest.mark.parametrize("scoring", [DEFAULT, (2, -3, -5, -2), (2, -9, -4, -1), (5, -4, -10, 0), (1, -1, -2, -2)])
+def test_gaps_around_block_edges(scoring):
+    rng = np.random.default_rng(17)
+    wl = _batch(_edge_pairs(rng, (39, 40, 41, 49, 50, 51, 63, 64, 65, 81, 101, 129, 151)) +
+                _edge_pairs(rng, (66, 102), alphabet=2))
+    assert_parity(wl, run_gpu(wl, scoring), scoring)
+
+
+def test_long_reads_and_wide_windows():
+    """Several row chunks per pair, and blocks whose band is as wide as an
+    intron (competing alignments on both sides of it)."""
+    rng = np.random.default_rng(18)
+    pairs = []
+    for m in (700, 1601, 3300):
+        for cut, intron in ((m // 2, 250), (m // 3, 900), (50, 2000)):
+            r = rng.integers(0, 4, m).astype(np.uint8)
+            w = np.concatenate([r[:cut], rng.integers(0, 4, intron).astype(np.uint8), r[cut:]])
+            flip = rng.random(len(w)) < 0.02
+            w = np.where(flip, (w + rng.integers(1, 4, len(w))) & 3, w).astype(np.uint8)
+            pairs += [(r, w), (r, np.concatenate([w, w[:200]]))]
+    wl = _batch(pairs)
+    assert_parity(wl, run_gpu(wl, DEFAULT), DEFAULT)
+
+
+@pytest.mark.parametrize("n_pairs", [500, 12_000, 25_000, 45_000])
+def test_lanes_per_pair(n_pairs):
+    """8, 4, 2 and 1 lanes per two pairs (chosen by the batch's size)."""
+    wl = synth.random_pairs(n_pairs, (30, 130), (20, 190), seed=n_pairs, alphabet=3)
+    got = run_gpu(wl, DEFAULT)
+    sample = np.random.default_rng(3).choice(n_pairs, 500, replace=False)
+    assert_parity(wl, got, DEFAULT, pairs=np.sort(sample))
+
+
+def test_block_doubling_when_the_pool_is_small():
+    """More checkpoint rows than the scratch of a batch this size holds: the
+    blocks double until they fit."""
+    rng = np.random.default_rng(19)
+    pairs = []
+    for _ in range(40):
+        r = rng.integers(0, 4, 6000).astype(np.uint8)
+        w = np.concatenate([rng.integers(0, 4, 14_000).astype(np.uint8), r])
+        flip = rng.random(len(w)) < 0.02
+        pairs.append((r, np.where(flip, (w + rng.integers(1, 4, len(w))) & 3, w).astype(np.uint8)))
+    wl = _batch(pairs)
+    assert_parity(wl, run_gpu(wl, DEFAULT), DEFAULT, pairs=np.arange(0, 40, 8))
