@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_score(const ClassInfo *__
             int ri = 0;
             const int64_t hmax = (int64_t)pp.sc.ma * min(mm, mn);
             score_plan_of(mode, mm, hmax, pp.ov, pp.n_overrides, lanes, ri);
+            const int vmode = score_vmode(mode, hmax, pp.sc);
             // a class with fewer tasks than half its launch's warps (a small
             // batch) finishes when one task does: fewer rows per lane, on
             // more lanes, shorten the task while it still fits one row chunk
@@ -47,7 +48,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_score(const ClassInfo *__
             while (!chosen && ri > 0) {
                 const int64_t per_warp = (int64_t)(32 / lanes) * (mode != MODE_I32 ? 2 : 1);
                 const int64_t tasks = (cnt + per_warp - 1) / per_warp;
-                if (2 * tasks >= pp.score_warps[ri * N_MODES + mode]) break;
+                if (2 * tasks >= pp.score_warps[ri * N_VMODES + vmode]) break;
                 const int t2 = (mm + score_rows_at(ri - 1) - 1) / score_rows_at(ri - 1);
                 if (t2 > 32) break;
                 --ri;
@@ -57,7 +58,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_score(const ClassInfo *__
             const int chunks = (mm + lanes * rows - 1) / (lanes * rows);
             // per group: two buffers x longest window x (H, F) x 4 bytes
             bnd = chunks > 1 ? 16 * mn : 0;
-            var = ri * N_MODES + mode;
+            var = ri * N_VMODES + vmode;
             if (pp.ck_bytes > 0 && mode != MODE_I32) ck = ck_block_rows(rows);
         }
         s_var[c] = var;

@@ -28,20 +28,20 @@ int launch_score(int rows, int mode, const ScoreLaunch &L, int blocks, int threa
     return launch_status();
 }
 
-// A device-planned launch of variant v = rows index * N_MODES + mode; the
+// A device-planned launch of variant v = rows index * N_VMODES + mode; the
 // FMA-pipe diagonal add is chosen from the scoring as for launch_score.
 int launch_score_variant(int v, const ScoreLaunch &L, int blocks, cudaStream_t st)
 {
     if (v < 0 || v >= N_SCORE_VARIANTS || !L.dp) return SW_ERR_INTERNAL;
     ScoreLaunch V = L;
     V.variant = v;
-    return launch_score(score_rows_at(v / N_MODES), v % N_MODES, V, blocks, 128, st);
+    return launch_score(score_rows_at(v / N_VMODES), v % N_VMODES, V, blocks, 128, st);
 }
 
 int score_variant_blocks(int v, int sm_count, int *blocks)
 {
     int regs = 0, bps = 0;
-    const int rc = score_kernel_regs(score_rows_at(v / N_MODES), v % N_MODES, &regs, &bps, 128);
+    const int rc = score_kernel_regs(score_rows_at(v / N_VMODES), v % N_VMODES, &regs, &bps, 128);
     if (rc) return rc;
     if (bps < 1) return SW_ERR_INTERNAL;
     *blocks = bps * sm_count;

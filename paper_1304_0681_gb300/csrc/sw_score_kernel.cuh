@@ -64,7 +64,9 @@
 // first row of that snapshot holding the best value.  This
 // moves the row tracking off the ALU pipe (the kernel's limit) onto the
 // shared-memory stores, so the wide mode costs the same ALU operations per
-// cell as the 16-bit-key mode.  The int32 mode covers the rest.
+// cell as the 16-bit-key mode.  Classes whose values stay within 2047
+// (MODE_I16S: reads of up to 407 bases at match 5) are a variant of it.  The
+// int32 mode covers the rest.
 //
 // Checkpoints.  With a CIGAR to follow, the lanes whose bottom row ends a
 // block of 40 to 64 read rows also store that row (H and F - o of every
@@ -153,6 +155,17 @@ struct Arith<MODE_I16> {
 };
 template <>
 struct Arith<MODE_I16W> : Arith<MODE_I16> {};
+template <>
+struct Arith<MODE_I16S> : Arith<MODE_I16> {};
+
+// max(a + b, 0) per half on the FMA pipe, for halves of a up to 2047 (see
+// half_exact): b as a sign and magnitude, -x as 0x8000 | x.
+__device__ __forceinline__ uint32_t half_add_relu(uint32_t a, uint32_t b)
+{
+    uint32_t d;
+    asm("fma.rn.relu.f16x2 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(0x3C003C00u), "r"(b));
+    return d;
+}
 
 // a * one + c on the FMA pipe; `one` is a kernel argument equal to 1, so the
 // multiply-add cannot be folded into an ALU add.  With both halves of a and c
@@ -200,7 +213,7 @@ __device__ __forceinline__ int snapshot_row(const uint4 *snap, unsigned stride, 
 // Dynamic shared memory of a launch: the MODE_I16W snapshot slots.
 __host__ __device__ constexpr int score_snapshot_bytes(int rows, int mode, int threads)
 {
-    return mode == MODE_I16W ? 2 * ((rows + 3) / 4) * 16 * threads : 0;
+    return mode == MODE_I16W || mode == MODE_I16S ? 2 * ((rows + 3) / 4) * 16 * threads : 0;
 }
 
 // CK: checkpoints are kept for a traceback (launches without a CIGAR to
@@ -211,6 +224,12 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
     typedef Arith<MODE> A;
     typedef typename A::V V;
     constexpr bool PAIR2 = MODE != MODE_I32;
+    // The add of gap_open with the floor at 0 runs on the FMA pipe
+    // (half_add_relu) instead of the ALU pipe, which bounds the kernel: 30,000
+    // reads of 150 bases x 1-64 windows of 250 score in 7.8 ms instead of 8.6,
+    // 1M pairs of 100 x 200 in 4.05 instead of 4.26.  (16-bit keys hold scores
+    // up to 510, and -gap_open is at most 126.)
+    constexpr bool HALF_ADD = MODE == MODE_I16 || MODE == MODE_I16S;
     constexpr int NW = (R + 7) / 8;
     // row tag in the low bits of a key: TAGM - r, so equal H prefers the
     // smaller row; 5 bits cover 32 rows, 6 bits 64
@@ -239,6 +258,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
     const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t one = (uint32_t)L.one;
     const V GO = A::splat(go), GE = A::splat(ge);
+    const uint32_t GOH = 0x80008000u | ((uint32_t)(-go) * 0x10001u);
     // input already found invalid (or a plan whose shape changed): the
     // scratch may be too small for it, so do nothing
     if (*(volatile const int32_t *)L.status & ST_BAD_INPUT) return;
@@ -264,7 +284,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
     // the wide 50-row kernels have no register to spare for a checkpoint
     // lane's place in the pool (uneven score pass 41.2 ms with 8 bytes
     // spilled, 40.8 with a shared-memory load per step)
-    constexpr bool CK_SHARED = MODE == MODE_I16W && R >= 50;
+    constexpr bool CK_SHARED = (MODE == MODE_I16W || MODE == MODE_I16S) && R >= 50;
     __shared__ uint32_t s_ck_at[CK && CK_SHARED ? 128 : 1];
     volatile ClassCtx *const cc = &s_cc[threadIdx.x >> 5];
     const bool planned = L.dp != nullptr;
@@ -446,6 +466,10 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
                     if (upB) { slotB = sl; jB = jj; }
                 }
             };
+            auto add_go = [&](V u) -> V {
+                if constexpr (HALF_ADD) return (V)half_add_relu((uint32_t)u, GOH);
+                else return A::addmax_relu(u, GO, 0);
+            };
             for (int u = 0; u < iters; ++u) {
                 const int j0 = 2 * (u - k);
                 V up_h0 = __shfl_up_sync(FULL, out_h, 1);
@@ -499,7 +523,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
                             d0n = FMA_ADD ? (V)mad_add((uint32_t)h1[r], one, (uint32_t)sn) : A::add(h1[r], sn);
                         }
                         f0 = A::addmax(f0, GE, hu0);
-                        const V hn = A::addmax_relu(A::max3(d, e[r], f0), GO, 0);
+                        const V hn = add_go(A::max3(d, e[r], f0));
                         h[r] = hn;
                         hu0 = hn;
                         const uint32_t k0 = MODE == MODE_I16 ? mad_add((uint32_t)hn, 1u << TAGB, (TAGM - (uint32_t)r) * 0x10001u)
@@ -516,7 +540,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
                             d1n = FMA_ADD ? (V)mad_add((uint32_t)h[q], one, (uint32_t)sn) : A::add(h[q], sn);
                         }
                         f1 = A::addmax(f1, GE, hu1);
-                        const V hn = A::addmax_relu(A::max3(d, e[q], f1), GO, 0);
+                        const V hn = add_go(A::max3(d, e[q], f1));
                         h1[q] = hn;
                         hu1 = hn;
                         const uint32_t k1 = MODE == MODE_I16 ? mad_add((uint32_t)hn, 1u << TAGB, (TAGM - (uint32_t)q) * 0x10001u)
@@ -665,6 +689,8 @@ const void *score_kernel_of(int mode, bool fma)
     case MODE_I16: return fma ? (const void *)k_score<R, MODE_I16, true, CK> : (const void *)k_score<R, MODE_I16, false, CK>;
     case MODE_I16W:
         return fma ? (const void *)k_score<R, MODE_I16W, true, CK> : (const void *)k_score<R, MODE_I16W, false, CK>;
+    case MODE_I16S:
+        return fma ? (const void *)k_score<R, MODE_I16S, true, CK> : (const void *)k_score<R, MODE_I16S, false, CK>;
     default: return nullptr;
     }
 }

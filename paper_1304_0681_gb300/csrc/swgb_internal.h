@@ -60,6 +60,10 @@ enum ScoreMode : int32_t {
     MODE_I16 = 1,   // two pairs per lane group in int16 halves, 16-bit keys
     MODE_I16W = 2,  // two pairs per lane group in int16 halves, 32-bit keys
     N_MODES = 3,
+    // a MODE_I16W class whose values all fit half_exact(): a score variant of
+    // its own, no class mode
+    MODE_I16S = 3,
+    N_VMODES = 4,
 };
 
 // Read-length classes: 16-base steps up to 1024, then 128-base steps.
@@ -179,7 +183,7 @@ __host__ __device__ inline int score_rows_at(int i)
 // is launched once, persistent at full occupancy; a launch serves the
 // classes (or traceback parts) its variant was given and exits at once when
 // it has none.
-constexpr int N_SCORE_VARIANTS = N_SCORE_ROWS * N_MODES;  // variant = rows index * N_MODES + mode
+constexpr int N_SCORE_VARIANTS = N_SCORE_ROWS * N_VMODES;  // variant = rows index * N_VMODES + mode
 constexpr int N_TB16_VARIANTS = 5;                        // 16-bit traceback: wide windows, T = 8; the rest, T = 8, 4, 2, 1
 constexpr int TB_VAR_TILED = 5;                           // int32 traceback, one lane per pair, warp tiles
 constexpr int TB_VAR_GROUPED = 6;                         // int32 traceback, T lanes per pair
@@ -291,6 +295,18 @@ __host__ __device__ inline int score_mode_for(int64_t hmax, int setting)
     if (hmax <= 510 && setting != SW_SCORE_WIDE16) return MODE_I16;
     if (hmax <= 32000) return MODE_I16W;
     return MODE_I32;
+}
+
+// Whether a 16-bit mode may take its add of gap_open with the floor at 0 as an
+// fp16 multiply-add: halves 0 .. 2047 are fp16 numbers 2^-24 apart
+// (subnormals and the first binade), so fp16 adds them as integers; the
+// largest value is the score bound hmax less gap_open.
+__host__ __device__ inline bool half_exact(int64_t hmax, const Scoring &sc) { return hmax - sc.go <= 2047; }
+
+// The kernel mode of a class of `mode` with score bound hmax.
+__host__ __device__ inline int score_vmode(int mode, int64_t hmax, const Scoring &sc)
+{
+    return mode == MODE_I16W && half_exact(hmax, sc) ? (int)MODE_I16S : mode;
 }
 
 // Score-pass plan of a length class: lanes per group and rows per lane
@@ -408,7 +424,7 @@ int launch_plan_score(const ClassInfo *info, const PlanParams &pp, DevScorePlan 
                       cudaStream_t st);
 int launch_plan_tb(const ClassInfo *info, const TbClassInfo *ti, const DevScorePlan *sp, const PlanParams &pp,
                    DevTbPlan *out, int32_t *status, cudaStream_t st);
-// One persistent launch of score variant v (rows index * N_MODES + mode) at
+// One persistent launch of score variant v (rows index * N_VMODES + mode) at
 // full occupancy; its grid (blocks) comes from score_variant_blocks.
 int launch_score_variant(int v, const ScoreLaunch &L, int blocks, cudaStream_t st);
 int score_variant_blocks(int v, int sm_count, int *blocks);
