@@ -5,6 +5,7 @@
 // lays the pairs out class by class, longest windows first, so that each
 // class can run under its own lane plan and lanes that share a warp see
 // windows of similar length.
+#include "sw_classify.cuh"
 #include "sw_device.cuh"
 #include "swgb_internal.h"
 
@@ -36,37 +37,7 @@ __global__ void k_classify(PairSet ps, int64_t n_reads, int64_t n_pairs, Scoring
         int32_t key = -1, cls = 0;
         int64_t m = 0, n = 0;
         if (p < n_pairs) {
-            const int64_t rd = ps.pair_read ? ps.pair_read[p] : p;
-            bool bad = rd < 0 || rd >= n_reads;
-            if (!bad) {
-                const int64_t r0 = ps.read_off[rd], r1 = ps.read_off[rd + 1];
-                const int64_t w0 = ps.win_off[p], w1 = ps.win_off[p + 1];
-                m = r1 - r0;
-                n = w1 - w0;
-                bad = r0 < 0 || w0 < 0 || m < 1 || m > SW_MAX_READ_LEN || n < 0 || n > SW_MAX_WINDOW_LEN;
-            }
-            if (bad) {
-                atomicOr(&info->status, ST_BAD_INPUT);
-            } else if (ps.mask && !ps.mask[p]) {
-                // not selected: no alignment
-                out_score[p] = -1;
-                out_end[2 * p] = -1;
-                out_end[2 * p + 1] = -1;
-                if (cig_n) cig_n[p] = 0;
-            } else if (n == 0) {
-                // an empty window aligns nothing: score 0, no end cell, no CIGAR
-                out_score[p] = 0;
-                out_end[2 * p] = -1;
-                out_end[2 * p + 1] = -1;
-                if (cig_n) cig_n[p] = 0;
-            } else {
-                const int64_t hmax = (int64_t)sc.ma * (m < n ? m : n);
-                const int mode = score_mode_for(hmax, score_setting);
-                cls = mode * N_MCLASS + mclass_of((int32_t)m);
-                int nb = (int)((n - 1) >> 5);
-                nb = nb > N_NBUCKET - 1 ? N_NBUCKET - 1 : nb;
-                key = cls * N_NBUCKET + (N_NBUCKET - 1 - nb);
-            }
+            key = classify_pair(ps, n_reads, p, sc, score_setting, &info->status, out_score, out_end, cig_n, cls, m, n);
             keys[p] = key;
         }
         // one set of atomics per distinct key in the warp (the key fixes the class)

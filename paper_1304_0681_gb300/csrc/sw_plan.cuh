@@ -1,0 +1,283 @@
+// sw_plan.cuh -- launch planning on the device (bodies of the planner kernels).
+//
+// The paper hands whole batches to OpenMP threads and balances the thread
+// counts of its stages by hand (Section 3.4, Section 4.3).  Here a batch is
+// sorted into length classes on the GPU, and one block each plans the
+// launches from the classification's per-class facts, so that the host
+// enqueues a fixed sequence of launches and never waits for the device:
+//
+//   plan_score    per class the lanes per pair and rows per lane (the cost
+//                 model of score_plan_of), the class's place in the sorted
+//                 order, its score variant (compiled rows x arithmetic
+//                 mode), the chunk-boundary scratch of classes whose
+//                 reads need several row chunks, and which classes keep row
+//                 checkpoints for the traceback;
+//   plan_tb       per class and part (pairs with wide windows, the rest) the
+//                 traceback kernel, its lanes per pair and slab sizes
+//                 (tb_part_shape), and per traceback variant the size of a
+//                 warp's scratch slot and how many warps fit the budget.
+//
+// Each variant's list is ordered longest reads first, so the persistent
+// launches end on short work.
+//
+// A batch has few classes: the first warp lists them once, and every later
+// step runs over that list, a lane per launch variant.
+#pragma once
+#include "sw_device.cuh"
+#include "swgb_internal.h"
+
+namespace swgb {
+
+// The non-empty classes (count[c] > 0), largest index first, by the first
+// warp; returns how many.
+__device__ __forceinline__ int list_classes(const int32_t *count, int16_t *list)
+{
+    const int lane = threadIdx.x & 31;
+    int n = 0;
+    for (int c0 = N_CLASS - 1; c0 >= 0; c0 -= 32) {
+        const int c = c0 - lane;
+        const bool hit = c >= 0 && count[c] > 0;
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        if (hit) list[n + __popc(m & ((1u << lane) - 1u))] = (int16_t)c;
+        n += __popc(m);
+    }
+    __syncwarp();
+    return n;
+}
+
+// A score plan for one class: lanes per group, rows index and kernel mode.
+__device__ __forceinline__ void plan_class(const PlanParams &pp, int mode, int32_t cnt, int32_t mm, int32_t mn,
+                                           int &lanes, int &ri, int &vmode)
+{
+    const int64_t hmax = (int64_t)pp.sc.ma * min(mm, mn);
+    score_plan_of(mode, mm, hmax, pp.ov, pp.n_overrides, lanes, ri);
+    vmode = score_vmode(mode, hmax, pp.sc);
+    // an override's plan is kept
+    for (int i = 0; i < pp.n_overrides; ++i)
+        if (mm <= pp.ov[i].max_read_len) return;
+    if (pp.small && !small_rows(ri)) {
+        // a small batch's one launch holds every other row count: the next
+        // larger one (its lanes then cover the read in no more chunks)
+        ++ri;
+        lanes = min(32, (mm + score_rows_at(ri) - 1) / score_rows_at(ri));
+    }
+    // a class with fewer tasks than half its launch's warps (a small batch)
+    // finishes when one task does: fewer rows per lane, on more lanes,
+    // shorten the task while it still fits one row chunk
+    while (ri > 0) {
+        const int64_t per_warp = (int64_t)(32 / lanes) * (mode != MODE_I32 ? 2 : 1);
+        const int64_t tasks = (cnt + per_warp - 1) / per_warp;
+        if (2 * tasks >= pp.score_warps[ri * N_VMODES + vmode]) break;
+        const int r2 = pp.small && !small_rows(ri - 1) ? ri - 2 : ri - 1;
+        const int t2 = (mm + score_rows_at(r2) - 1) / score_rows_at(r2);
+        if (t2 > 32) break;
+        ri = r2;
+        lanes = t2;
+    }
+}
+
+// Whole block; the first warp finishes (no barrier at the end).
+__device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanParams &pp, DevScorePlan *out,
+                                           int32_t *status)
+{
+    __shared__ int32_t s_var[N_CLASS], s_cnt[N_CLASS], s_bnd[N_CLASS], s_lanes[N_CLASS], s_ck[N_CLASS];
+    __shared__ int16_t s_list[N_CLASS];
+    for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
+        const int32_t cnt = info->count[c];
+        int32_t var = -1, bnd = 0, ck = 0;
+        int lanes = 1;
+        if (cnt > 0) {
+            const int mode = c / N_MCLASS;
+            const int32_t mm = info->max_m[c], mn = info->max_n[c];
+            int ri = 0, vmode = mode;
+            plan_class(pp, mode, cnt, mm, mn, lanes, ri, vmode);
+            const int rows = score_rows_at(ri);
+            const int chunks = (mm + lanes * rows - 1) / (lanes * rows);
+            // per group: two buffers x longest window x (H, F) x 4 bytes
+            bnd = chunks > 1 ? 16 * mn : 0;
+            var = ri * N_VMODES + vmode;
+            if (pp.ck_bytes > 0 && mode != MODE_I32) ck = ck_block_rows(rows);
+            out->cls_count[c] = cnt;
+            out->cls_lanes[c] = lanes;
+            out->cls_bnd_bytes[c] = bnd;
+        }
+        s_var[c] = var;
+        s_cnt[c] = cnt;
+        s_bnd[c] = bnd;
+        s_lanes[c] = lanes;
+        s_ck[c] = ck;
+    }
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    // class starts in the sorted order: a warp scan over the counts
+    {
+        constexpr int PER = (N_CLASS + 31) / 32;
+        int32_t sum = 0;
+        for (int i = 0; i < PER; ++i) {
+            const int c = lane * PER + i;
+            if (c < N_CLASS) sum += s_cnt[c];
+        }
+        int32_t x = sum;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
+        }
+        int32_t run = x - sum;
+        for (int i = 0; i < PER; ++i) {
+            const int c = lane * PER + i;
+            if (c < N_CLASS && s_cnt[c]) {
+                out->cls_start[c] = run;
+                run += s_cnt[c];
+            }
+        }
+    }
+    const int n_list = list_classes(s_cnt, s_list);
+    // checkpoints: blocks are doubled until the most they may take fits the
+    // pool (a block of the whole read needs none)
+    {
+        const int64_t limit = min(pp.ck_bytes / 16, (int64_t)0xFFFFFFF0u);
+        int64_t used = 0;
+        int shift = 0;
+        for (;; ++shift) {
+            used = 0;
+            for (int q = lane; q < n_list; q += 32) {
+                const int c = s_list[q];
+                if (s_ck[c])
+                    used += ck_class_units(s_cnt[c], (int64_t)info->sum_n[c], info->max_m[c], info->max_n[c],
+                                           s_lanes[c], s_ck[c] << shift);
+            }
+            for (int d = 16; d; d >>= 1) used += __shfl_xor_sync(0xffffffffu, used, d);
+            if (used <= limit) break;  // at the latest when no read is longer than its block
+        }
+        for (int q = lane; q < n_list; q += 32) out->cls_ck[s_list[q]] = s_ck[s_list[q]] << shift;
+        if (lane == 0) out->ck_units = (used + 15) & ~(int64_t)15;  // 256-byte alignment
+    }
+    // each variant's class list, longest reads first (classes are mode-major,
+    // so within a variant -- one mode -- a larger class index is a longer
+    // read class)
+    static_assert(N_SCORE_VARIANTS <= 32, "a lane per variant");
+    int32_t n = 0;
+    int64_t slot = 0;
+    for (int q = 0; q < n_list; ++q) {
+        const int c = s_list[q];
+        if (s_var[c] == lane) {
+            out->var_cls[lane][n++] = (int16_t)c;
+            slot = max(slot, (int64_t)(32 / s_lanes[c]) * s_bnd[c]);  // a warp's groups
+        }
+    }
+    const unsigned chunked = __ballot_sync(0xffffffffu, slot > 0);
+    if (lane < N_SCORE_VARIANTS) {
+        const int nb = __popc(chunked);
+        const int64_t share = nb ? (pp.score_bnd_bytes / nb) & ~(int64_t)255 : 0;
+        int64_t w = 0;
+        if (slot > 0) {
+            w = min((int64_t)pp.score_warps[lane], share / slot);
+            if (w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's rows do not fit the scratch
+        }
+        out->var_n[lane] = n;
+        out->var_bnd_warps[lane] = (int32_t)w;
+        out->var_bnd_offset[lane] = __popc(chunked & ((1u << lane) - 1u)) * share;
+        out->var_bnd_slot[lane] = slot;
+    }
+}
+
+// Whole block; the first warp finishes.  joint: the 16-bit parts run in one
+// launch, all with 8 lanes per two pairs and slots of one size.
+__device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo *ti, const DevScorePlan *sp,
+                                        const PlanParams &pp, bool joint, DevTbPlan *out, int32_t *status)
+{
+    __shared__ int64_t s_slot[N_TB_PARTS];
+    __shared__ int32_t s_tbcnt[N_CLASS], s_part[N_TB_PARTS];
+    __shared__ int8_t s_pv[N_TB_PARTS];  // each part's variant (-1: none)
+    __shared__ int16_t s_tblist[N_CLASS];
+    __shared__ int32_t s_n16;            // pairs of the 16-bit classes
+    if (threadIdx.x == 0) s_n16 = 0;
+    __syncthreads();
+    for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
+        s_tbcnt[c] = info->count[c];
+        if (c >= N_MCLASS && s_tbcnt[c] > 0) atomicAdd(&s_n16, s_tbcnt[c]);
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
+        const int32_t cnt = s_tbcnt[c];
+        if (!cnt) continue;
+        const int32_t big = ti->n_big[c];
+        const int32_t counts[2] = {big, cnt - big};
+        const int32_t starts[2] = {sp->cls_start[c], sp->cls_start[c] + big};
+        for (int part = 0; part < 2; ++part) {
+            TbPartPlan t{};
+            t.cls = c;
+            t.part = part;
+            t.start = starts[part];
+            t.count = counts[part];
+            t.variant = -1;
+            int64_t slot = 0;
+            if (t.count > 0) {
+                const int64_t need = ti->max_need[c] > 1 ? ti->max_need[c] : 1;
+                // a batch too small to give a task (64 / T pairs) to a
+                // quarter of the warps of a launch spreads each two pairs
+                // over more lanes, and so does a small part of long reads
+                // (its tasks are many blocks one after another): the tasks
+                // then finish sooner, which is what the call waits for
+                int lanes = part == 0 || joint ? 8 : 1;  // wide windows: see kTbWide
+                const int64_t enough = (int64_t)pp.tb_warps[0] * 16;
+                while (lanes < 8 && ((int64_t)s_n16 * lanes < enough ||
+                                     (info->max_m[c] > 512 && (int64_t)t.count * lanes < enough)))
+                    lanes *= 2;
+                slot = tb_part_shape(c / N_MCLASS, pp.allow16 != 0, sp->cls_ck[c], info->max_m[c], need,
+                                     ti->max_wcap[part][c], part, pp.sc, lanes, t);
+                out->part[2 * c + part] = t;
+            }
+            s_slot[2 * c + part] = slot;
+            s_part[2 * c + part] = t.count;
+            s_pv[2 * c + part] = (int8_t)t.variant;
+        }
+    }
+    __syncthreads();
+    // the first warp finishes: each variant's part list (longest reads
+    // first, wide part first), its slot size, and the split
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    const int n_list = list_classes(s_tbcnt, s_tblist);
+    const int64_t ck_words = 4 * sp->ck_units;
+    const int64_t total = pp.tb_bytes / 4 - ck_words;
+    int32_t n = 0;
+    int64_t words = 0, pairs = 0;
+    for (int q = 0; q < n_list; ++q)
+        for (int part = 0; part < 2; ++part) {
+            const int x = 2 * s_tblist[q] + part;
+            if (s_pv[x] == lane) {
+                out->var_part[lane][n++] = (int16_t)x;
+                words = max(words, s_slot[x]);
+                pairs += s_part[x];
+            }
+        }
+    if (joint)
+        for (int v = 0; v < N_TB16_VARIANTS; ++v) {
+            const int64_t o = __shfl_sync(0xffffffffu, words, v);
+            if (lane < N_TB16_VARIANTS) words = max(words, o);
+        }
+    words = (words + 63) & ~(int64_t)63;  // 256-byte alignment
+    int64_t split16 = lane < N_TB16_VARIANTS ? pairs : 0, split32 = lane >= N_TB16_VARIANTS ? pairs : 0;
+    for (int d = 16; d; d >>= 1) {
+        split16 += __shfl_xor_sync(0xffffffffu, split16, d);
+        split32 += __shfl_xor_sync(0xffffffffu, split32, d);
+    }
+    if (lane < N_TB_VARIANTS) {
+        // a slot per warp, as many warps as fit (the launches run one after
+        // another, each with everything the checkpoints leave)
+        const int64_t w = n ? min((int64_t)pp.tb_warps[lane], total / max(words, (int64_t)1)) : 0;
+        if (n && w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's slot does not fit the scratch
+        out->var_n[lane] = n;
+        out->var_slot_words[lane] = words;
+        out->var_slot_offset[lane] = ck_words;
+        out->var_warps[lane] = (int32_t)w;
+    }
+    if (lane == 0) {
+        out->split[0] = split16;
+        out->split[1] = split32;
+    }
+}
+
+}  // namespace swgb

@@ -48,6 +48,35 @@ int score_variant_blocks(int v, int sm_count, int *blocks)
     return SW_OK;
 }
 
+constexpr int kAnySmem = score_snapshot_bytes(50, MODE_I16W, 128);
+
+int launch_score_any(const ScoreLaunch &L, int blocks, cudaStream_t st)
+{
+    if (!L.dp || blocks < 1) return SW_ERR_INTERNAL;
+    ScoreLaunch V = L;
+    void *args[] = {&V};
+    if (cuda_failed(cudaLaunchKernel(score_kernel_any(fma_add_ok(L)), dim3(blocks), dim3(128), args, kAnySmem, st)))
+        return SW_ERR_CUDA;
+    count_launch();
+    return launch_status();
+}
+
+int score_any_blocks(int sm_count, int *blocks)
+{
+    int fewest = 0;
+    for (int f = 0; f < 2; ++f) {
+        const void *fn = score_kernel_any(f);
+        int bps = 0;
+        if (cuda_failed(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kAnySmem)) ||
+            cuda_failed(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 128, kAnySmem)))
+            return SW_ERR_CUDA;
+        fewest = f == 0 ? bps : std::min(fewest, bps);
+    }
+    if (fewest < 1) return SW_ERR_INTERNAL;
+    *blocks = fewest * sm_count;
+    return SW_OK;
+}
+
 // Registers and resident blocks per SM of the (rows, mode) kernels; also
 // lets them take their dynamic shared memory, so it runs before any launch
 // of them (both diagonal-add forms, with and without checkpoints; the grid

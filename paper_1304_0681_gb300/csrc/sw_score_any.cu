@@ -1,0 +1,41 @@
+// sw_score_any.cu -- the score pass of a small batch in one launch: the bodies
+// of four row counts in every mode, run for the variants that have classes.
+// (255 registers, so 8 warps per SM whatever runs: a small batch has no more
+// tasks than that.)
+#include "sw_score_kernel.cuh"
+
+namespace swgb {
+
+template <int R, bool FMA_ADD>
+__device__ __forceinline__ void score_rows_any(const ScoreLaunch &L, int v)
+{
+    switch (v % N_VMODES) {
+    case MODE_I32: score_body<R, MODE_I32, true, false>(L, v); break;
+    case MODE_I16: score_body<R, MODE_I16, FMA_ADD, true>(L, v); break;
+    case MODE_I16W: score_body<R, MODE_I16W, FMA_ADD, true>(L, v); break;
+    default: score_body<R, MODE_I16S, FMA_ADD, true>(L, v); break;
+    }
+}
+
+template <bool FMA_ADD>
+__global__ void __launch_bounds__(128) k_score_any(const __grid_constant__ ScoreLaunch L)
+{
+    for (int v = N_SCORE_VARIANTS - 1; v >= 0; --v) {
+        if (L.dp->var_n[v] == 0) continue;
+        switch (v / N_VMODES) {
+        case 0: score_rows_any<8, FMA_ADD>(L, v); break;
+        case 1: score_rows_any<16, FMA_ADD>(L, v); break;
+        case 3: score_rows_any<25, FMA_ADD>(L, v); break;
+        case 5: score_rows_any<50, FMA_ADD>(L, v); break;
+        default: break;
+        }
+        __syncthreads();
+    }
+}
+
+const void *score_kernel_any(bool fma)
+{
+    return fma ? (const void *)k_score_any<true> : (const void *)k_score_any<false>;
+}
+
+}  // namespace swgb

@@ -219,7 +219,7 @@ __host__ __device__ constexpr int score_snapshot_bytes(int rows, int mode, int t
 // CK: checkpoints are kept for a traceback (launches without a CIGAR to
 // follow run the kernels without that code: 1 % faster).
 template <int R, int MODE, bool FMA_ADD, bool CK>
-__global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
+__device__ __forceinline__ void score_body(const ScoreLaunch &L, const int variant)
 {
     typedef Arith<MODE> A;
     typedef typename A::V V;
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
     const bool planned = L.dp != nullptr;
     if (lane == 0) {
         cc->ci = 0;
-        cc->n_cls = planned ? L.dp->var_n[L.variant] : 1;
+        cc->n_cls = planned ? L.dp->var_n[variant] : 1;
     }
     __syncwarp();
     for (; cc->ci < cc->n_cls; __syncwarp(), cc->ci = cc->ci + (lane == 0 ? 1 : 0), __syncwarp()) {
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
     int64_t bnd_warp_bytes = 0;  // warp stride of the boundary slots (host-given: G groups of this class)
     if (planned) {
         const DevScorePlan &dp = *L.dp;
-        cls = dp.var_cls[L.variant][ci];
+        cls = dp.var_cls[variant][ci];
         T = dp.cls_lanes[cls];
         order = L.order + dp.cls_start[cls];
         n_items = dp.cls_count[cls];
@@ -312,11 +312,11 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
         bnd_base = nullptr;
         if (bnd_group_bytes) {
             // reads in several row chunks: only warps with a boundary slot
-            if (warp_global >= dp.var_bnd_warps[L.variant]) continue;
-            bnd_base = L.boundary + dp.var_bnd_offset[L.variant];
+            if (warp_global >= dp.var_bnd_warps[variant]) continue;
+            bnd_base = L.boundary + dp.var_bnd_offset[variant];
             // every class of the variant uses the same warp stride, so that
             // warps working on different classes never share bytes
-            bnd_warp_bytes = dp.var_bnd_slot[L.variant];
+            bnd_warp_bytes = dp.var_bnd_slot[variant];
         }
     }
     const int G = 32 / T;
@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
         cc->work_counter = work_counter;
         cc->n_items = n_items;
         cc->cls = cls;
-        if (CK) cc->ck_rows = planned ? L.dp->cls_ck[cls] : 0;
+        if (CK) cc->ck_rows = planned && L.ck_pos ? L.dp->cls_ck[cls] : 0;
         cc->bnd_warp = bnd_base ? bnd_base + warp_global * bnd_warp_bytes : nullptr;
         cc->bnd_group_bytes = bnd_group_bytes;
     }
@@ -680,6 +680,12 @@ __global__ void __launch_bounds__(128) k_score(const ScoreLaunch L)
     }  // classes
 }
 
+template <int R, int MODE, bool FMA_ADD, bool CK>
+__global__ void __launch_bounds__(128) k_score(const __grid_constant__ ScoreLaunch L)
+{
+    score_body<R, MODE, FMA_ADD, CK>(L, L.variant);
+}
+
 // The kernel of a mode, with or without checkpoints (the int32 mode keeps none).
 template <int R, bool CK>
 const void *score_kernel_of(int mode, bool fma)
@@ -713,5 +719,7 @@ const void *score_kernel_at(int rows, int mode, bool fma)
 // (sw_score_ck.cu): two translation units, compiled in parallel.
 const void *score_kernel(int rows, int mode, bool fma);
 const void *score_kernel_ck(int rows, int mode, bool fma);
+// A small batch's kernel (sw_score_any.cu).
+const void *score_kernel_any(bool fma);
 
 }  // namespace swgb

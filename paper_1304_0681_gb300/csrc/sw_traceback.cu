@@ -596,12 +596,11 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
     const int g = lane / T, k = lane % T;
     const int64_t warp_global = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const DevTbPlan &dp = *L.dp;
-    const int v = L.variant;
     // input already found invalid (an unsupported size means some pairs were
     // not scored, so the traceback order is incomplete): do nothing
     if (*(volatile const int32_t *)L.status & (ST_BAD_INPUT | ST_UNSUPPORTED)) return;
-    if (warp_global >= dp.var_warps[v]) return;  // no scratch slot
-    uint32_t *const slot = L.slab + dp.var_slot_offset[v] + warp_global * dp.var_slot_words[v];
+    // (the variants of one launch share the size of a slot)
+    uint32_t *const slot = L.slab + dp.var_slot_offset[L.variant] + warp_global * dp.var_slot_words[L.variant];
     const uint32_t GE2 = splat16(P.sc.ge), GO2 = splat16(P.sc.go);
     const uint32_t one = (uint32_t)L.one;
     const uint32_t m1 = 0u - one, two = one + one, four = two + two, eight = four + four;
@@ -622,6 +621,9 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
     };
     __shared__ PartCtx s_pc[4];
     volatile PartCtx *const pc = &s_pc[threadIdx.x >> 5];
+    for (int v = L.variant; v < L.variant + L.n_variants; ++v) {
+    if (warp_global >= dp.var_warps[v]) continue;  // no scratch slot
+    __syncwarp();
     if (lane == 0) pc->pi = 0;
     __syncwarp();
     for (; pc->pi < dp.var_n[v]; __syncwarp(), pc->pi = pc->pi + (lane == 0 ? 1 : 0), __syncwarp()) {
@@ -1109,6 +1111,7 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
         }
     }
     }  // parts
+    }  // variants
 }
 
 // A device-planned launch of traceback variant v: the 16-bit kernel with

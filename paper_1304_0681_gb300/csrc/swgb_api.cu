@@ -55,6 +55,7 @@ struct Buffer {
 struct ExecCtx {
     int score_blocks[N_SCORE_VARIANTS] = {};
     int tb_blocks[N_TB_VARIANTS] = {};
+    int any_blocks = 0;
     cudaStream_t aux[kAuxStreams] = {};
     cudaEvent_t fork_ev = nullptr;
     cudaEvent_t join_ev[kAuxStreams] = {};
@@ -69,6 +70,7 @@ int exec_ctx_init(ExecCtx &x, int sm_count)
         if ((rc = score_variant_blocks(v, sm_count, &x.score_blocks[v]))) return rc;
     for (int v = 0; v < N_TB_VARIANTS; ++v)
         if ((rc = traceback_variant_blocks(v, sm_count, &x.tb_blocks[v]))) return rc;
+    if ((rc = score_any_blocks(sm_count, &x.any_blocks))) return rc;
     for (int k = 0; k < kAuxStreams; ++k) {
         if (cuda_failed(cudaStreamCreateWithFlags(&x.aux[k], cudaStreamNonBlocking))) return SW_ERR_CUDA;
         if (cuda_failed(cudaEventCreateWithFlags(&x.join_ev[k], cudaEventDisableTiming))) return SW_ERR_CUDA;
@@ -325,6 +327,81 @@ PlanParams plan_params(const ExecCtx &x, const Scoring &sc, bool allow16, int64_
     return pp;
 }
 
+// The score launches' and the traceback launches' parameters of a batch.
+ScoreLaunch score_launch(const PairSet &ps, const Scoring &sc, int32_t *out_score, int32_t *out_end, bool cigar,
+                         const Scratch &S)
+{
+    ScoreLaunch L{};
+    L.ps = ps;
+    L.sc = sc;
+    L.order = S.order;
+    L.out_score = out_score;
+    L.out_end = out_end;
+    L.boundary = S.score_bnd;
+    L.work_counter = S.counters;
+    L.status = &S.info->status;
+    if (cigar) {
+        L.tb_keys = S.tb_keys;
+        L.tb_hist = S.hist;
+        L.tb_info = S.tbinfo;
+        L.ck_pool = (uint4 *)S.tb;
+        L.ck_cursor = (uint32_t *)(S.counters + CTR_CK);
+        L.ck_pos = S.ck_pos;
+    }
+    L.dp = S.splan;
+    return L;
+}
+
+TracebackLaunch traceback_launch(const PairSet &ps, const Scoring &sc, const int32_t *out_score,
+                                 const int32_t *out_end, const sw_cigar_t &cig, const Scratch &S)
+{
+    TracebackLaunch B{};
+    B.P = TbParams{ps, sc, out_score, out_end, cig.ops, cig.offsets, cig.n_ops, (const uint4 *)S.tb, S.ck_pos};
+    B.order = S.tb_order;
+    B.slab = S.tb;
+    B.work_counter = S.counters + CTR_TB;
+    B.status = &S.info->status;
+    B.dp = S.tplan;
+    return B;
+}
+
+// A small batch on st (sw_small.cu): the same results in six launches.
+int enqueue_small(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scoring &sc, int score_setting,
+                  PlanParams pp, int32_t *out_score, int32_t *out_end, const sw_cigar_t *cig, const Scratch &S,
+                  const int32_t *expect, const ExecCtx &x, cudaStream_t st)
+{
+    int rc = SW_OK;
+    const bool timing = x.timing && x.phase;
+    pp.small = 1;
+    for (int v = 0; v < N_SCORE_VARIANTS; ++v) pp.score_warps[v] = x.any_blocks * (kThreads / 32);
+    auto blocks = [&](int full) { return (int)std::min<int64_t>(full, n_pairs); };
+    if (timing && cuda_failed(cudaEventRecord(x.phase[0], st))) return SW_ERR_CUDA;
+    if ((rc = launch_small_plan(ps, n_reads, n_pairs, sc, score_setting, pp, expect, S.info, S.tbinfo, S.counters,
+                                cig ? S.tb_keys : nullptr, S.order, out_score, out_end, cig ? cig->n_ops : nullptr,
+                                S.splan, st)))
+        return rc;
+    if (timing && cuda_failed(cudaEventRecord(x.phase[1], st))) return SW_ERR_CUDA;
+    if ((rc = launch_score_any(score_launch(ps, sc, out_score, out_end, cig != nullptr, S), blocks(x.any_blocks), st)))
+        return rc;
+    if (timing && cuda_failed(cudaEventRecord(x.phase[2], st))) return SW_ERR_CUDA;
+    if (cig) {
+        if ((rc = launch_small_tbplan(S.tb_keys, n_pairs, S.info, S.tbinfo, S.splan, pp, S.tb_order, S.tplan,
+                                      &S.info->status, st)))
+            return rc;
+        // the wide and the narrow windows (8 lanes per two pairs: so few
+        // pairs never take fewer), then the int32 kernels
+        TracebackLaunch B = traceback_launch(ps, sc, out_score, out_end, *cig, S);
+        B.n_variants = 2;
+        const bool fma = sc.mi >= sc.go;
+        if ((rc = launch_traceback_variant(0, fma, B, blocks(x.tb_blocks[0]), st))) return rc;
+        B.n_variants = 1;
+        for (int v : {TB_VAR_TILED, TB_VAR_GROUPED})
+            if ((rc = launch_traceback_variant(v, fma, B, blocks(x.tb_blocks[v]), st))) return rc;
+    }
+    if (timing && cuda_failed(cudaEventRecord(x.phase[3], st))) return SW_ERR_CUDA;
+    return SW_OK;
+}
+
 // Enqueues one whole batch on st: classification, the device planners,
 // every score variant (forked over the auxiliary streams), and with a CIGAR
 // the traceback sort, its planner and every traceback variant.  A fixed
@@ -337,6 +414,8 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
     int rc = SW_OK;
     const size_t nh = (size_t)N_CLASS * N_NBUCKET;
     const PlanParams pp = plan_params(x, sc, allow16, S.score_bnd_bytes, S.tb_bytes);
+    if (n_pairs <= kSmallPairs && pp.n_overrides == 0)
+        return enqueue_small(ps, n_reads, n_pairs, sc, score_setting, pp, out_score, out_end, cig, S, expect, x, st);
     const bool timing = x.timing && x.phase;
     if (timing && cuda_failed(cudaEventRecord(x.phase[0], st))) return SW_ERR_CUDA;
     if (cuda_failed(cudaMemsetAsync(S.hist, 0, sizeof(int32_t) * nh, st))) return SW_ERR_CUDA;
@@ -356,27 +435,9 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
     }
     if (timing && cuda_failed(cudaEventRecord(x.phase[1], st))) return SW_ERR_CUDA;
     if ((rc = fork_streams(x, st, kAuxStreams))) return rc;
-    for (int v = 0; v < N_SCORE_VARIANTS; ++v) {
-        ScoreLaunch L{};
-        L.ps = ps;
-        L.sc = sc;
-        L.order = S.order;
-        L.out_score = out_score;
-        L.out_end = out_end;
-        L.boundary = S.score_bnd;
-        L.work_counter = S.counters;
-        L.status = &S.info->status;
-        if (cig) {
-            L.tb_keys = S.tb_keys;
-            L.tb_hist = S.hist;
-            L.tb_info = S.tbinfo;
-            L.ck_pool = (uint4 *)S.tb;
-            L.ck_cursor = (uint32_t *)(S.counters + CTR_CK);
-            L.ck_pos = S.ck_pos;
-        }
-        L.dp = S.splan;
+    const ScoreLaunch L = score_launch(ps, sc, out_score, out_end, cig != nullptr, S);
+    for (int v = 0; v < N_SCORE_VARIANTS; ++v)
         if ((rc = launch_score_variant(v, L, x.score_blocks[v], x.aux[v % kAuxStreams]))) return rc;
-    }
     if ((rc = join_streams(x, st, kAuxStreams))) return rc;
     if (timing && cuda_failed(cudaEventRecord(x.phase[2], st))) return SW_ERR_CUDA;
     if (cig) {
@@ -384,20 +445,11 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
                                       st)))
             return rc;
         if ((rc = launch_plan_tb(S.info, S.tbinfo, S.splan, pp, S.tplan, &S.info->status, st))) return rc;
-        const TbParams P{ps, sc, out_score, out_end, cig->ops, cig->offsets, cig->n_ops, (const uint4 *)S.tb,
-                         S.ck_pos};
         const bool fma = sc.mi >= sc.go;
+        const TracebackLaunch B = traceback_launch(ps, sc, out_score, out_end, *cig, S);
         // one after another: each launch has the whole slot budget
-        for (int v = 0; v < N_TB_VARIANTS; ++v) {
-            TracebackLaunch B{};
-            B.P = P;
-            B.order = S.tb_order;
-            B.slab = S.tb;
-            B.work_counter = S.counters + CTR_TB;
-            B.status = &S.info->status;
-            B.dp = S.tplan;
+        for (int v = 0; v < N_TB_VARIANTS; ++v)
             if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], st))) return rc;
-        }
     }
     if (timing && cuda_failed(cudaEventRecord(x.phase[3], st))) return SW_ERR_CUDA;
     return SW_OK;

@@ -157,6 +157,7 @@ struct TracebackLaunch {
     int32_t one = 1;         // a multiplier the compiler cannot fold
     const DevTbPlan *dp = nullptr;
     int32_t variant = 0;
+    int32_t n_variants = 1;  // variants from `variant` on that this launch serves (of one kernel, equal slots)
 };
 
 // Row counts compiled for the score kernels.
@@ -202,6 +203,12 @@ constexpr int kTbWide = 256;
 constexpr int kMaxPlanOverrides = 16;
 constexpr int kPlanThreads = 384;                         // >= N_CLASS
 
+// Batches of up to this many pairs (without plan overrides) take the few
+// launches of sw_small.cu.
+constexpr int kSmallPairs = 4096;
+// Row counts in the one score launch of a small batch (8, 16, 25, 50).
+__host__ __device__ inline bool small_rows(int rows_idx) { return rows_idx != 2 && rows_idx != 4; }
+
 struct PlanOverride {
     int32_t max_read_len, lanes, rows;
 };
@@ -217,6 +224,7 @@ struct PlanParams {
     int64_t tb_bytes;                       // traceback scratch: row checkpoints, then the warps' slots
     int64_t ck_bytes;                       // most of it that row checkpoints may take (0: none)
     int32_t allow16;                        // 16-bit traceback allowed (SW_TB_AUTO)
+    int32_t small;                          // the launches of a small batch
 };
 
 struct DevScorePlan {
@@ -428,7 +436,18 @@ int launch_plan_tb(const ClassInfo *info, const TbClassInfo *ti, const DevScoreP
 // full occupancy; its grid (blocks) comes from score_variant_blocks.
 int launch_score_variant(int v, const ScoreLaunch &L, int blocks, cudaStream_t st);
 int score_variant_blocks(int v, int sm_count, int *blocks);
+// (n_variants > 1: as many variants from v on that share a kernel)
 int launch_traceback_variant(int v, bool fma, const TracebackLaunch &L, int blocks, cudaStream_t st);
+// The one score launch of a small batch: every class of every variant.
+int launch_score_any(const ScoreLaunch &L, int blocks, cudaStream_t st);
+int score_any_blocks(int sm_count, int *blocks);
+int launch_small_plan(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scoring &sc, int score_setting,
+                      const PlanParams &pp, const int32_t *expect, ClassInfo *info, TbClassInfo *tbinfo,
+                      int32_t *counters, int32_t *tb_keys, int32_t *order, int32_t *out_score, int32_t *out_end,
+                      int32_t *cig_n, DevScorePlan *splan, cudaStream_t st);
+int launch_small_tbplan(const int32_t *tb_keys, int64_t n_pairs, const ClassInfo *info, const TbClassInfo *tbinfo,
+                        const DevScorePlan *splan, const PlanParams &pp, int32_t *tb_order, DevTbPlan *tplan,
+                        int32_t *status, cudaStream_t st);
 int traceback_variant_blocks(int v, int sm_count, int *blocks);
 // Work counters of one batch: score (per class), traceback (per part), and
 // the checkpoint pool's cursor.
