@@ -39,16 +39,16 @@ __device__ __forceinline__ Band band_of(int32_t score, int32_t ie, int32_t je, c
     return q;
 }
 
-// Traceback sort key of a pair of class cls (class-major): pairs whose chunk
-// window is wider than kTbWide first, then the rest, each by falling chunk
-// window (~9 % and ~4 % buckets).  A warp sweeps the widest window of its
+// Traceback sort key of a pair of class cls (class-major): by part, each by
+// falling chunk window (~9 % and ~2 % buckets, single columns in the last
+// part).  A warp sweeps the widest window of its
 // pairs at every chunk, so pairs of one task should share the width: sorted
 // by it, a task of the 1M-pair batch of 100 x 200 pairs sweeps 1.07x the
 // cells of its pairs' own windows, against 1.24x sorted by rows x width.
 // Also the one-lane slab words (need) and chunk window (wc) the launch sizing
 // uses.  score <= 0: no alignment (width 0, need 0).
 __device__ __forceinline__ void tb_cost_key(int cls, int32_t score, int32_t ie, int32_t je, const Scoring &sc,
-                                            int32_t &key, int32_t &need32, int32_t &wc, bool &big)
+                                            int32_t &key, int32_t &need32, int32_t &wc)
 {
     int64_t need = 0;
     wc = 0;
@@ -58,35 +58,34 @@ __device__ __forceinline__ void tb_cost_key(int cls, int32_t score, int32_t ie, 
         need = (int64_t)((t.rows + 7) / 8) * w;
         wc = w;
     }
-    const float lw = __log2f((float)(wc > 1 ? wc : 1));
-    big = wc > kTbWide;
-    if (big) {
-        const int cb = min(63, max(0, (int)(8.f * lw) - 64));
-        key = cls * N_NBUCKET + (63 - cb);
-    } else {
-        const int cb = min(191, max(0, (int)(16.f * lw)));
-        key = cls * N_NBUCKET + 64 + (191 - cb);
+    const int part = tb_part_of(wc);
+    int b = 128 + 2 * (kTbMid - wc);                         // 1 .. 64 columns (0: no alignment) in 128 .. 256
+    if (part < 2) {
+        const float lw = __log2f((float)wc);
+        b = part == 0 ? 63 - min(63, max(0, (int)(8.f * lw) - 64))      // from 2^8 on
+                      : 127 - min(63, max(0, (int)(32.f * lw) - 192));  // 2^6 to 2^8
     }
+    key = cls * N_NBUCKET + min(b, N_NBUCKET - 1);
     need32 = (int32_t)(need < (int64_t)INT32_MAX ? need : (int64_t)INT32_MAX);
 }
 
 // Adds a warp's keys to the traceback histogram and class table, one set of
 // atomics per distinct key (every lane of the warp calls it; key < 0: none).
-__device__ __forceinline__ void tb_key_atomics(int32_t key, int cls, int32_t need32, int32_t wc, bool big,
-                                               int32_t *hist, TbClassInfo *info)
+__device__ __forceinline__ void tb_key_atomics(int32_t key, int cls, int32_t need32, int32_t wc, int32_t *hist,
+                                               TbClassInfo *info)
 {
     const KeyGroup g = key_group(key);
     if (key >= 0) {
         const unsigned mx_need = __reduce_max_sync(g.mask, (unsigned)need32);
         const unsigned mx_wc = __reduce_max_sync(g.mask, (unsigned)wc);
-        const unsigned n_big = __reduce_add_sync(g.mask, (unsigned)(big && need32 > 0));
+        const int part = tb_part_of(wc);  // one per key
         if (g.rank == 0) {
             atomicAdd(&hist[key], g.size);
             if (mx_need > 0) {
                 atomicMax(&info->max_need[cls], (int32_t)mx_need);
-                atomicMax(&info->max_wcap[big ? 0 : 1][cls], (int32_t)mx_wc);
+                atomicMax(&info->max_wcap[part][cls], (int32_t)mx_wc);
             }
-            if (n_big) atomicAdd(&info->n_big[cls], (int32_t)n_big);
+            if (part < 2) atomicAdd(&info->n_part[part][cls], g.size);
         }
     }
 }

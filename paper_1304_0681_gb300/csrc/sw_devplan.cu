@@ -15,7 +15,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_plan_tb(const ClassInfo *__res
                                                           const DevScorePlan *__restrict__ sp, const PlanParams pp,
                                                           DevTbPlan *__restrict__ out, int32_t *__restrict__ status)
 {
-    plan_tb(info, ti, sp, pp, false, out, status);
+    plan_tb(info, ti, sp, pp, out, status);
 }
 
 int launch_plan_score(const ClassInfo *info, const PlanParams &pp, DevScorePlan *out, int32_t *status,

@@ -182,56 +182,66 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
     }
 }
 
-// Whole block; the first warp finishes.  joint: the 16-bit parts run in one
-// launch, all with 8 lanes per two pairs and slots of one size.
+// Whole block; the first warp finishes.
 __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo *ti, const DevScorePlan *sp,
-                                        const PlanParams &pp, bool joint, DevTbPlan *out, int32_t *status)
+                                        const PlanParams &pp, DevTbPlan *out, int32_t *status)
 {
     __shared__ int64_t s_slot[N_TB_PARTS];
     __shared__ int32_t s_tbcnt[N_CLASS], s_part[N_TB_PARTS];
     __shared__ int8_t s_pv[N_TB_PARTS];  // each part's variant (-1: none)
     __shared__ int16_t s_tblist[N_CLASS];
-    __shared__ int32_t s_n16;            // pairs of the 16-bit classes
-    if (threadIdx.x == 0) s_n16 = 0;
+    __shared__ int32_t s_n16[kTbParts];  // pairs of the 16-bit classes by part
+    if (threadIdx.x < kTbParts) s_n16[threadIdx.x] = 0;
     __syncthreads();
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
-        s_tbcnt[c] = info->count[c];
-        if (c >= N_MCLASS && s_tbcnt[c] > 0) atomicAdd(&s_n16, s_tbcnt[c]);
+        const int32_t cnt = s_tbcnt[c] = info->count[c];
+        if (c >= N_MCLASS && cnt > 0) {
+            atomicAdd(&s_n16[0], ti->n_part[0][c]);
+            atomicAdd(&s_n16[1], ti->n_part[1][c]);
+            atomicAdd(&s_n16[2], cnt);
+        }
     }
     __syncthreads();
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = s_tbcnt[c];
         if (!cnt) continue;
-        const int32_t big = ti->n_big[c];
-        const int32_t counts[2] = {big, cnt - big};
-        const int32_t starts[2] = {sp->cls_start[c], sp->cls_start[c] + big};
-        for (int part = 0; part < 2; ++part) {
+        const int32_t n0 = ti->n_part[0][c], n1 = ti->n_part[1][c];
+        const int32_t counts[kTbParts] = {n0, n1, cnt - n0 - n1};
+        int32_t start = sp->cls_start[c];
+        for (int part = 0; part < kTbParts; ++part) {
             TbPartPlan t{};
             t.cls = c;
             t.part = part;
-            t.start = starts[part];
+            t.start = start;
             t.count = counts[part];
             t.variant = -1;
+            start += t.count;
             int64_t slot = 0;
             if (t.count > 0) {
                 const int64_t need = ti->max_need[c] > 1 ? ti->max_need[c] : 1;
-                // a batch too small to give a task (64 / T pairs) to a
-                // quarter of the warps of a launch spreads each two pairs
-                // over more lanes, and so does a small part of long reads
-                // (its tasks are many blocks one after another): the tasks
-                // then finish sooner, which is what the call waits for
-                int lanes = part == 0 || joint ? 8 : 1;  // wide windows: see kTbWide
-                const int64_t enough = (int64_t)pp.tb_warps[0] * 16;
-                while (lanes < 8 && ((int64_t)s_n16 * lanes < enough ||
-                                     (info->max_m[c] > 512 && (int64_t)t.count * lanes < enough)))
+                // Lanes per two pairs.  A batch too small to give a wave of
+                // warps tasks of 64 / T pairs spreads each two pairs over
+                // more lanes: its tasks (several blocks one after another)
+                // then finish sooner, which is what the call waits for.  The
+                // smallest run with 16 lanes in one launch; else the narrow
+                // windows of a batch stay at one lane from a quarter of a
+                // wave on (their tasks are short), the others from a whole
+                // wave of such pairs on, and long reads follow their
+                // class's count.
+                const int64_t wave = (int64_t)pp.tb_warps[0] * 64;
+                const int64_t all = s_n16[2], same = part < 2 ? s_n16[part] : all;
+                const int64_t enough = part < 2 ? wave : wave / 4;
+                int lanes = pp.small || 16 * all < wave ? 16 : part == 0 ? 8 : 1;  // (wide windows: see kTbWide)
+                while (lanes < 16 &&
+                       (same * lanes < enough || (info->max_m[c] > 512 && (int64_t)cnt * lanes < wave / 4)))
                     lanes *= 2;
                 slot = tb_part_shape(c / N_MCLASS, pp.allow16 != 0, sp->cls_ck[c], info->max_m[c], need,
                                      ti->max_wcap[part][c], part, pp.sc, lanes, t);
-                out->part[2 * c + part] = t;
+                out->part[kTbParts * c + part] = t;
             }
-            s_slot[2 * c + part] = slot;
-            s_part[2 * c + part] = t.count;
-            s_pv[2 * c + part] = (int8_t)t.variant;
+            s_slot[kTbParts * c + part] = slot;
+            s_part[kTbParts * c + part] = t.count;
+            s_pv[kTbParts * c + part] = (int8_t)t.variant;
         }
     }
     __syncthreads();
@@ -245,19 +255,19 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
     int32_t n = 0;
     int64_t words = 0, pairs = 0;
     for (int q = 0; q < n_list; ++q)
-        for (int part = 0; part < 2; ++part) {
-            const int x = 2 * s_tblist[q] + part;
+        for (int part = 0; part < kTbParts; ++part) {
+            const int x = kTbParts * s_tblist[q] + part;
             if (s_pv[x] == lane) {
                 out->var_part[lane][n++] = (int16_t)x;
                 words = max(words, s_slot[x]);
                 pairs += s_part[x];
             }
         }
-    if (joint)
-        for (int v = 0; v < N_TB16_VARIANTS; ++v) {
-            const int64_t o = __shfl_sync(0xffffffffu, words, v);
-            if (lane < N_TB16_VARIANTS) words = max(words, o);
-        }
+    // the variants of one launch share the size of a slot
+    {
+        const int64_t o = __shfl_xor_sync(0xffffffffu, words, 1);
+        if (lane < 4) words = max(words, o);
+    }
     words = (words + 63) & ~(int64_t)63;  // 256-byte alignment
     int64_t split16 = lane < N_TB16_VARIANTS ? pairs : 0, split32 = lane >= N_TB16_VARIANTS ? pairs : 0;
     for (int d = 16; d; d >>= 1) {

@@ -657,7 +657,6 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
         for (int h2 = 0; h2 < (PAIR2 ? 2 : 1); ++h2) {
             const int64_t it = item + h2;
             int32_t tkey = -1, need32 = 0, wc = 0;
-            bool big = false;
             if (on && k == 0 && it < cc->n_items) {
                 const uint64_t b = h2 ? bestB : bestA;
                 const int32_t p = cc->order[it];
@@ -667,14 +666,14 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                 L.out_end[2 * p] = ie;
                 L.out_end[2 * p + 1] = je;
                 if (L.tb_keys) {
-                    tb_cost_key(cc->cls, (int32_t)sc, ie, je, L.sc, tkey, need32, wc, big);
+                    tb_cost_key(cc->cls, (int32_t)sc, ie, je, L.sc, tkey, need32, wc);
                     L.tb_keys[p] = tkey;
                     if (CK && cc->ck_rows)
                         L.ck_pos[p] = make_uint2(cc->ck_base + (uint32_t)(g * cc->ck_n * cc->ck_row_units),
                                                  (uint32_t)(2 * cc->ck_row_units + h2));
                 }
             }
-            if (L.tb_keys) tb_key_atomics(tkey, cc->cls, need32, wc, big, L.tb_hist, L.tb_info);
+            if (L.tb_keys) tb_key_atomics(tkey, cc->cls, need32, wc, L.tb_hist, L.tb_info);
         }
     }
     }  // classes

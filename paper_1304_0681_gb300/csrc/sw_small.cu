@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kSmallThreads)
     bitonic_sort(s_key, np);
     for (int i = threadIdx.x; i < n_pairs; i += blockDim.x)
         if (s_key[i] != 0xFFFFFFFFu) tb_order[i] = (int32_t)(s_key[i] & 0xFFFu);
-    plan_tb(info, tbinfo, splan, pp, true, tplan, status);
+    plan_tb(info, tbinfo, splan, pp, tplan, status);
 }
 
 int launch_small_plan(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scoring &sc, int score_setting,

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(128) k_traceback(const TracebackLaunch L)
     const int64_t slab_words = tp.slab_words, bnd_ints = tp.bnd_ints;
     const int32_t *const order = L.order + tp.start;
     const int64_t n_items = tp.count;
-    int32_t *const counter = L.work_counter + 2 * tp.cls + tp.part;
+    int32_t *const counter = L.work_counter + kTbParts * tp.cls + tp.part;
     // the warp's slot: TILED -> one tile indexed with the lane, then the
     // boundary rows; else every group's slab, then every group's boundary row
     uint32_t *slab = !on ? nullptr : TILED ? slot : slot + g * slab_words;
@@ -457,8 +457,8 @@ __global__ void __launch_bounds__(128) k_traceback(const TracebackLaunch L)
 // by whole-read bands took 45 ms, plus 7.5 ms for walks in kernels of their
 // own.
 //
-// Sweep.  Lane k of a group holds 8 rows of a chunk of 8T rows on a one-step
-// wavefront.  A lane stores two 32-bit words per window offset (rows 0-3 and
+// Sweep.  Lane k of a group holds 8 rows (4 with 16 lanes) of a chunk of 8T
+// (64) rows on a one-step wavefront.  A lane stores two 32-bit words per window offset (rows 0-3 and
 // rows 4-7; pair A in bits 0-15, pair B in bits 16-31), and its words of four
 // consecutive offsets share one 32-byte sector: uint2
 // [((chunk x S4 + t / 4) x 32 + lane) x 4 + t % 4].  Per cell four bits record
@@ -581,7 +581,8 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
 {
     constexpr int G = 32 / T;       // groups per warp, two pairs each
     constexpr int PAIRS = 2 * G;    // pairs per task
-    constexpr int rc = T * TB_ROWS; // rows per chunk
+    constexpr int ROWS = tb16_rows(T);  // rows per lane
+    constexpr int rc = T * ROWS;        // rows per chunk
     const TbParams &P = L.P;
     // s_tab[w] byte x = s(x, w) - o; s_tab[4] = 0 (s = o, past a window end)
     __shared__ uint32_t s_tab[8];
@@ -631,9 +632,9 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
         const TbPartPlan &pp = dp.part[dp.var_part[v][pc->pi]];
         const int32_t s4 = (pp.wcap + T - 1 + 3) >> 2;
         pc->order = L.order + pp.start;
-        pc->ctr = L.work_counter + 2 * pp.cls + pp.part;
+        pc->ctr = L.work_counter + kTbParts * pp.cls + pp.part;
         pc->bnd = (uint4 *)(slot + ((32 * pp.slab_words + 63) & ~(int64_t)63));
-        pc->lane_chunks = pp.slab_words / (8 * (int64_t)max(s4, 1));
+        pc->lane_chunks = pp.slab_words / (ROWS * (int64_t)max(s4, 1));
         pc->n_items = pp.count;
         pc->wcap = pp.wcap;
         pc->s4 = s4;
@@ -816,29 +817,30 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                     ww[x] = 0u;
                     wn[x] = rem[x] > 0 ? load_bases(P.ps.wins, tp.ws[wi] + lo[x], min(16, rem[x])) : 0u;
                     codes[x] = 0x44444444u;  // 4 bits per row, 4 = no base
-                    const int row = tp.i0[wi] + c * rc + k * TB_ROWS;
-                    const int cnt = rem[x] > 0 ? min(TB_ROWS, tp.i[wi] - row + 1) : 0;
+                    const int row = tp.i0[wi] + c * rc + k * ROWS;
+                    const int cnt = rem[x] > 0 ? min(ROWS, tp.i[wi] - row + 1) : 0;
                     if (cnt > 0) {
                         const uint32_t w = load_bases(P.ps.reads, tp.rs[wi] + row, cnt);
 #pragma unroll
-                        for (int r = 0; r < TB_ROWS; ++r)
+                        for (int r = 0; r < ROWS; ++r)
                             if (r < cnt)
                                 codes[x] = (codes[x] & ~(0xFu << (4 * r))) | (((w >> (2 * r)) & 3u) << (4 * r));
                     }
                 }
-                uint32_t sel[TB_ROWS];
+                uint32_t sel[ROWS];
 #pragma unroll
-                for (int r = 0; r < TB_ROWS; ++r)
+                for (int r = 0; r < ROWS; ++r)
                     sel[r] = sel16((codes[0] >> (4 * r)) & 0xFu, (codes[1] >> (4 * r)) & 0xFu);
-                uint32_t E[TB_ROWS], Hp[TB_ROWS];
+                uint32_t E[ROWS], Hp[ROWS];
 #pragma unroll
-                for (int r = 0; r < TB_ROWS; ++r) {
+                for (int r = 0; r < ROWS; ++r) {
                     E[r] = 0u;
                     Hp[r] = 0u;
                 }
                 uint32_t diag_in = prmt(dg0, dg1, 0x5410u);
                 uint32_t out_h = 0u, out_f = 0u;
-                uint4 *tile = (uint4 *)slot + ((int64_t)c * pc->s4 * 32 + lane) * 2;  // sector of steps t0 .. t0 + 3
+                // a lane's words of four steps: 32 bytes (16 with four rows)
+                uint4 *tile = (uint4 *)slot + ((int64_t)c * pc->s4 * 32 + lane) * (ROWS / 4);
 
                 for (int t0 = 0; t0 < steps; t0 += 4) {
                     uint4 nx[2], ob[2];
@@ -880,7 +882,7 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                             ww[1] >>= 2;
                             uint32_t d0 = diag_in, hu = up_h, f = up_f;
 #pragma unroll
-                            for (int r = 0; r < TB_ROWS; ++r) {
+                            for (int r = 0; r < ROWS; ++r) {
                                 const uint32_t sp = prmt(tA, tB, sel[r]);  // s - o, both pairs
                                 const uint32_t e = __viaddmax_s16x2(E[r], GE2, Hp[r]);
                                 f = __viaddmax_s16x2(f, GE2, hu);
@@ -921,7 +923,8 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                         (s == 0 ? wq.x : wq.z) = w0;
                         (s == 0 ? wq.y : wq.w) = w1;
                     }
-                    __stcg(tile + half, wq);
+                    if (ROWS == 8) __stcg(tile + half, wq);
+                    else __stcg((uint2 *)tile + half, make_uint2(wq.x, wq.z));
                     if (half == 0) {
 #pragma unroll
                         for (int x = 0; x < 2; ++x) {
@@ -932,7 +935,7 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                         }
                     }
                     }
-                    tile += 64;
+                    tile += 32 * (ROWS / 4);
                     if (T == 1 && has_out) {
                         __stcg(bnd + 2 * G * (t0 >> 2), ob[0]);
                         __stcg(bnd + 2 * G * (t0 >> 2) + 1, ob[1]);
@@ -1037,13 +1040,14 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                             lo_[x] = block_lo(tp.i[wi], tp.j[wi], tp.v[wi], tp.D[wi], tp.S[wi], tp.i0[wi] + c * rc,
                                               P.sc);
                         }
-                        const int jl = j_[x] - lo_[x], kk = (rel - c * rc) >> 3, t = jl + kk;
-                        row[x] = rel & 7;
+                        const int jl = j_[x] - lo_[x], kk = (rel - c * rc) / ROWS, t = jl + kk;
+                        row[x] = rel % ROWS;
                         if (jl < 0 || jl >= wcap) {  // left the band: inconsistent
                             ok_[x] = go_[x] = cell[x] = false;
                         } else {
                             const int64_t sector = ((int64_t)c * S4 + (t >> 2)) * 32 + g * T + kk;
-                            word[x] = __ldcg((const uint2 *)slot + 4 * sector + (t & 3));
+                            if (ROWS == 8) word[x] = __ldcg((const uint2 *)slot + 4 * sector + (t & 3));
+                            else word[x].x = __ldcg(slot + 4 * sector + (t & 3));
                         }
                     }
                 }
@@ -1125,7 +1129,8 @@ static const void *tb16_kernel(int lanes, bool fma)
     case 1: return fma ? (const void *)k_traceback16<1, true> : (const void *)k_traceback16<1, false>;
     case 2: return fma ? (const void *)k_traceback16<2, true> : (const void *)k_traceback16<2, false>;
     case 4: return fma ? (const void *)k_traceback16<4, true> : (const void *)k_traceback16<4, false>;
-    default: return fma ? (const void *)k_traceback16<8, true> : (const void *)k_traceback16<8, false>;
+    case 8: return fma ? (const void *)k_traceback16<8, true> : (const void *)k_traceback16<8, false>;
+    default: return fma ? (const void *)k_traceback16<16, true> : (const void *)k_traceback16<16, false>;
     }
 }
 
@@ -1143,6 +1148,7 @@ int launch_traceback_variant(int v, bool fma, const TracebackLaunch &L, int bloc
     if (!fn || !L.dp || blocks < 1) return SW_ERR_INTERNAL;
     TracebackLaunch V = L;
     V.variant = v;
+    V.n_variants = tb_launch_variants(v);
     void *args[] = {&V};
     if (cuda_failed(cudaLaunchKernel(fn, dim3(blocks), dim3(128), args, 0, st))) return SW_ERR_CUDA;
     count_launch();

@@ -388,13 +388,10 @@ int enqueue_small(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Sco
         if ((rc = launch_small_tbplan(S.tb_keys, n_pairs, S.info, S.tbinfo, S.splan, pp, S.tb_order, S.tplan,
                                       &S.info->status, st)))
             return rc;
-        // the wide and the narrow windows (8 lanes per two pairs: so few
-        // pairs never take fewer), then the int32 kernels
-        TracebackLaunch B = traceback_launch(ps, sc, out_score, out_end, *cig, S);
-        B.n_variants = 2;
+        // every 16-bit part (16 lanes per two pairs), then the int32 kernels
+        const TracebackLaunch B = traceback_launch(ps, sc, out_score, out_end, *cig, S);
         const bool fma = sc.mi >= sc.go;
         if ((rc = launch_traceback_variant(0, fma, B, blocks(x.tb_blocks[0]), st))) return rc;
-        B.n_variants = 1;
         for (int v : {TB_VAR_TILED, TB_VAR_GROUPED})
             if ((rc = launch_traceback_variant(v, fma, B, blocks(x.tb_blocks[v]), st))) return rc;
     }
@@ -448,7 +445,7 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
         const bool fma = sc.mi >= sc.go;
         const TracebackLaunch B = traceback_launch(ps, sc, out_score, out_end, *cig, S);
         // one after another: each launch has the whole slot budget
-        for (int v = 0; v < N_TB_VARIANTS; ++v)
+        for (int v = 0; v < N_TB_VARIANTS; v += tb_launch_variants(v))
             if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], st))) return rc;
     }
     if (timing && cuda_failed(cudaEventRecord(x.phase[3], st))) return SW_ERR_CUDA;
@@ -586,10 +583,10 @@ void plan_budgets(const ClassInfo &ci, const PlanParams &pp, bool cigar, int64_t
         const int64_t cand[3] = {mn, std::min<int64_t>(mn, kTbWide), std::min<int64_t>(mn, kTiledLaneWords / chunks)};
         for (int64_t w : cand) {
             if (w < 1) continue;
-            for (int lanes = w > kTbWide ? 8 : 1; lanes <= 8; lanes *= 2) {
+            for (int lanes = w > kTbWide ? 8 : 1; lanes <= 16; lanes *= 2) {
                 TbPartPlan t{};
                 const int64_t slot = tb_part_shape(mode, pp.allow16 != 0, 64, mm, chunks * w, (int32_t)w,
-                                                   w > kTbWide ? 0 : 1, pp.sc, lanes, t);
+                                                   tb_part_of((int32_t)w), pp.sc, lanes, t);
                 slot_v[t.variant] = std::max(slot_v[t.variant], (slot + 63) & ~(int64_t)63);
             }
         }

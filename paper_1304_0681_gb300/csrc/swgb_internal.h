@@ -142,8 +142,8 @@ struct TbParams {
 // Per-class facts of the traceback sort, read back to size the slabs.
 struct TbClassInfo {
     int32_t max_need[N_CLASS];  // largest slab (words) a pair of the class needs
-    int32_t n_big[N_CLASS];     // pairs with chunk windows wider than kTbWide
-    int32_t max_wcap[2][N_CLASS];  // widest chunk window: [0] the wide part, [1] the rest
+    int32_t n_part[2][N_CLASS];    // pairs of the first two parts (tb_part_of)
+    int32_t max_wcap[3][N_CLASS];  // widest chunk window of each part
 };
 
 // A persistent traceback launch: every part of traceback variant `variant`
@@ -152,13 +152,16 @@ struct TracebackLaunch {
     TbParams P;
     const int32_t *order;    // the whole traceback order (parts index into it)
     uint32_t *slab;          // base of the per-warp scratch slots
-    int32_t *work_counter;   // base of the per-part counters (2 per class)
+    int32_t *work_counter;   // base of the per-part counters
     int32_t *status;
     int32_t one = 1;         // a multiplier the compiler cannot fold
     const DevTbPlan *dp = nullptr;
     int32_t variant = 0;
     int32_t n_variants = 1;  // variants from `variant` on that this launch serves (of one kernel, equal slots)
 };
+// A launch serves the variants of one kernel: those of 16 lanes, of 8 lanes,
+// then one each.
+__host__ __device__ inline int tb_launch_variants(int v) { return v == 0 || v == 2 ? 2 : 1; }
 
 // Row counts compiled for the score kernels.
 constexpr int N_SCORE_ROWS = 6;
@@ -185,21 +188,30 @@ __host__ __device__ inline int score_rows_at(int i)
 // classes (or traceback parts) its variant was given and exits at once when
 // it has none.
 constexpr int N_SCORE_VARIANTS = N_SCORE_ROWS * N_VMODES;  // variant = rows index * N_VMODES + mode
-constexpr int N_TB16_VARIANTS = 5;                        // 16-bit traceback: wide windows, T = 8; the rest, T = 8, 4, 2, 1
-constexpr int TB_VAR_TILED = 5;                           // int32 traceback, one lane per pair, warp tiles
-constexpr int TB_VAR_GROUPED = 6;                         // int32 traceback, T lanes per pair
-constexpr int N_TB_VARIANTS = 7;
-__host__ __device__ inline int tb16_variant_lanes(int v) { return v == 0 ? 8 : 16 >> v; }
-constexpr int N_TB_PARTS = 2 * N_CLASS;                   // per class: the wide part, then the rest
-// Chunk windows wider than this form a part (and launches) of their own: a
-// warp's scratch slot is sized for the widest window of its launch, and a
-// few spliced pairs with windows of thousands of columns would otherwise
-// leave room for a fraction of the warps.  They take 8 lanes per two pairs:
-// over windows this wide the wavefront's extra steps cost little, a warp
-// waits for the widest of 8 pairs rather than of 64, and a task (many blocks
-// one after another) ends 7 times sooner -- the wide pairs of the 2M uneven
-// batch took 33 ms with one or two lanes, most of it in the last few tasks.
-constexpr int kTbWide = 256;
+constexpr int N_TB16_VARIANTS = 7;                        // 16-bit traceback: T = 16 (wide windows, the rest), T = 8 (the same), T = 4, 2, 1
+constexpr int TB_VAR_TILED = 7;                           // int32 traceback, one lane per pair, warp tiles
+constexpr int TB_VAR_GROUPED = 8;                         // int32 traceback, T lanes per pair
+constexpr int N_TB_VARIANTS = 9;
+__host__ __device__ inline int tb16_variant_lanes(int v) { return v < 2 ? 16 : v < 4 ? 8 : 64 >> v; }
+// Rows per lane of the 16-bit kernel: with 16 lanes per two pairs, taken where
+// there are too few pairs to fill the GPU, four -- a lone warp's step then
+// takes 100 instructions instead of 170 while a chunk stays 64 rows.
+__host__ __device__ constexpr int tb16_rows(int T) { return T == 16 ? 4 : 8; }
+// Parts of a class by chunk window width: over kTbWide columns, over kTbMid,
+// the rest.  A warp's scratch slot is sized for the widest window of its
+// launch, and a few spliced pairs with windows of thousands of columns would
+// otherwise leave room for a fraction of the warps: the wide part takes 8 or
+// 16 lanes per two pairs, apart from the large narrow parts.  Over windows
+// this wide the wavefront's extra steps cost little, a warp waits for the widest
+// of 8 pairs rather than of 64, and a task (many blocks one after another)
+// ends 7 times sooner -- the wide pairs of the 2M uneven batch took 33 ms with
+// one or two lanes, most of it in the last few tasks.  The middle part
+// (decoys and short introns, several times the narrow part's steps) gets its
+// own number of lanes.
+constexpr int kTbWide = 256, kTbMid = 64;
+constexpr int kTbParts = 3;
+__host__ __device__ inline int tb_part_of(int32_t wc) { return wc > kTbWide ? 0 : wc > kTbMid ? 1 : 2; }
+constexpr int N_TB_PARTS = kTbParts * N_CLASS;
 constexpr int kMaxPlanOverrides = 16;
 constexpr int kPlanThreads = 384;                         // >= N_CLASS
 
@@ -362,8 +374,7 @@ __host__ __device__ inline void score_plan_of(int mode, int32_t m_max, int64_t h
     }
 }
 
-// Traceback launch shape of one part of a class (part 0: chunk windows wider
-// than kTbWide, part 1: the rest).  m_max: the class's longest read;
+// Traceback launch shape of one part of a class.  m_max: the class's longest read;
 // max_need: the largest one-lane slab of the class (int32 kernels); wcap_in:
 // the part's widest chunk window; block_rows: rows between the class's
 // checkpoints (0 or m_max and more: the whole read is one block).  The 16-bit kernel
@@ -384,18 +395,19 @@ __host__ __device__ inline int64_t tb_part_shape(int mode, bool allow16, int32_t
     if (allow16 && mode != MODE_I32) {
         const int T = lanes16;
         const int64_t rows = block_rows && block_rows < m_max ? block_rows : m_max;
-        const int64_t chunks_t = (rows + 8 * T - 1) / (8 * T);
+        const int rc = T * tb16_rows(T);
+        const int64_t chunks_t = (rows + rc - 1) / rc;
         // a block entered inside an insertion run does not pay for opening
         // it, so its band may be a few columns wider than the whole pair's;
         // windows start at multiples of four columns
-        wcap = (wcap + (sc.ge - sc.go) / (sc.ma - sc.ge) + 2 + 8 * (T - 1) + 3 + 3) / 4 * 4;
+        wcap = (wcap + (sc.ge - sc.go) / (sc.ma - sc.ge) + 2 + (rc - 8) + 3 + 3) / 4 * 4;
         const int64_t s4 = (wcap + T - 1 + 3) / 4;
         t.lanes = T;
         t.wcap = wcap;
         t.block_rows = block_rows;
-        t.slab_words = chunks_t * s4 * 8;                // per lane
+        t.slab_words = chunks_t * s4 * tb16_rows(T);     // per lane
         t.bnd_ints = (int64_t)(32 / T) * 2 * (wcap + 8);  // per warp: one row
-        t.variant = part == 0 ? 0 : T == 8 ? 1 : T == 4 ? 2 : T == 2 ? 3 : 4;
+        t.variant = T == 16 ? (part ? 1 : 0) : T == 8 ? (part ? 3 : 2) : T == 4 ? 4 : T == 2 ? 5 : 6;
         return ((32 * t.slab_words + 63) & ~(int64_t)63) + t.bnd_ints;
     }
     int T = 1;
@@ -436,7 +448,7 @@ int launch_plan_tb(const ClassInfo *info, const TbClassInfo *ti, const DevScoreP
 // full occupancy; its grid (blocks) comes from score_variant_blocks.
 int launch_score_variant(int v, const ScoreLaunch &L, int blocks, cudaStream_t st);
 int score_variant_blocks(int v, int sm_count, int *blocks);
-// (n_variants > 1: as many variants from v on that share a kernel)
+// (every variant from v on of its kernel)
 int launch_traceback_variant(int v, bool fma, const TracebackLaunch &L, int blocks, cudaStream_t st);
 // The one score launch of a small batch: every class of every variant.
 int launch_score_any(const ScoreLaunch &L, int blocks, cudaStream_t st);
