@@ -249,7 +249,7 @@ int sw_mlp_forward(const float *model, const uint16_t *features, int64_t n, floa
  * on the CUDA cores instead.  A timed-out tensor-core wait is reported as
  * SW_ERR_DEVICE_TIMEOUT by sw_sync_status.  sw_set_mlp_grad_kernel is
  * process-wide; SW_ERR_INVALID_ARG for other values.  The library keeps the
- * partial gradients in scratch of this stream (33,153 floats per CTA). */
+ * partial gradients in scratch of this stream (33,156 floats per CTA). */
 #define SW_GRAD_AUTO 0
 #define SW_GRAD_FP32 1
 int sw_set_mlp_grad_kernel(int32_t kind);

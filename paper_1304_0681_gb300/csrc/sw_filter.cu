@@ -474,18 +474,28 @@ __global__ void __launch_bounds__(GR_THREADS, 1)
     if (j == 0) atomicAdd(&G[MD_B3], gb3);
 }
 
-// One Adam step (Kingma & Ba) on the fp32 parameters from the gradient in G.
+// One Adam step (Kingma & Ba) on the fp32 parameters from the gradient in G;
+// the bf16 serving copies (k_mlp_refresh) are written by the same thread.
 __global__ void k_mlp_adam(float *model, float lr, int32_t step)
 {
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
+    __nv_bfloat16 *w1t = reinterpret_cast<__nv_bfloat16 *>(model + MD_W1T);
+    __nv_bfloat16 *w2t = reinterpret_cast<__nv_bfloat16 *>(model + MD_W2T);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < MD_NP; i += (int64_t)gridDim.x * blockDim.x) {
         const float g = model[MD_G + i];
         const float m = b1 * model[MD_M + i] + (1.f - b1) * g;
         const float v = b2 * model[MD_V + i] + (1.f - b2) * g * g;
         model[MD_M + i] = m;
         model[MD_V + i] = v;
-        model[i] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+        const float p = model[i] - lr * (m / c1) / (sqrtf(v / c2) + eps);
+        model[i] = p;
+        if (i < MD_B1) {
+            w1t[(i % 256) * 64 + i / 256] = __float2bfloat16_rn(p);
+        } else if (i >= MD_W2 && i < MD_B2) {
+            const int64_t w = i - MD_W2;
+            w2t[(w % 64) * 256 + w / 64] = __float2bfloat16_rn(p);
+        }
     }
 }
 
@@ -655,8 +665,7 @@ int launch_mlp_grad(float *model, const uint16_t *feat, const float *target, con
 int launch_mlp_adam(float *model, float lr, int32_t step, cudaStream_t st)
 {
     k_mlp_adam<<<grid_for(MD_NP, 256, 152 * 2), 256, 0, st>>>(model, lr, step);
-    k_mlp_refresh<<<64, 256, 0, st>>>(model);
-    count_launch(2);
+    count_launch();
     return launch_status();
 }
 
@@ -772,7 +781,7 @@ int sw_mlp_grad(float *model, const uint16_t *features, const float *target, con
         int32_t *status = nullptr;
         if ((rc = aux_status_word(st, &status))) return rc;
         float *partial = nullptr;
-        if ((rc = grad_scratch(st, sizeof(float) * (size_t)MD_NP * mlp_grad_tc_parts(n, sms), &partial))) return rc;
+        if ((rc = grad_scratch(st, sizeof(float) * (size_t)GRAD_PART * mlp_grad_tc_parts(n, sms), &partial))) return rc;
         return launch_mlp_grad_tc(model, features, target, idx, n, sms, partial, status, st);
     }
     return launch_mlp_grad(model, features, target, idx, n, sms, st);

@@ -434,6 +434,31 @@ __device__ __forceinline__ float warp_sum(float v)
     return v;
 }
 
+// Column sums of a warp's rows, N = 16 or 32 columns per lane, as one tree:
+// every exchange halves the columns a lane keeps (N shuffles or one fewer,
+// where N butterflies take 5 N; the shuffles were a tenth of a tile's time).
+// Returns the sum of column column_of<N>(lane); with N = 16 both lanes of a
+// pair hold it.
+template <int N>
+__device__ __forceinline__ int column_of(int lane) { return (int)((__brev((unsigned)lane) >> 27) & (N - 1)); }
+
+template <int N>
+__device__ __forceinline__ float column_sums(float (&v)[N], int lane)
+{
+    int d = 16;
+#pragma unroll
+    for (int keep = N / 2; keep >= 1; keep >>= 1, d >>= 1) {
+        const bool up = (lane & d) != 0;
+#pragma unroll
+        for (int j = 0; j < keep; ++j) {
+            const float give = up ? v[2 * j] : v[2 * j + 1];
+            v[j] = (up ? v[2 * j + 1] : v[2 * j]) + __shfl_xor_sync(0xffffffffu, give, d);
+        }
+    }
+    if (N == 16) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+}
+
 __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict__ model,
                                                         const __nv_bfloat16 *__restrict__ feat,
                                                         const float *__restrict__ target,
@@ -504,26 +529,44 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
         __syncthreads();
         fence_after_sync();
     };
-    // copies a [rows][cols] bf16 matrix from global memory into K-major layout
-    auto load_kmajor = [&](int region, const uint4 *g, int rows, int cols) {
+    // a 32 KB bf16 weight matrix of `cols` columns: fetch puts a thread's
+    // eight 16-byte pieces in registers (all loads in flight, and for the
+    // later layers behind the MMAs before them), place lays them out K-major
+    auto fetch = [&](const float *g, uint4 (&v)[8]) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = __ldg(reinterpret_cast<const uint4 *>(g) + tid + 256 * q);
+    };
+    auto place = [&](const uint4 (&v)[8], int cols) {
         const int per_row = cols / 8;
-        for (int c = tid; c < rows * per_row; c += blockDim.x) {
-            const int r = c / per_row, k = (c % per_row) * 8;
-            *reinterpret_cast<uint4 *>(smem + region + kmajor_off(r, k, cols)) = g[c];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int c = tid + 256 * q;
+            *reinterpret_cast<uint4 *>(smem + GB_R3 + kmajor_off(c / per_row, (c % per_row) * 8, cols)) = v[q];
         }
     };
     bool first = true;
     for (int64_t tile = blockIdx.x; tile < tiles && ok; tile += gridDim.x) {
         const int64_t row0 = tile * TC_ROWS;
         // 1. X (K-major along features), X^T (along samples), targets, W1^T
-        for (int c = tid; c < TC_ROWS * 8; c += blockDim.x) {
-            const int r = c >> 3, k = (c & 7) * 8;
-            const int64_t s = row0 + r;
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (s < n) {
-                const int64_t row = idx ? idx[s] : s;
-                v = reinterpret_cast<const uint4 *>(feat)[row * 8 + (c & 7)];
+        uint4 wq[8], xq[4];
+        fetch(model + MD_W1T, wq);
+        {
+            int64_t row[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int64_t s = row0 + ((tid + 256 * q) >> 3);
+                row[q] = s < n ? (idx ? (int64_t)__ldg(idx + s) : s) : -1;
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                xq[q] = row[q] >= 0 ? __ldg(reinterpret_cast<const uint4 *>(feat) + row[q] * 8 + (tid & 7))
+                                    : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int q4 = 0; q4 < 4; ++q4) {
+            const int c = tid + 256 * q4;
+            const int r = c >> 3, k = (c & 7) * 8;
+            const uint4 v = xq[q4];
             *reinterpret_cast<uint4 *>(smem + GB_R5 + kmajor_off(r, k, 64)) = v;
             const __nv_bfloat16 *e = reinterpret_cast<const __nv_bfloat16 *>(&v);
 #pragma unroll
@@ -534,7 +577,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
             const int64_t s = row0 + r;
             ts[r] = s < n ? target[idx ? idx[s] : s] : 0.f;
         }
-        load_kmajor(GB_R3, reinterpret_cast<const uint4 *>(model + MD_W1T), 256, 64);
+        place(wq, 64);
+        fetch(model + MD_W2T, wq);
         publish();
         // 2. Z1 = X . W1
         if (tid == 0)
@@ -544,7 +588,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
                          smem_desc(s_base + GB_R3 + 256 * ks, 128, 1024), idesc_bf16(128, 256), ks > 0);
         if (!(ok = commit_wait())) break;
         // 3. W2^T for layer 2; A1 = bf16(relu(Z1 + b1)) as A1 and A1^T
-        load_kmajor(GB_R3, reinterpret_cast<const uint4 *>(model + MD_W2T), 64, 256);
+        place(wq, 256);
         {
             const int r = 32 * quarter + lane;
             for (int c0 = 128 * half; c0 < 128 * half + 128; c0 += 16) {
@@ -566,6 +610,14 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
                     make_uint4(pk[4], pk[5], pk[6], pk[7]);
             }
         }
+        // (the fp32 W2 of step 5, on its way during step 4)
+        float4 w2q[16];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const float4 *src = reinterpret_cast<const float4 *>(model + MD_W2) + 2 * (tid + 256 * q);
+            w2q[2 * q] = __ldg(src);
+            w2q[2 * q + 1] = __ldg(src + 1);
+        }
         publish();
         // 4. Z2 = A1 . W2
         if (tid == 0)
@@ -576,10 +628,10 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
         if (!(ok = commit_wait())) break;
         // 5. W2 for dA1 (bf16 of the fp32 parameters, as the serving copies
         // round them); y, dy, dZ2 (as dZ2 and dZ2^T) and the small gradients
-        for (int c = tid; c < 256 * 8; c += blockDim.x) {
-            const int r = c >> 3, k = (c & 7) * 8;
-            const float4 *src = reinterpret_cast<const float4 *>(model + MD_W2 + r * 64 + k);
-            const float4 lo = src[0], hi = src[1];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            const int c = tid + 256 * q, r = c >> 3, k = (c & 7) * 8;
+            const float4 lo = w2q[2 * q], hi = w2q[2 * q + 1];
             const __nv_bfloat162 p0 = __floats2bfloat162_rn(lo.x, lo.y), p1 = __floats2bfloat162_rn(lo.z, lo.w);
             const __nv_bfloat162 p2 = __floats2bfloat162_rn(hi.x, hi.y), p3 = __floats2bfloat162_rn(hi.z, hi.w);
             *reinterpret_cast<uint4 *>(smem + GB_R3 + kmajor_off(r, k, 64)) =
@@ -611,12 +663,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
                 const int c = 32 * half + j;
                 dz[j] = z[j] > 0.f ? dy * w3[c] : 0.f;
                 st_bf16(smem, GB_R7 + kmajor_off(c, r, 128), dz[j]);
-                const float s2 = warp_sum(dz[j]);
-                const float s3 = warp_sum(fmaxf(z[j], 0.f) * dy);
-                if (lane == 0) {
-                    gb2[quarter * 64 + c] += s2;
-                    gw3[quarter * 64 + c] += s3;
-                }
+                z[j] = fmaxf(z[j], 0.f) * dy;
             }
 #pragma unroll
             for (int j = 0; j < 32; j += 8) {
@@ -628,6 +675,12 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
                 }
                 *reinterpret_cast<uint4 *>(smem + GB_R5 + kmajor_off(r, 32 * half + j, 64)) =
                     make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            }
+            {
+                const float s2 = column_sums<32>(dz, lane), s3 = column_sums<32>(z, lane);
+                const int c = quarter * 64 + 32 * half + column_of<32>(lane);
+                gb2[c] += s2;
+                gw3[c] += s3;
             }
             if (half == 0) {
                 const float s = warp_sum(dy);
@@ -657,6 +710,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
                 uint32_t v[16];
                 tmem_ld16(accA + lane_off + (uint32_t)c0, v);
                 tmem_wait_ld();
+                float dz1[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
                     const int c = c0 + j;
@@ -664,9 +718,10 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
                         *reinterpret_cast<const __nv_bfloat16 *>(smem + GB_R2 + kmajor_off(c, r, 128)));
                     const float d = a > 0.f ? __uint_as_float(v[j]) : 0.f;
                     st_bf16(smem, GB_R1 + kmajor_off(c, r, 128), d);
-                    const float s1 = warp_sum(d);
-                    if (lane == 0) gb1[quarter * 256 + c] += s1;
+                    dz1[j] = d;
                 }
+                const float s1 = column_sums<16>(dz1, lane);
+                if (!(lane & 1)) gb1[quarter * 256 + c0 + column_of<16>(lane)] += s1;
             }
         }
         publish();
@@ -684,14 +739,16 @@ __global__ void __launch_bounds__(256, 1) k_mlp_grad_tc(const float *__restrict_
     }
     // the CTA's partial gradient: gW1, gW2 from tensor memory, biases
     if (ok && !first) {
-        float *out = partial + (int64_t)blockIdx.x * MD_NP;
+        float *out = partial + (int64_t)blockIdx.x * GRAD_PART;
         const int j = 128 * half + 32 * quarter + lane;  // hidden unit of this lane
         for (int c0 = 0; c0 < 64; c0 += 16) {
             uint32_t v[16];
             tmem_ld16(accB + 64u * (uint32_t)half + lane_off + (uint32_t)c0, v);
             tmem_wait_ld();
 #pragma unroll
-            for (int q = 0; q < 16; ++q) out[MD_W2 + j * 64 + c0 + q] = __uint_as_float(v[q]);
+            for (int q = 0; q < 16; q += 4)
+                *reinterpret_cast<uint4 *>(out + MD_W2 + j * 64 + c0 + q) =
+                    make_uint4(v[q], v[q + 1], v[q + 2], v[q + 3]);
             tmem_ld16(accC + 64u * (uint32_t)half + lane_off + (uint32_t)c0, v);
             tmem_wait_ld();
 #pragma unroll
@@ -725,7 +782,8 @@ __global__ void k_mlp_grad_reduce(const float *__restrict__ partial, int n_part,
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < MD_NP; i += (int64_t)gridDim.x * blockDim.x) {
         float s = 0.f;
-        for (int p = 0; p < n_part; ++p) s += partial[(int64_t)p * MD_NP + i];
+#pragma unroll 8
+        for (int p = 0; p < n_part; ++p) s += partial[(int64_t)p * GRAD_PART + i];
         G[i] = s * inv_n;
     }
 }

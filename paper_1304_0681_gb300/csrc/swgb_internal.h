@@ -515,7 +515,7 @@ int launch_dense_cigar(const uint32_t *ops, const int64_t *off, const int32_t *n
 int launch_mlp_forward_tc(const float *model, const uint16_t *feat, int64_t n, float *out, int sm_count,
                           int32_t *status, cudaStream_t st);
 // The gradient on the tensor cores: one partial per CTA (partial: that many
-// x MD_NP floats), then their sum in CTA order into the model's gradient.
+// x GRAD_PART floats), then their sum in CTA order into the model's gradient.
 int mlp_grad_tc_parts(int64_t n, int sm_count);
 int launch_mlp_grad_tc(float *model, const uint16_t *feat, const float *target, const int32_t *idx, int64_t n,
                        int sm_count, float *partial, int32_t *status, cudaStream_t st);
@@ -536,6 +536,7 @@ constexpr int64_t MD_M = MD_NP, MD_V = 2 * MD_NP, MD_G = 3 * MD_NP, MD_STEP = 4 
 constexpr int64_t MD_W1T = 132616;          // bf16 [256][64], 16-byte aligned
 constexpr int64_t MD_W2T = MD_W1T + 8192;   // bf16 [64][256]
 constexpr int64_t MD_TOTAL = MD_W2T + 8192;
+constexpr int64_t GRAD_PART = (MD_NP + 3) / 4 * 4;  // one CTA's partial gradient, 16-byte aligned
 
 void count_launch(int n = 1);
 
