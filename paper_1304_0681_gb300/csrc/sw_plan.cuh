@@ -182,7 +182,12 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
     }
 }
 
-// Whole block; the first warp finishes.
+// Whole block.  The 16-bit launches run at once (a few wide pairs' tasks are
+// long and leave the SMs half empty), each with its part of the scratch: a
+// slot for every warp that gets a task while they fit, else a slot each and
+// the rest in proportion.  Where not even one slot each fits, every 16-bit
+// part takes the 16-lane launch, whose slots are the smallest.  The int32
+// launches follow, each with all of the scratch.
 __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo *ti, const DevScorePlan *sp,
                                         const PlanParams &pp, DevTbPlan *out, int32_t *status)
 {
@@ -191,6 +196,7 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
     __shared__ int8_t s_pv[N_TB_PARTS];  // each part's variant (-1: none)
     __shared__ int16_t s_tblist[N_CLASS];
     __shared__ int32_t s_n16[kTbParts];  // pairs of the 16-bit classes by part
+    __shared__ int32_t s_retry;
     if (threadIdx.x < kTbParts) s_n16[threadIdx.x] = 0;
     __syncthreads();
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
@@ -202,6 +208,7 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
         }
     }
     __syncthreads();
+    for (bool one_launch = pp.small != 0;; one_launch = true) {
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = s_tbcnt[c];
         if (!cnt) continue;
@@ -231,7 +238,7 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
                 const int64_t wave = (int64_t)pp.tb_warps[0] * 64;
                 const int64_t all = s_n16[2], same = part < 2 ? s_n16[part] : all;
                 const int64_t enough = part < 2 ? wave : wave / 4;
-                int lanes = pp.small || 16 * all < wave ? 16 : part == 0 ? 8 : 1;  // (wide windows: see kTbWide)
+                int lanes = one_launch || 16 * all < wave ? 16 : part == 0 ? 8 : 1;  // (wide windows: see kTbWide)
                 while (lanes < 16 &&
                        (same * lanes < enough || (info->max_m[c] > 512 && (int64_t)cnt * lanes < wave / 4)))
                     lanes *= 2;
@@ -246,47 +253,90 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
     }
     __syncthreads();
     // the first warp finishes: each variant's part list (longest reads
-    // first, wide part first), its slot size, and the split
-    if (threadIdx.x >= 32) return;
-    const int lane = threadIdx.x;
-    const int n_list = list_classes(s_tbcnt, s_tblist);
-    const int64_t ck_words = 4 * sp->ck_units;
-    const int64_t total = pp.tb_bytes / 4 - ck_words;
-    int32_t n = 0;
-    int64_t words = 0, pairs = 0;
-    for (int q = 0; q < n_list; ++q)
-        for (int part = 0; part < kTbParts; ++part) {
-            const int x = kTbParts * s_tblist[q] + part;
-            if (s_pv[x] == lane) {
-                out->var_part[lane][n++] = (int16_t)x;
-                words = max(words, s_slot[x]);
-                pairs += s_part[x];
+    // first, wide part first), its slots, and the split
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        const int n_list = list_classes(s_tbcnt, s_tblist);
+        const int64_t ck_words = 4 * sp->ck_units;
+        const int64_t total = pp.tb_bytes / 4 - ck_words;
+        const int32_t per_task = lane < N_TB16_VARIANTS ? 64 / tb16_variant_lanes(lane) : 1;
+        int32_t n = 0;
+        int64_t words = 0, pairs = 0, tasks = 0;
+        for (int q = 0; q < n_list; ++q)
+            for (int part = 0; part < kTbParts; ++part) {
+                const int x = kTbParts * s_tblist[q] + part;
+                if (s_pv[x] == lane) {
+                    out->var_part[lane][n++] = (int16_t)x;
+                    words = max(words, s_slot[x]);
+                    pairs += s_part[x];
+                    tasks += (s_part[x] + per_task - 1) / per_task;
+                }
+            }
+        // the variants of one launch share its slots
+        {
+            const int64_t w = __shfl_xor_sync(0xffffffffu, words, 1), t = __shfl_xor_sync(0xffffffffu, tasks, 1);
+            if (lane < 4) {
+                words = max(words, w);
+                tasks += t;
             }
         }
-    // the variants of one launch share the size of a slot
-    {
-        const int64_t o = __shfl_xor_sync(0xffffffffu, words, 1);
-        if (lane < 4) words = max(words, o);
+        words = (words + 63) & ~(int64_t)63;  // 256-byte alignment
+        const int64_t warps = lane < N_TB_VARIANTS ? min((int64_t)pp.tb_warps[lane], tasks) : 0;
+        const bool leads = lane < N_TB16_VARIANTS && (lane >= 4 || !(lane & 1)) && warps > 0;
+        const int64_t one = leads ? words : 0, more = leads ? (warps - 1) * words : 0;
+        int64_t ones = one, mores = more;
+        for (int d = 16; d; d >>= 1) {
+            ones += __shfl_xor_sync(0xffffffffu, ones, d);
+            mores += __shfl_xor_sync(0xffffffffu, mores, d);
+        }
+        int64_t w = leads ? 1 : 0;
+        if (leads) {
+            if (ones + mores <= total) w = warps;
+            else if (ones < total) w += (int64_t)((double)(total - ones) * ((double)more / (double)mores)) / words;
+        }
+        const int64_t area = w * words;
+        int64_t at = area;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int64_t y = __shfl_up_sync(0xffffffffu, at, d);
+            if (lane >= d) at += y;
+        }
+        at -= area;
+        {
+            const int64_t w0 = __shfl_sync(0xffffffffu, w, lane & ~1), at0 = __shfl_sync(0xffffffffu, at, lane & ~1);
+            if (lane < 4) {
+                w = w0;
+                at = at0;
+            }
+        }
+        if (lane >= N_TB16_VARIANTS && lane < N_TB_VARIANTS) {
+            // int32: as many warps as fit all of the scratch
+            w = n ? min((int64_t)pp.tb_warps[lane], total / max(words, (int64_t)1)) : 0;
+            at = 0;
+            if (n && w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's slot does not fit the scratch
+        }
+        if (lane == 0) {
+            s_retry = ones > total && !one_launch;
+            if (ones > total && one_launch) atomicOr(status, ST_UNSUPPORTED);
+        }
+        int64_t split16 = lane < N_TB16_VARIANTS ? pairs : 0, split32 = lane >= N_TB16_VARIANTS ? pairs : 0;
+        for (int d = 16; d; d >>= 1) {
+            split16 += __shfl_xor_sync(0xffffffffu, split16, d);
+            split32 += __shfl_xor_sync(0xffffffffu, split32, d);
+        }
+        if (lane < N_TB_VARIANTS) {
+            out->var_n[lane] = n;
+            out->var_slot_words[lane] = words;
+            out->var_slot_offset[lane] = ck_words + at;
+            out->var_warps[lane] = (int32_t)w;
+        }
+        if (lane == 0) {
+            out->split[0] = split16;
+            out->split[1] = split32;
+        }
     }
-    words = (words + 63) & ~(int64_t)63;  // 256-byte alignment
-    int64_t split16 = lane < N_TB16_VARIANTS ? pairs : 0, split32 = lane >= N_TB16_VARIANTS ? pairs : 0;
-    for (int d = 16; d; d >>= 1) {
-        split16 += __shfl_xor_sync(0xffffffffu, split16, d);
-        split32 += __shfl_xor_sync(0xffffffffu, split32, d);
-    }
-    if (lane < N_TB_VARIANTS) {
-        // a slot per warp, as many warps as fit (the launches run one after
-        // another, each with everything the checkpoints leave)
-        const int64_t w = n ? min((int64_t)pp.tb_warps[lane], total / max(words, (int64_t)1)) : 0;
-        if (n && w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's slot does not fit the scratch
-        out->var_n[lane] = n;
-        out->var_slot_words[lane] = words;
-        out->var_slot_offset[lane] = ck_words;
-        out->var_warps[lane] = (int32_t)w;
-    }
-    if (lane == 0) {
-        out->split[0] = split16;
-        out->split[1] = split32;
+    __syncthreads();
+    if (!s_retry) break;
+    __syncthreads();
     }
 }
 

@@ -40,7 +40,7 @@ constexpr int64_t kHostChunkMin = 65536;       // ... of at least this many pair
 // and the per-warp slots of the traceback.  A warp's slot is sized on the
 // device for its launch's largest part; launches use as many warps as fit.
 constexpr int64_t kScoreBndMin = (int64_t)32 << 20, kScoreBndMax = (int64_t)1 << 30, kScoreBndPerPair = 1024;
-constexpr int64_t kTbMin = (int64_t)256 << 20, kTbPerPair = (int64_t)96 << 10;
+constexpr int64_t kTbMin = (int64_t)256 << 20, kTbPerPair = (int64_t)160 << 10;
 constexpr int64_t kTbCapMax = (int64_t)16 << 30, kTbCapMin = (int64_t)1 << 30;
 constexpr double kTbFreeShare = 0.3;
 
@@ -444,8 +444,15 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
         if ((rc = launch_plan_tb(S.info, S.tbinfo, S.splan, pp, S.tplan, &S.info->status, st))) return rc;
         const bool fma = sc.mi >= sc.go;
         const TracebackLaunch B = traceback_launch(ps, sc, out_score, out_end, *cig, S);
-        // one after another: each launch has the whole slot budget
-        for (int v = 0; v < N_TB_VARIANTS; v += tb_launch_variants(v))
+        // the 16-bit launches at once, each in its part of the scratch, those
+        // with the longest tasks first; then the int32 launches, each with
+        // all of it
+        if ((rc = fork_streams(x, st, kAuxStreams))) return rc;
+        int k = 0;
+        for (int v = 0; v < N_TB16_VARIANTS; v += tb_launch_variants(v), ++k)
+            if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], x.aux[k % kAuxStreams]))) return rc;
+        if ((rc = join_streams(x, st, kAuxStreams))) return rc;
+        for (int v = N_TB16_VARIANTS; v < N_TB_VARIANTS; ++v)
             if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], st))) return rc;
     }
     if (timing && cuda_failed(cudaEventRecord(x.phase[3], st))) return SW_ERR_CUDA;
@@ -592,9 +599,13 @@ void plan_budgets(const ClassInfo &ci, const PlanParams &pp, bool cigar, int64_t
         }
     }
     const int64_t cap = kTbCapMax / 4;  // words
-    for (int v = 0; v < N_TB_VARIANTS; ++v)
-        if (slot_v[v])
-            tb_bytes = std::max(tb_bytes, 4 * std::max(std::min(pp.tb_warps[v] * slot_v[v], cap), 4 * slot_v[v]));
+    int64_t all16 = 0;  // the 16-bit launches run at once
+    for (int v = 0; v < N_TB_VARIANTS; ++v) {
+        const int64_t words = std::max(std::min(pp.tb_warps[v] * slot_v[v], cap), 4 * slot_v[v]);
+        if (v < N_TB16_VARIANTS) all16 += words;
+        else tb_bytes = std::max(tb_bytes, 4 * words);
+    }
+    tb_bytes = std::max(tb_bytes, 4 * std::min(all16, 2 * cap));
     // the planner lets checkpoints take three quarters of the scratch
     tb_bytes = std::max(tb_bytes + std::min(ck, kTbCapMax), (std::min(ck, kTbCapMax) + 2) / 3 * 4);
 }
