@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                 for (int x = 0; x < 2; ++x) {
                     const int wi = 2 * g + x;
                     ww[x] = 0u;
-                    wn[x] = rem[x] > 0 ? load_bases(P.ps.wins, tp.ws[wi] + lo[x], min(16, rem[x])) : 0u;
+                    wn[x] = k == 0 && rem[x] > 0 ? load_bases(P.ps.wins, tp.ws[wi] + lo[x], min(16, rem[x])) : 0u;
                     codes[x] = 0x44444444u;  // 4 bits per row, 4 = no base
                     const int row = tp.i0[wi] + c * rc + k * ROWS;
                     const int cnt = rem[x] > 0 ? min(ROWS, tp.i[wi] - row + 1) : 0;
@@ -838,7 +838,7 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                     Hp[r] = 0u;
                 }
                 uint32_t diag_in = prmt(dg0, dg1, 0x5410u);
-                uint32_t out_h = 0u, out_f = 0u;
+                uint32_t out_h = 0u, out_f = 0u, bases = 0u;
                 // a lane's words of four steps: 32 bytes (16 with four rows)
                 uint4 *tile = (uint4 *)slot + ((int64_t)c * pc->s4 * 32 + lane) * (ROWS / 4);
 
@@ -864,22 +864,28 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                         }
                         const int jl = t - k;  // this lane's window offset
                         uint32_t w0 = 0u, w1 = 0u;
-                        if (T == 1 || jl >= 0) {
-                            if ((T > 1 || s == 0) && (jl & 15) == 0) {
-                                // the next 16 columns' bases, requested 16 columns before
+                        // the column's bases (4: past the window) of both
+                        // pairs: the first lane streams them, 16 columns
+                        // requested 16 columns ahead, and each lane takes
+                        // the lane before's of the last step (with a stream
+                        // per lane some lane refilled its own at every step)
+                        if (s == 0 && (t & 15) == 0 && k == 0) {
 #pragma unroll
-                                for (int x = 0; x < 2; ++x) {
-                                    ww[x] = wn[x];
-                                    const int left = rem[x] - jl - 16;
-                                    wn[x] = left > 0 ? load_bases(P.ps.wins, tp.ws[2 * g + x] + lo[x] + jl + 16,
-                                                                  min(16, left))
-                                                     : 0u;
-                                }
+                            for (int x = 0; x < 2; ++x) {
+                                ww[x] = wn[x];
+                                const int left = rem[x] - t - 16;
+                                wn[x] = left > 0 ? load_bases(P.ps.wins, tp.ws[2 * g + x] + lo[x] + t + 16,
+                                                              min(16, left))
+                                                 : 0u;
                             }
-                            const uint32_t tA = s_tab[jl < rem[0] ? ww[0] & 3u : 4u];
-                            const uint32_t tB = s_tab[jl < rem[1] ? ww[1] & 3u : 4u];
-                            ww[0] >>= 2;
-                            ww[1] >>= 2;
+                        }
+                        const uint32_t bprev = T > 1 ? __shfl_up_sync(FULLMASK, bases, 1) : 0u;
+                        bases = (t < rem[0] ? ww[0] & 3u : 4u) | ((t < rem[1] ? ww[1] & 3u : 4u) << 3);
+                        ww[0] >>= 2;
+                        ww[1] >>= 2;
+                        if (T > 1 && k > 0) bases = bprev;
+                        if (T == 1 || jl >= 0) {
+                            const uint32_t tA = s_tab[bases & 7u], tB = s_tab[bases >> 3];
                             uint32_t d0 = diag_in, hu = up_h, f = up_f;
 #pragma unroll
                             for (int r = 0; r < ROWS; ++r) {
