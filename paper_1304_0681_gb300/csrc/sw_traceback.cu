@@ -1033,10 +1033,12 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                     }
                 }
                 uint2 word[NW];
-                int row[NW];
+                int row[NW], run_cols[NW];
+                uint32_t run_bits[NW];
 #pragma unroll
                 for (int x = 0; x < NW; ++x) {
-                    row[x] = 0;
+                    row[x] = run_cols[x] = 0;
+                    run_bits[x] = 0u;
                     word[x] = make_uint2(0u, 0u);
                     if (cell[x]) {
                         const int wi = wi_[x];
@@ -1054,6 +1056,22 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                             const int64_t sector = ((int64_t)c * S4 + (t >> 2)) * 32 + g * T + kk;
                             if (ROWS == 8) word[x] = __ldcg((const uint2 *)slot + 4 * sector + (t & 3));
                             else word[x].x = __ldcg(slot + 4 * sector + (t & 3));
+                            // a deletion run under way: up to three columns
+                            // more of this sector (an intron's run is
+                            // hundreds of columns)
+                            if (wst_[x] == 1 && (t & 3) > 0 && jl > 0) {
+                                const int bit = 16 * (wi & 1) + 4 * (row[x] & 3) + 2;
+                                run_cols[x] = min(t & 3, jl);
+#pragma unroll
+                                for (int q = 1; q < 4; ++q)
+                                    if (q <= run_cols[x]) {
+                                        const int64_t at = 4 * sector + (t & 3) - q;
+                                        const uint32_t w = ROWS == 8
+                                                               ? __ldcg(slot + 2 * at + (row[x] >> 2))
+                                                               : __ldcg(slot + at);
+                                        run_bits[x] |= ((w >> bit) & 1u) << q;
+                                    }
+                            }
                         }
                     }
                 }
@@ -1073,10 +1091,23 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
                             // E(i,j) = H(i,j-1) + o or E(i,j-1) + e, and F
                             // the same way up
                             const bool del = wst_[x] == 1;
-                            push(x, del ? 2u : 1u, 1);
-                            if (!(code & (del ? 4u : 8u))) wst_[x] = 0;
-                            v_[x] -= wst_[x] == 0 ? P.sc.go : P.sc.ge;
-                            if (del) --j_[x];
+                            int32_t cols = 1;
+                            bool open = !(code & (del ? 4u : 8u));
+                            if (del && !open) {
+                                // extended columns of the sector, then
+                                // perhaps the opening one
+                                const int more_cols = run_cols[x];
+#pragma unroll
+                                for (int q = 1; q < 4; ++q)
+                                    if (q <= more_cols && !open) {
+                                        ++cols;
+                                        open = !((run_bits[x] >> q) & 1u);
+                                    }
+                            }
+                            push(x, del ? 2u : 1u, cols);
+                            v_[x] -= (cols - 1) * P.sc.ge + (open ? P.sc.go : P.sc.ge);
+                            if (open) wst_[x] = 0;
+                            if (del) j_[x] -= cols;
                             else --i_[x];
                         }
                         if (stopped(x)) go_[x] = false;
