@@ -32,6 +32,16 @@ __device__ __forceinline__ uint32_t load_bases(const uint32_t *__restrict__ buf,
     return __funnelshift_r(lo, hi, sh);
 }
 
+// The two words that hold the next 16 (at most cnt) bases from q on; none for
+// cnt <= 0.
+__device__ __forceinline__ void load_words(const uint32_t *__restrict__ buf, int64_t q, int cnt, uint32_t &lo,
+                                           uint32_t &hi)
+{
+    const uint32_t *const w = buf + (q >> 4);
+    lo = cnt > 0 ? __ldg(w) : 0u;
+    hi = cnt > 0 && ((int)q & 15) + min(cnt, 16) > 16 ? __ldg(w + 1) : 0u;
+}
+
 // Lanes of a converged warp that hold the same key form one group, led by
 // its lowest lane.  Per-pair atomics on a few hot counters (a batch whose
 // pairs share one length class sends every pair to the same histogram bin)

@@ -20,8 +20,13 @@ __device__ __forceinline__ void score_rows_any(const ScoreLaunch &L, int v)
 template <bool FMA_ADD>
 __global__ void __launch_bounds__(128) k_score_any(const __grid_constant__ ScoreLaunch L)
 {
-    for (int v = N_SCORE_VARIANTS - 1; v >= 0; --v) {
-        if (L.dp->var_n[v] == 0) continue;
+    // (one load for the list of variants: asking for each in turn cost 24 L2
+    // latencies in a row, a sixth of this kernel's time for 64 pairs)
+    const int lane = threadIdx.x & 31;
+    unsigned todo = __ballot_sync(0xffffffffu, lane < N_SCORE_VARIANTS && L.dp->var_n[lane] != 0);
+    while (todo) {
+        const int v = 31 - __clz(todo);  // longest reads first
+        todo ^= 1u << v;
         switch (v / N_VMODES) {
         case 0: score_rows_any<8, FMA_ADD>(L, v); break;
         case 1: score_rows_any<16, FMA_ADD>(L, v); break;
