@@ -82,6 +82,17 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
 {
     __shared__ int32_t s_var[N_CLASS], s_cnt[N_CLASS], s_bnd[N_CLASS], s_lanes[N_CLASS], s_ck[N_CLASS];
     __shared__ int16_t s_list[N_CLASS];
+    __shared__ int32_t s_pipe_tasks;
+    __shared__ unsigned long long s_pipe_bytes;
+    if (threadIdx.x == 0) {
+        s_pipe_tasks = 0;
+        s_pipe_bytes = 0;
+    }
+    __syncthreads();
+    auto long_class = [&](int c) { return pp.small && c >= N_MCLASS && info->max_m[c] > kPipeMinRead; };
+    for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x)
+        if (info->count[c] > 0 && long_class(c)) atomicAdd(&s_pipe_tasks, (info->count[c] + 1) / 2);
+    __syncthreads();
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = info->count[c];
         int32_t var = -1, bnd = 0, ck = 0;
@@ -90,16 +101,29 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
             const int mode = c / N_MCLASS;
             const int32_t mm = info->max_m[c], mn = info->max_n[c];
             int ri = 0, vmode = mode;
-            plan_class(pp, mode, cnt, mm, mn, lanes, ri, vmode);
+            // per group: two buffers x longest window x (H, F) x 4 bytes
+            int64_t pipe = -1;
+            if (long_class(c) && s_pipe_tasks <= pp.score_warps[0] / kPipeWarps) {
+                const unsigned long long need = 16ull * mn * ((cnt + 1) / 2);
+                const unsigned long long at = atomicAdd(&s_pipe_bytes, need);
+                if (at + need <= (unsigned long long)pp.pipe_bytes) pipe = (int64_t)at;
+            }
+            out->cls_pipe[c] = pipe;
+            if (pipe >= 0) {
+                lanes = 32;
+                ri = pipe_rows_idx(mm);
+                vmode = MODE_I16W;
+            } else {
+                plan_class(pp, mode, cnt, mm, mn, lanes, ri, vmode);
+            }
             const int rows = score_rows_at(ri);
             const int chunks = (mm + lanes * rows - 1) / (lanes * rows);
-            // per group: two buffers x longest window x (H, F) x 4 bytes
-            bnd = chunks > 1 ? 16 * mn : 0;
+            bnd = chunks > 1 && pipe < 0 ? 16 * mn : 0;
             var = ri * N_VMODES + vmode;
             if (pp.ck_bytes > 0 && mode != MODE_I32) ck = ck_block_rows(rows);
             out->cls_count[c] = cnt;
             out->cls_lanes[c] = lanes;
-            out->cls_bnd_bytes[c] = bnd;
+            out->cls_bnd_bytes[c] = pipe >= 0 ? 16 * mn : bnd;
         }
         s_var[c] = var;
         s_cnt[c] = cnt;

@@ -12,7 +12,15 @@ __device__ __forceinline__ void score_rows_any(const ScoreLaunch &L, int v)
     switch (v % N_VMODES) {
     case MODE_I32: score_body<R, MODE_I32, true, false>(L, v); break;
     case MODE_I16: score_body<R, MODE_I16, FMA_ADD, true>(L, v); break;
-    case MODE_I16W: score_body<R, MODE_I16W, FMA_ADD, true>(L, v); break;
+    case MODE_I16W:
+        if constexpr (R < 50) {
+            score_body<R, MODE_I16W, FMA_ADD, true, SCORE_WARP_TASKS>(L, v);
+            __syncthreads();
+            score_body<R, MODE_I16W, FMA_ADD, true, SCORE_BLOCK_TASKS>(L, v);
+        } else {
+            score_body<R, MODE_I16W, FMA_ADD, true>(L, v);
+        }
+        break;
     default: score_body<R, MODE_I16S, FMA_ADD, true>(L, v); break;
     }
 }

@@ -216,9 +216,21 @@ __host__ __device__ constexpr int score_snapshot_bytes(int rows, int mode, int t
     return mode == MODE_I16W || mode == MODE_I16S ? 2 * ((rows + 3) / 4) * 16 * threads : 0;
 }
 
+// The classes of its variant that a body serves: all (their tasks are a
+// warp's), those whose tasks are a warp's, or those whose tasks are a block's.
+enum { SCORE_ALL, SCORE_WARP_TASKS, SCORE_BLOCK_TASKS };
+
 // CK: checkpoints are kept for a traceback (launches without a CIGAR to
 // follow run the kernels without that code: 1 % faster).
-template <int R, int MODE, bool FMA_ADD, bool CK>
+//
+// Block tasks (TASKS == SCORE_BLOCK_TASKS, 32 lanes per two pairs): warp w
+// takes the row chunks w, w + 4, ... of the task.  A chunk's last lane leaves
+// the boundary row in the task's rows, as between the chunks of a warp's task,
+// and its warp says every eight iterations how many units of two columns are
+// there; the warp of the next chunk waits for them (s_prog), eight at a time,
+// and requests each one iteration ahead.  A wait gives up after a limit and
+// reports ST_INTERNAL.
+template <int R, int MODE, bool FMA_ADD, bool CK, int TASKS = SCORE_ALL>
 __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int variant)
 {
     typedef Arith<MODE> A;
@@ -261,7 +273,19 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
     const uint32_t GOH = 0x80008000u | ((uint32_t)(-go) * 0x10001u);
     // input already found invalid (or a plan whose shape changed): the
     // scratch may be too small for it, so do nothing
-    if (*(volatile const int32_t *)L.status & ST_BAD_INPUT) return;
+    constexpr bool PIPE = TASKS == SCORE_BLOCK_TASKS;
+    const int warp = threadIdx.x >> 5;
+    if constexpr (PIPE) {
+        if (__syncthreads_or(*(volatile const int32_t *)L.status & ST_BAD_INPUT)) return;
+    } else {
+        if (*(volatile const int32_t *)L.status & ST_BAD_INPUT) return;
+    }
+    // block tasks: the next task, its checkpoints, each warp's best, and the
+    // chunk (+ 1, upper half) and units of its boundary row that are stored
+    __shared__ uint64_t s_best[PIPE ? 2 * kPipeWarps : 1], s_prog[PIPE ? kPipeWarps : 1];
+    __shared__ int32_t s_base;
+    __shared__ uint32_t s_ck_base;
+    bool late = false;  // a wait gave up
 
     // One class given by the host, or every class of this launch's variant
     // in the device plan (longest reads first); the warps of the launch move
@@ -304,13 +328,15 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
     if (planned) {
         const DevScorePlan &dp = *L.dp;
         cls = dp.var_cls[variant][ci];
-        T = dp.cls_lanes[cls];
+        if (TASKS != SCORE_ALL && PIPE != (dp.cls_pipe[cls] >= 0)) continue;
+        T = PIPE ? 32 : dp.cls_lanes[cls];
         order = L.order + dp.cls_start[cls];
         n_items = dp.cls_count[cls];
         work_counter = L.work_counter + cls;
         bnd_group_bytes = dp.cls_bnd_bytes[cls];
         bnd_base = nullptr;
-        if (bnd_group_bytes) {
+        if (PIPE) bnd_base = L.pipe + dp.cls_pipe[cls];
+        if (!PIPE && bnd_group_bytes) {
             // reads in several row chunks: only warps with a boundary slot
             if (warp_global >= dp.var_bnd_warps[variant]) continue;
             bnd_base = L.boundary + dp.var_bnd_offset[variant];
@@ -331,15 +357,23 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
         cc->n_items = n_items;
         cc->cls = cls;
         if (CK) cc->ck_rows = planned && L.ck_pos ? L.dp->cls_ck[cls] : 0;
-        cc->bnd_warp = bnd_base ? bnd_base + warp_global * bnd_warp_bytes : nullptr;
+        cc->bnd_warp = bnd_base ? bnd_base + (PIPE ? 0 : warp_global * bnd_warp_bytes) : nullptr;
         cc->bnd_group_bytes = bnd_group_bytes;
     }
     __syncwarp();
 
     for (;;) {
         int base = 0;
-        if (lane == 0) base = atomicAdd(cc->work_counter, per_warp);
-        base = __shfl_sync(FULL, base, 0);
+        if constexpr (PIPE) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_base = atomicAdd(cc->work_counter, per_warp);
+            if (lane == 0) *(volatile uint64_t *)&s_prog[warp] = 0;
+            __syncthreads();
+            base = s_base;
+        } else {
+            if (lane == 0) base = atomicAdd(cc->work_counter, per_warp);
+            base = __shfl_sync(FULL, base, 0);
+        }
         if (base >= cc->n_items) break;
 
         const int64_t item = base + (int64_t)g * (PAIR2 ? 2 : 1);
@@ -357,6 +391,13 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
         const int steps = nw + T - 1;
 
         uint64_t bestA = 0, bestB = 0;
+        if (PIPE && CK) {
+            if (threadIdx.x == 0 && cc->ck_rows) {
+                const int32_t rl = ((nw + 1) >> 1) + T - 1, nr = mw > 0 ? (mw - 1) / cc->ck_rows : 0;
+                s_ck_base = nr ? atomicAdd(L.ck_cursor, (uint32_t)(nr * rl)) : 0u;
+            }
+            __syncthreads();
+        }
         if (CK && cc->ck_rows) {
             if (lane == 0) {
                 // (room for the columns past the window that lanes before
@@ -364,12 +405,13 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                 const int32_t rl = ((nw + 1) >> 1) + T - 1, nr = mw > 0 ? (mw - 1) / cc->ck_rows : 0;
                 cc->ck_row_units = rl;
                 cc->ck_n = nr;
-                cc->ck_base = nr ? atomicAdd(L.ck_cursor, (uint32_t)(G * nr * rl)) : 0u;
+                if (PIPE) cc->ck_base = s_ck_base;
+                else cc->ck_base = nr ? atomicAdd(L.ck_cursor, (uint32_t)(G * nr * rl)) : 0u;
             }
             __syncwarp();
         }
 
-        for (int c = 0; c < chunks; ++c) {
+        for (int c = PIPE ? warp : 0; c < chunks; c += PIPE ? kPipeWarps : 1) {
             const int i0 = c * rows_per_chunk + k * R;
             // per-row selectors
             uint32_t sel[R];
@@ -411,8 +453,8 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
             const bool store_bnd = c + 1 < chunks;
             // this group's double-buffered boundary row (bytes per buffer: half)
             uint8_t *const bnd_w = cc->bnd_warp;
-            const int64_t bgb = cc->bnd_group_bytes;
-            uint8_t *const bnd = (on && bnd_w) ? bnd_w + g * bgb : nullptr;
+            const int64_t bgb = PIPE ? (int64_t)16 * nw : cc->bnd_group_bytes;
+            uint8_t *const bnd = (on && bnd_w) ? bnd_w + (PIPE ? (int64_t)(base >> 1) * cc->bnd_group_bytes : g * bgb) : nullptr;
             const int64_t bnd_half = bgb / 2;
             const V *bin = load_bnd && bnd ? (const V *)(bnd + (c & 1) * bnd_half) : nullptr;
             V *bout = store_bnd && bnd ? (V *)(bnd + ((c + 1) & 1) * bnd_half) : nullptr;
@@ -455,6 +497,32 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
             };
             fetch(0);
             const int iters = (nw + 1) / 2 + T - 1;
+            // block tasks: unit u of the row above, requested an iteration ahead
+            uint2 in0 = make_uint2(0, 0), in1 = in0;
+            auto wait_units = [&](int units) {
+                if (lane == 0 && !late) {
+                    const uint64_t want = ((uint64_t)c << 32) | (uint32_t)min(units, (ng + 1) >> 1);
+                    volatile uint64_t *const at = &s_prog[(warp + kPipeWarps - 1) % kPipeWarps];
+                    for (int spin = 0; *at < want; ++spin) {
+                        if (spin >= (1 << 22)) {
+                            late = true;
+                            atomicOr(L.status, ST_INTERNAL);
+                            break;
+                        }
+                        __nanosleep(40);
+                    }
+                }
+                __threadfence_block();
+                __syncwarp();
+            };
+            auto request_unit = [&](int u) {
+                in0 = 2 * u < ng ? *(const uint2 *)&bin[4 * u] : make_uint2(0, 0);
+                in1 = 2 * u + 1 < ng ? *(const uint2 *)&bin[4 * u + 2] : make_uint2(0, 0);
+            };
+            if (PIPE && load_bnd) {
+                wait_units(9);
+                if (k == 0) request_unit(0);
+            }
             auto col_best = [&](const V (&hv)[R], uint32_t ck, int jj) {
                 if constexpr (MODE == MODE_I16) {
                     const uint32_t nb = __vimax_s16x2_relu(bk0, ck | (TAGM * 0x10001u));
@@ -487,7 +555,18 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                 V up_f0 = __shfl_up_sync(FULL, out_f, 1);
                 V up_h1 = __shfl_up_sync(FULL, out_h1, 1);
                 V up_f1 = __shfl_up_sync(FULL, out_f1, 1);
-                if (k == 0) {
+                if constexpr (PIPE) {
+                    if (k == 0) {
+                        up_h0 = (V)in0.x;
+                        up_f0 = (V)in0.y;
+                        up_h1 = (V)in1.x;
+                        up_f1 = (V)in1.y;
+                    }
+                    if (load_bnd) {
+                        if ((u & 7) == 0 && u) wait_units(u + 9);
+                        if (k == 0) request_unit(u + 1);
+                    }
+                } else if (k == 0) {
                     up_h0 = bin && j0 < ng ? bin[2 * j0] : 0;
                     up_f0 = bin && j0 < ng ? bin[2 * j0 + 1] : 0;
                     up_h1 = bin && j0 + 1 < ng ? bin[2 * j0 + 2] : 0;
@@ -587,6 +666,10 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                         bout[2 * j0 + 3] = out_f1;
                     }
                 }
+                if (PIPE && store_bnd && k == T - 1 && ((u & 7) == 7 || u + 1 == iters)) {
+                    __threadfence_block();
+                    *(volatile uint64_t *)&s_prog[warp] = ((uint64_t)(c + 1) << 32) | (uint32_t)max(0, u + 2 - T);
+                }
                 // strict improvement keeps the first column: j0 before j0 + 1
                 col_best(h, ckA, j0);
                 col_best(h1, ckB, j0 + 1);
@@ -662,6 +745,18 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
             const int src = (k + d < T) ? lane + d : lane;
             bestA = max(bestA, __shfl_sync(FULL, bestA, src));
             if (PAIR2) bestB = max(bestB, __shfl_sync(FULL, bestB, src));
+        }
+        if constexpr (PIPE) {
+            if (lane == 0) {
+                s_best[2 * warp] = bestA;
+                s_best[2 * warp + 1] = bestB;
+            }
+            __syncthreads();
+            if (warp) continue;
+            for (int w = 1; w < kPipeWarps; ++w) {
+                bestA = max(bestA, s_best[2 * w]);
+                bestB = max(bestB, s_best[2 * w + 1]);
+            }
         }
         // outputs, and with a traceback to follow, each pair's traceback cost
         // key (the key pass folded into this epilogue)

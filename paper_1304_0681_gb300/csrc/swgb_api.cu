@@ -274,6 +274,7 @@ struct Scratch {
     TbClassInfo *tbinfo;
     DevScorePlan *splan;
     DevTbPlan *tplan;
+    uint8_t *pipe;  // boundary rows of a small batch's block tasks
     uint8_t *score_bnd;
     int64_t score_bnd_bytes;
     uint32_t *tb;
@@ -282,7 +283,7 @@ struct Scratch {
 
 // Lays out the pair-count-sized part at base (nullptr: sizes only); returns
 // its bytes.
-size_t fixed_layout(int64_t n_pairs, uint8_t *base, Scratch &S)
+size_t fixed_layout(int64_t n_pairs, int64_t pipe_bytes, uint8_t *base, Scratch &S)
 {
     const size_t nh = (size_t)N_CLASS * N_NBUCKET;
     size_t off = 0;
@@ -305,6 +306,7 @@ size_t fixed_layout(int64_t n_pairs, uint8_t *base, Scratch &S)
     S.expect = (int32_t *)take(sizeof(int32_t) * 3 * N_CLASS);
     S.splan = (DevScorePlan *)take(sizeof(DevScorePlan));
     S.tplan = (DevTbPlan *)take(sizeof(DevTbPlan));
+    S.pipe = take(pipe_bytes);
     return off;
 }
 
@@ -338,6 +340,7 @@ ScoreLaunch score_launch(const PairSet &ps, const Scoring &sc, int32_t *out_scor
     L.out_score = out_score;
     L.out_end = out_end;
     L.boundary = S.score_bnd;
+    L.pipe = S.pipe;
     L.work_counter = S.counters;
     L.status = &S.info->status;
     if (cigar) {
@@ -373,6 +376,7 @@ int enqueue_small(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Sco
     int rc = SW_OK;
     const bool timing = x.timing && x.phase;
     pp.small = 1;
+    pp.pipe_bytes = kPipeBytes;
     for (int v = 0; v < N_SCORE_VARIANTS; ++v) pp.score_warps[v] = x.any_blocks * (kThreads / 32);
     auto blocks = [&](int full) { return (int)std::min<int64_t>(full, n_pairs); };
     if (timing && cuda_failed(cudaEventRecord(x.phase[0], st))) return SW_ERR_CUDA;
@@ -468,7 +472,9 @@ int run_batch(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const sw_scor
     std::lock_guard<std::mutex> lk(ds->mu);
     const Scoring sc{scoring->match, scoring->mismatch, scoring->gap_open, scoring->gap_extend};
     Scratch S{};
-    const size_t fixed_bytes = fixed_layout(n_pairs, nullptr, S);
+    // (the block tasks' rows are taken for every size: a small call captured on
+    // a stream of larger ones finds them there)
+    const size_t fixed_bytes = fixed_layout(n_pairs, kPipeBytes, nullptr, S);
     const int64_t bnd_bytes = std::min(kScoreBndMax, std::max(kScoreBndMin, n_pairs * kScoreBndPerPair));
     int64_t tb_bytes = 0;
     if (cig) {
@@ -483,7 +489,7 @@ int run_batch(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const sw_scor
     }
     if ((rc = ensure_on(ds->fixed, fixed_bytes, st))) return rc;
     if ((rc = ensure_on(ds->dyn, (size_t)(bnd_bytes + tb_bytes), st))) return rc;
-    fixed_layout(n_pairs, (uint8_t *)ds->fixed.ptr, S);
+    fixed_layout(n_pairs, kPipeBytes, (uint8_t *)ds->fixed.ptr, S);
     S.score_bnd = (uint8_t *)ds->dyn.ptr;
     S.score_bnd_bytes = bnd_bytes;
     S.tb = (uint32_t *)((uint8_t *)ds->dyn.ptr + bnd_bytes);
@@ -615,8 +621,9 @@ int plan_build(sw_plan *pl, DeviceState *ds, cudaStream_t st)
     int rc = SW_OK;
     const int64_t n_pairs = pl->n_pairs;
     Scratch &S = pl->S;
-    if ((rc = ensure(pl->fixed, fixed_layout(n_pairs, nullptr, S)))) return rc;
-    fixed_layout(n_pairs, (uint8_t *)pl->fixed.ptr, S);
+    const int64_t pipe_bytes = n_pairs <= kSmallPairs ? kPipeBytes : 0;
+    if ((rc = ensure(pl->fixed, fixed_layout(n_pairs, pipe_bytes, nullptr, S)))) return rc;
+    fixed_layout(n_pairs, pipe_bytes, (uint8_t *)pl->fixed.ptr, S);
     // classify once (it reads offsets only) and read the class table back
     const size_t nh = (size_t)N_CLASS * N_NBUCKET;
     if (cuda_failed(cudaMemsetAsync(S.hist, 0, sizeof(int32_t) * nh, st))) return SW_ERR_CUDA;

@@ -103,6 +103,7 @@ struct ScoreLaunch {
     int32_t *out_score;
     int32_t *out_end;
     uint8_t *boundary;       // per-group chunk boundaries, or nullptr
+    uint8_t *pipe = nullptr; // boundary rows of block tasks
     int64_t boundary_group_bytes;
     int32_t *work_counter;
     int32_t *status;
@@ -221,6 +222,19 @@ constexpr int kSmallPairs = 4096;
 // Row counts in the one score launch of a small batch (8, 16, 25, 50).
 __host__ __device__ inline bool small_rows(int rows_idx) { return rows_idx != 2 && rows_idx != 4; }
 
+// Block tasks.  A long read's two pairs in one warp take a row chunk after
+// another, and a few of them leave the SMs empty: 200 reads of 1000 to 4000
+// bases took 8.9 ms.  While there are at most kPipeTasks such tasks the four
+// warps of a block take a task's chunks side by side, each one wavefront
+// behind the other, with as few rows per lane as keep it at four chunks.
+// Classes of reads of up to 256 bases (one chunk of the fewest rows) never do.
+constexpr int kPipeMinRead = 512, kPipeWarps = 4;
+constexpr int64_t kPipeBytes = (int64_t)64 << 20;
+__host__ __device__ inline int pipe_rows_idx(int32_t m_max)
+{
+    return m_max <= kPipeWarps * 32 * 8 ? 0 : m_max <= kPipeWarps * 32 * 16 ? 1 : 3;  // 8, 16, 25 rows
+}
+
 struct PlanOverride {
     int32_t max_read_len, lanes, rows;
 };
@@ -237,6 +251,7 @@ struct PlanParams {
     int64_t ck_bytes;                       // most of it that row checkpoints may take (0: none)
     int32_t allow16;                        // 16-bit traceback allowed (SW_TB_AUTO)
     int32_t small;                          // the launches of a small batch
+    int64_t pipe_bytes;                     // boundary rows of block tasks (small batches)
 };
 
 struct DevScorePlan {
@@ -249,6 +264,7 @@ struct DevScorePlan {
     int32_t cls_lanes[N_CLASS];
     int32_t cls_bnd_bytes[N_CLASS];           // per group; 0 when a read fits one row chunk
     int32_t cls_ck[N_CLASS];                  // rows between checkpoints (0: none kept)
+    int64_t cls_pipe[N_CLASS];                // a small batch's classes of block tasks: their boundary rows' offset, else -1
     int64_t ck_units;                         // 16-byte units of the pool the checkpoints may take
     int16_t var_cls[N_SCORE_VARIANTS][N_CLASS];  // longest reads first
 };
