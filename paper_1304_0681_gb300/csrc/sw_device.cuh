@@ -32,14 +32,17 @@ __device__ __forceinline__ uint32_t load_bases(const uint32_t *__restrict__ buf,
     return __funnelshift_r(lo, hi, sh);
 }
 
-// The two words that hold the next 16 (at most cnt) bases from q on; none for
-// cnt <= 0.
-__device__ __forceinline__ void load_words(const uint32_t *__restrict__ buf, int64_t q, int cnt, uint32_t &lo,
-                                           uint32_t &hi)
+// The two words that hold the 16 columns from j on of a window of n columns
+// whose column 0 is base q0 (columns before the window or past its end are
+// whatever those words hold, or 0).
+__device__ __forceinline__ void load_columns(const uint32_t *__restrict__ buf, int64_t q0, int j, int n, uint32_t &lo,
+                                             uint32_t &hi)
 {
+    const int64_t q = q0 + j;
     const uint32_t *const w = buf + (q >> 4);
-    lo = cnt > 0 ? __ldg(w) : 0u;
-    hi = cnt > 0 && ((int)q & 15) + min(cnt, 16) > 16 ? __ldg(w + 1) : 0u;
+    const bool any = j > -16 && j < n;
+    lo = any && q >= 0 ? __ldg(w) : 0u;
+    hi = any && ((int)q & 15) + min(n - j, 16) > 16 ? __ldg(w + 1) : 0u;
 }
 
 // Lanes of a converged warp that hold the same key form one group, led by

@@ -250,13 +250,19 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
     static_assert(R <= 64, "row tags cover at most 64 rows");
 
     // column tables: s_tab[w] byte x = s(x, w) - o; s_tab[4] = 0 (padding)
+    // s_tab2: two columns at once, w0 + 4 w1; 16 + w0 without the second one;
+    // 20 neither
     __shared__ uint32_t s_tab[8];
+    __shared__ uint2 s_tab2[21];
     const int32_t go = L.sc.go, ge = L.sc.ge;
     {
         const uint32_t mis4 = ((uint32_t)(uint8_t)(int8_t)(L.sc.mi - go)) * 0x01010101u;
         const uint32_t ma4 = ((uint32_t)(uint8_t)(int8_t)(L.sc.ma - go)) * 0x01010101u;
-        if (threadIdx.x < 8)
-            s_tab[threadIdx.x] = threadIdx.x < 4 ? prmt(mis4, ma4, 0x3210u + (4u << (4u * threadIdx.x))) : 0u;
+        auto column = [&](uint32_t w) { return prmt(mis4, ma4, 0x3210u + (4u << (4u * w))); };
+        if (!PAIR2 && threadIdx.x < 8) s_tab[threadIdx.x] = threadIdx.x < 4 ? column(threadIdx.x) : 0u;
+        if (PAIR2 && threadIdx.x < 21)
+            s_tab2[threadIdx.x] = make_uint2(threadIdx.x < 20 ? column(threadIdx.x & 3u) : 0u,
+                                             threadIdx.x < 16 ? column(threadIdx.x >> 2) : 0u);
         __syncthreads();
     }
 
@@ -485,17 +491,24 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                 }
                 if (CK_SHARED) s_ck_at[threadIdx.x] = ck_at;
             }
-            // The window's next 16 bases are requested an iteration before they
-            // are used, as the two words that hold them: some lane of the
-            // wavefront starts a word in every iteration, and the warp waited
-            // for it (30,000 reads of 150 bases x 1-64 windows 7.90 -> 7.56 ms,
-            // 2M uneven pairs 51.8 -> 51.0 with the traceback).
+            // Window bases: every eight iterations each lane takes its next 16
+            // columns, requested an iteration before as the two words that
+            // hold them.  (When each lane asked as it got there the warp waited
+            // in nearly every iteration: 30,000 reads of 150 bases x 1-64
+            // windows 7.90 ms instead of 7.63, 2M uneven pairs 51.8 instead of
+            // 49.1.  The loop around the cells is 130 of a step's 280
+            // instructions at 8 rows per lane, 600 at 25: one branch for all
+            // lanes, one 8-byte table read per pair and step.)
             uint32_t wxA = 0, wxB = 0;
-            auto fetch = [&](int j) {
-                load_words(L.ps.wins, pa.ws + j, pa.n - j, wwA, wxA);
-                load_words(L.ps.wins, pb.ws + j, pb.n - j, wwB, wxB);
+            const uint32_t sh = (uint32_t)(2 * (((int)pa.ws - 2 * k) & 15)) | (uint32_t)(2 * (((int)pb.ws - 2 * k) & 15)) << 8;
+            auto request = [&](int j) {
+                load_columns(L.ps.wins, pa.ws, j, pa.n, wwA, wxA);
+                load_columns(L.ps.wins, pb.ws, j, pb.n, wwB, wxB);
             };
-            fetch(0);
+            request(-2 * k);
+            // iterations in which every lane has two columns of every real
+            // pair: from T - 1 on, so many
+            const unsigned inner = (unsigned)max(0, (nmin_w >> 1) - (T - 1));
             const int iters = (nw + 1) / 2 + T - 1;
             // block tasks: unit u of the row above, requested an iteration ahead
             uint2 in0 = make_uint2(0, 0), in1 = in0;
@@ -566,33 +579,29 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                         if ((u & 7) == 0 && u) wait_units(u + 9);
                         if (k == 0) request_unit(u + 1);
                     }
-                } else if (k == 0) {
-                    up_h0 = bin && j0 < ng ? bin[2 * j0] : 0;
-                    up_f0 = bin && j0 < ng ? bin[2 * j0 + 1] : 0;
-                    up_h1 = bin && j0 + 1 < ng ? bin[2 * j0 + 2] : 0;
-                    up_f1 = bin && j0 + 1 < ng ? bin[2 * j0 + 3] : 0;
-                }
-                uint32_t t0A = 0, t0B = 0, t1A = 0, t1B = 0;
-                if (j0 >= 0) {
-                    if ((j0 & 15) == 0) {
-                        wwA = __funnelshift_r(wwA, wxA, 2 * ((int)pa.ws & 15));
-                        wwB = __funnelshift_r(wwB, wxB, 2 * ((int)pb.ws & 15));
+                } else {
+                    if (k == 0) up_h0 = up_f0 = up_h1 = up_f1 = 0;
+                    if (load_bnd && bin && k == 0) {
+                        up_h0 = j0 < ng ? bin[2 * j0] : 0;
+                        up_f0 = j0 < ng ? bin[2 * j0 + 1] : 0;
+                        up_h1 = j0 + 1 < ng ? bin[2 * j0 + 2] : 0;
+                        up_f1 = j0 + 1 < ng ? bin[2 * j0 + 3] : 0;
                     }
-                    if (2 * u + 1 < nmin_w) {  // every real pair of the warp has columns j0 and j0 + 1
-                        t0A = s_tab[wwA & 3u];
-                        t1A = s_tab[(wwA >> 2) & 3u];
-                        t0B = s_tab[wwB & 3u];
-                        t1B = s_tab[(wwB >> 2) & 3u];
-                    } else {
-                        t0A = s_tab[j0 < pa.n ? wwA & 3u : 4u];
-                        t1A = s_tab[j0 + 1 < pa.n ? (wwA >> 2) & 3u : 4u];
-                        t0B = s_tab[j0 < pb.n ? wwB & 3u : 4u];
-                        t1B = s_tab[j0 + 1 < pb.n ? (wwB >> 2) & 3u : 4u];
-                    }
-                    wwA >>= 4;
-                    wwB >>= 4;
-                    if ((j0 & 15) == 14) fetch(j0 + 2);
                 }
+                if ((u & 7) == 0) {
+                    wwA = __funnelshift_r(wwA, wxA, sh);
+                    wwB = __funnelshift_r(wwB, wxB, sh >> 8);
+                }
+                uint32_t xA = wwA & 15u, xB = wwB & 15u;
+                if ((unsigned)(u - (T - 1)) >= inner) {
+                    xA = j0 < 0 || j0 >= pa.n ? 20u : j0 + 1 < pa.n ? xA : 16u + (xA & 3u);
+                    xB = j0 < 0 || j0 >= pb.n ? 20u : j0 + 1 < pb.n ? xB : 16u + (xB & 3u);
+                }
+                const uint2 tA = s_tab2[xA], tB = s_tab2[xB];
+                const uint32_t t0A = tA.x, t1A = tA.y, t0B = tB.x, t1B = tB.y;
+                wwA >>= 4;
+                wwB >>= 4;
+                if ((u & 7) == 7) request(j0 + 2);
                 V hu0 = up_h0, f0 = up_f0, hu1 = up_h1, f1 = up_f1;
                 uint32_t ckA = 0, pkA = 0, ckB = 0, pkB = 0;
                 V d0n, d1n;
@@ -656,7 +665,7 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
                         L.ck_pool[at + ((uint32_t)j0 >> 1)] =
                             make_uint4((uint32_t)out_h, (uint32_t)out_f, (uint32_t)out_h1, (uint32_t)out_f1);
                 }
-                if (bout && k == T - 1 && j0 >= 0) {
+                if (store_bnd && bout && k == T - 1 && j0 >= 0) {
                     if (j0 < ng) {
                         bout[2 * j0] = out_h;
                         bout[2 * j0 + 1] = out_f;
@@ -786,8 +795,14 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
     }  // classes
 }
 
+// Blocks per SM that the registers are held to.
+constexpr int score_min_blocks(int R, int mode)
+{
+    return R <= 16 ? 4 : R <= 25 || (R == 32 && mode == MODE_I16) ? 3 : 2;
+}
+
 template <int R, int MODE, bool FMA_ADD, bool CK>
-__global__ void __launch_bounds__(128) k_score(const __grid_constant__ ScoreLaunch L)
+__global__ void __launch_bounds__(128, score_min_blocks(R, MODE)) k_score(const __grid_constant__ ScoreLaunch L)
 {
     score_body<R, MODE, FMA_ADD, CK>(L, L.variant);
 }
