@@ -45,34 +45,86 @@ __device__ __forceinline__ int list_classes(const int32_t *count, int16_t *list)
     return n;
 }
 
-// A score plan for one class: lanes per group, rows index and kernel mode.
-__device__ __forceinline__ void plan_class(const PlanParams &pp, int mode, int32_t cnt, int32_t mm, int32_t mn,
-                                           int &lanes, int &ri, int &vmode)
+// The score plan of a class in a batch that fills the GPU: lanes per group,
+// rows index and kernel mode.  Returns whether an override gives it.
+__device__ __forceinline__ bool plan_class(const PlanParams &pp, int mode, int32_t mm, int32_t mn, int &lanes, int &ri,
+                                           int &vmode)
 {
     const int64_t hmax = (int64_t)pp.sc.ma * min(mm, mn);
     score_plan_of(mode, mm, hmax, pp.ov, pp.n_overrides, lanes, ri);
     vmode = score_vmode(mode, hmax, pp.sc);
-    // an override's plan is kept
     for (int i = 0; i < pp.n_overrides; ++i)
-        if (mm <= pp.ov[i].max_read_len) return;
+        if (mm <= pp.ov[i].max_read_len) return true;
     if (pp.small && !small_rows(ri)) {
         // a small batch's one launch holds every other row count: the next
         // larger one (its lanes then cover the read in no more chunks)
         ++ri;
         lanes = min(32, (mm + score_rows_at(ri) - 1) / score_rows_at(ri));
     }
-    // a class with fewer tasks than half its launch's warps (a small batch)
-    // finishes when one task does: fewer rows per lane, on more lanes,
-    // shorten the task while it still fits one row chunk
-    while (ri > 0) {
-        const int64_t per_warp = (int64_t)(32 / lanes) * (mode != MODE_I32 ? 2 : 1);
-        const int64_t tasks = (cnt + per_warp - 1) / per_warp;
-        if (2 * tasks >= pp.score_warps[ri * N_VMODES + vmode]) break;
-        const int r2 = pp.small && !small_rows(ri - 1) ? ri - 2 : ri - 1;
-        const int t2 = (mm + score_rows_at(r2) - 1) / score_rows_at(r2);
-        if (t2 > 32) break;
-        ri = r2;
-        lanes = t2;
+    return false;
+}
+
+// Issue slots of a class's task (a warp's groups) at a rows index, in the
+// units of score_plan_of's cost.
+__device__ __forceinline__ int64_t task_slots(int mode, int ri, int lanes, int32_t mean_n)
+{
+    return (int64_t)((mode != MODE_I32 ? mean_n / 2 : mean_n) + lanes) * (13 * score_rows_at(ri) + 80);
+}
+
+// Tasks of cnt pairs at this many lanes per group.
+__device__ __forceinline__ uint32_t class_tasks(int mode, int32_t cnt, int lanes)
+{
+    const uint32_t per_warp = (uint32_t)(32 / lanes) * (mode != MODE_I32 ? 2u : 1u);
+    return ((uint32_t)cnt + per_warp - 1u) / per_warp;
+}
+
+// Fewer rows per lane, on more lanes, make a class's tasks shorter and more,
+// and cost slots.
+//
+// A class that is most of its batch takes the plan with the least estimated
+// time, of those with the read in one row chunk.  A launch's warps take tasks
+// in waves; a warp by itself issues an instruction every 2.7 cycles, a scheduler
+// with enough warps one every 1.25, so a wave takes a task's slots times the
+// warps on a scheduler or times 13/6, whichever is more.  Score pass with its
+// launches at 16,384 pairs of 100 x 200: 50 rows 0.209 ms, 32 0.203, 25 0.175
+// (taken), 20 0.154, 16 0.165, 8 0.183; of 150 x 250: 50 rows 0.256, 25 0.209
+// (taken), 16 0.244; 40,000 of 250 x 350: 50 rows 0.907, 25 0.863 (taken), 16
+// 0.948.  From about 100,000 pairs on it is the full GPU's plan.
+//
+// The other classes run beside more work than their own, and so do a small
+// batch's, whose launch holds every plan: fewer rows while a class has fewer
+// tasks than half its launch's warps (20,000 reads of six lengths: the estimate
+// above took 2.8 ms, this 1.5).
+__device__ __forceinline__ void plan_rows(const PlanParams &pp, int mode, int vmode, int32_t cnt, int32_t mm,
+                                          int32_t mean_n, bool most, int &lanes, int &ri)
+{
+    if (pp.small || !most) {
+        while (ri > 0) {
+            if (2 * (int64_t)class_tasks(mode, cnt, lanes) >= pp.score_warps[ri * N_VMODES + vmode]) break;
+            const int r2 = pp.small && !small_rows(ri - 1) ? ri - 2 : ri - 1;
+            const int t2 = (mm + score_rows_at(r2) - 1) / score_rows_at(r2);
+            if (t2 > 32) break;
+            ri = r2;
+            lanes = t2;
+        }
+        return;
+    }
+    int64_t best = -1;
+    for (int r = ri; r >= 0; --r) {
+        const int t = (mm + score_rows_at(r) - 1) / score_rows_at(r);
+        if (t > 32) break;
+        const uint32_t tasks = class_tasks(mode, cnt, t), warps = (uint32_t)pp.score_warps[r * N_VMODES + vmode];
+        // in sixths of a task's slots
+        const uint32_t sch = (uint32_t)pp.schedulers;
+        auto wave = [&](uint32_t w) { return max(13u, 6u * ((w + sch - 1u) / sch)); };
+        const uint32_t full = tasks / warps, last = tasks - full * warps;
+        const int64_t cost =
+            task_slots(mode, r, t, mean_n) * ((int64_t)full * wave(warps) + (last ? wave(last) : 0u));
+        if (best < 0 || cost < best) {
+            best = cost;
+            ri = r;
+            lanes = t;
+        }
     }
 }
 
@@ -83,15 +135,29 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
     __shared__ int32_t s_var[N_CLASS], s_cnt[N_CLASS], s_bnd[N_CLASS], s_lanes[N_CLASS], s_ck[N_CLASS];
     __shared__ int16_t s_list[N_CLASS];
     __shared__ int32_t s_pipe_tasks;
-    __shared__ unsigned long long s_pipe_bytes;
+    __shared__ unsigned long long s_pipe_bytes, s_slots, s_work[N_CLASS];
     if (threadIdx.x == 0) {
         s_pipe_tasks = 0;
         s_pipe_bytes = 0;
+        s_slots = 0;
     }
     __syncthreads();
     auto long_class = [&](int c) { return pp.small && c >= N_MCLASS && info->max_m[c] > kPipeMinRead; };
-    for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x)
-        if (info->count[c] > 0 && long_class(c)) atomicAdd(&s_pipe_tasks, (info->count[c] + 1) / 2);
+    auto mean_n = [&](int c) { return (int32_t)__fdividef((float)info->sum_n[c], (float)info->count[c]); };
+    for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
+        const int32_t cnt = info->count[c];
+        if (cnt == 0) continue;
+        if (long_class(c)) atomicAdd(&s_pipe_tasks, (cnt + 1) / 2);
+        const int mode = c / N_MCLASS;
+        int lanes = 1, ri = 0, vmode = 0;
+        const bool fixed = plan_class(pp, mode, info->max_m[c], info->max_n[c], lanes, ri, vmode);
+        const unsigned long long work =
+            (unsigned long long)class_tasks(mode, cnt, lanes) * (unsigned long long)task_slots(mode, ri, lanes, mean_n(c));
+        s_var[c] = fixed ? ~(ri * N_VMODES + vmode) : ri * N_VMODES + vmode;
+        s_lanes[c] = lanes;
+        s_work[c] = work;
+        atomicAdd(&s_slots, work);
+    }
     __syncthreads();
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = info->count[c];
@@ -114,7 +180,12 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
                 ri = pipe_rows_idx(mm);
                 vmode = MODE_I16W;
             } else {
-                plan_class(pp, mode, cnt, mm, mn, lanes, ri, vmode);
+                const bool fixed = s_var[c] < 0, most = 4 * s_work[c] >= 3 * s_slots;
+                const int v = fixed ? ~s_var[c] : s_var[c];
+                ri = v / N_VMODES;
+                vmode = v % N_VMODES;
+                lanes = s_lanes[c];
+                if (!fixed) plan_rows(pp, mode, vmode, cnt, mm, mean_n(c), most, lanes, ri);
             }
             const int rows = score_rows_at(ri);
             const int chunks = (mm + lanes * rows - 1) / (lanes * rows);

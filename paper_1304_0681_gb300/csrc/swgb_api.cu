@@ -56,6 +56,7 @@ struct ExecCtx {
     int score_blocks[N_SCORE_VARIANTS] = {};
     int tb_blocks[N_TB_VARIANTS] = {};
     int any_blocks = 0;
+    int sm_count = 0;
     cudaStream_t aux[kAuxStreams] = {};
     cudaEvent_t fork_ev = nullptr;
     cudaEvent_t join_ev[kAuxStreams] = {};
@@ -66,6 +67,7 @@ struct ExecCtx {
 int exec_ctx_init(ExecCtx &x, int sm_count)
 {
     int rc = SW_OK;
+    x.sm_count = sm_count;
     for (int v = 0; v < N_SCORE_VARIANTS; ++v)
         if ((rc = score_variant_blocks(v, sm_count, &x.score_blocks[v]))) return rc;
     for (int v = 0; v < N_TB_VARIANTS; ++v)
@@ -322,6 +324,7 @@ PlanParams plan_params(const ExecCtx &x, const Scoring &sc, bool allow16, int64_
     }
     for (int v = 0; v < N_SCORE_VARIANTS; ++v) pp.score_warps[v] = x.score_blocks[v] * (kThreads / 32);
     for (int v = 0; v < N_TB_VARIANTS; ++v) pp.tb_warps[v] = x.tb_blocks[v] * (kThreads / 32);
+    pp.schedulers = 4 * x.sm_count;
     pp.score_bnd_bytes = score_bnd_bytes;
     pp.tb_bytes = tb_bytes;
     pp.ck_bytes = allow16 ? tb_bytes / 4 * 3 : 0;

@@ -251,6 +251,7 @@ struct PlanParams {
     int64_t ck_bytes;                       // most of it that row checkpoints may take (0: none)
     int32_t allow16;                        // 16-bit traceback allowed (SW_TB_AUTO)
     int32_t small;                          // the launches of a small batch
+    int32_t schedulers;                     // warp schedulers of the device
     int64_t pipe_bytes;                     // boundary rows of block tasks (small batches)
 };
 
@@ -296,7 +297,7 @@ struct DevTbPlan {
 // narrower bands (a block's band allows for its own loss) but store more.
 __host__ __device__ inline int ck_block_rows(int R)
 {
-    return R >= 50 ? R : R > 16 ? 2 * R : 64;
+    return R >= 50 ? R : R == 20 ? 60 : R > 16 ? 2 * R : 64;
 }
 
 // 16-byte units that the checkpoints of a class take at most: a task of
