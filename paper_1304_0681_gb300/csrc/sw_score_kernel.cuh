@@ -69,7 +69,7 @@
 // int32 mode covers the rest.
 //
 // Checkpoints.  With a CIGAR to follow, the lanes whose bottom row ends a
-// block of 40 to 64 read rows also store that row (H and F - o of every
+// block of 50 to 64 read rows also store that row (H and F - o of every
 // column, both pairs, two columns to a 16-byte store) in a pool from which
 // the traceback recomputes one block at a time.  One store per ~800
 // instructions of a step: 0.08 bytes per cell.

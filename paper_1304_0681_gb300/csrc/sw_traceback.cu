@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(128) k_traceback(const TracebackLaunch L)
 // cells.
 //
 // Blocks.  The score pass kept H and F of every column for the rows that end
-// a block of 40 to 64 read rows (the checkpoints).  A pair's path is at
+// a block of 50 to 64 read rows (the checkpoints).  A pair's path is at
 // (i, j) with the exact value v of its state; the block of row i is swept
 // from the checkpoint above it (row i0 - 1, or the matrix edge) down to row
 // i over the columns the path can use, the walk goes back through the block
@@ -458,9 +458,10 @@ __global__ void __launch_bounds__(128) k_traceback(const TracebackLaunch L)
 // own.
 //
 // Sweep.  Lane k of a group holds 8 rows (4 with 16 lanes) of a chunk of 8T
-// (64) rows on a one-step wavefront.  A lane stores two 32-bit words per window offset (rows 0-3 and
-// rows 4-7; pair A in bits 0-15, pair B in bits 16-31), and its words of four
-// consecutive offsets share one 32-byte sector: uint2
+// (64) rows on a one-step wavefront.  A lane stores two 32-bit words per
+// window offset (rows 0-3 and rows 4-7; pair A in bits 0-15, pair B in bits
+// 16-31), and its words of four consecutive offsets share one 32-byte sector:
+// uint2
 // [((chunk x S4 + t / 4) x 32 + lane) x 4 + t % 4].  Per cell four bits record
 // which equalities fail (1 = not equal):
 //   bit 0  H != H(i-1,j-1) + s    bit 1  H != E

@@ -292,7 +292,7 @@ struct DevTbPlan {
 };
 
 // Rows between the checkpoints of a score plan with R rows per lane: a
-// multiple of R (checkpoints are bottom rows of lanes) of 40 to 64 rows,
+// multiple of R (checkpoints are bottom rows of lanes) of 50 to 64 rows,
 // doubled as often as the pool's size asks for.  Narrower blocks would have
 // narrower bands (a block's band allows for its own loss) but store more.
 __host__ __device__ inline int ck_block_rows(int R)
