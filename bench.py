@@ -1064,7 +1064,7 @@ def _fullmix_headline(args, rank: int, ws: int, pg, peak: dict, local: int) -> d
     # of a smaller full mix (every k_score launch of its last filtered call),
     # scaled by the pairs aligned (the kernel reads each aligned pair's
     # packed read and window once)
-    trec = _traffic_record(os.path.join(ROOT, "paper_1304_0681_gb300", "csrc", "sw_score.cu"),
+    trec = _traffic_record(os.path.join(ROOT, "paper_1304_0681_gb300", "csrc", "sw_score_kernel.cuh"),
                            "traffic_fullmix.json")
     traffic = trec["dram_bytes_per_step"] * aligned / trec["aligned_pairs"] if trec else None
     out = {"value": all_reads / total_s, "ms_per_step": total_s * 1e3 / args.steps, "clocks": clk,
@@ -1207,7 +1207,7 @@ def _throughput_section(args, rank: int, ws: int, pg, peak: dict, local: int, wo
     all_reads, _ = reduce_run(n_reads * steps, 0.0)
     score_ms = statistics.mean(p[1] for p in phases)
     achieved = cells / (score_ms * 1e-3) / 1e9
-    traffic = (_traffic_record(os.path.join(ROOT, "paper_1304_0681_gb300", "csrc", "sw_score.cu"))
+    traffic = (_traffic_record(os.path.join(ROOT, "paper_1304_0681_gb300", "csrc", "sw_score_kernel.cuh"))
                if workload == "throughput" and args.pairs is None else None)
     in_mb = (len(wl.packed_reads()) + len(wl.packed_windows())) / 1e6
     res = {"value": all_cells / total_s / 1e9, "unit": "GCUPS", "ms_per_step": total_s * 1e3 / steps,

@@ -123,7 +123,8 @@ int64_t sw_packed_bytes(int64_t n_bases);
  * batch is classified into length classes on the device, one-block planner
  * kernels size the launches there, and every compiled kernel variant runs
  * once as a persistent launch over the classes planned for it (launches with
- * nothing to do exit at once).  The host never waits for the device, so the
+ * nothing to do exit at once); a batch of at most 4,096 pairs without plan
+ * overrides takes six launches instead.  The host never waits for the device, so the
  * call can be captured into a CUDA graph, provided that an uncaptured call on
  * the same stream with at least as many pairs came first: the first call of
  * a size on a stream allocates the library's scratch for it, and a call that
@@ -561,10 +562,10 @@ int sw_set_plan(int32_t max_read_len, int32_t lanes, int32_t r_rows);
  * match x min(max_read_len, max_window_len) as for a pair, then the
  * overrides of sw_set_plan apply (an override with more than 32 rows is
  * skipped by a 16-bit-key class whose bound exceeds 510), else the built-in
- * cost model.  Without an override, a class whose pairs would give fewer
- * tasks than half the warps of its launch (a small batch) runs with fewer
- * rows per lane on more lanes; the query reports the plan before that
- * adjustment, which depends on the class's pair count.  Host-only;
+ * cost model.  Without an override, a class with too few tasks for its
+ * launch's warps runs with fewer rows per lane on more lanes; the query
+ * reports the plan before that adjustment, which depends on the batch's pair
+ * counts.  Host-only;
  * SW_ERR_INVALID_ARG for null outputs or values out of range.
  */
 int sw_plan_query(int32_t max_read_len, int32_t max_window_len, int32_t match, int32_t *lanes, int32_t *r_rows);

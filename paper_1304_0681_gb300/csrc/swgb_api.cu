@@ -1,10 +1,10 @@
 // swgb_api.cu -- host side of the C ABI declared in include/swgb.h.
 //
-// One call = classify (validate, sort pairs by length class) -> read back the
-// per-class counts -> per class: score pass, then (when a CIGAR is wanted)
-// traceback pass.  Scratch memory is owned by the library, cached per device
-// and grown on demand; calls on one device are serialised through an event so
-// that two calls never share scratch concurrently.
+// One call enqueues a fixed sequence and never waits for the device: classify
+// (validate, sort pairs by length class), plan, score pass, and when a CIGAR is
+// wanted the traceback's sort, plan and launches; batches of at most kSmallPairs
+// pairs take the few launches of sw_small.cu.  Scratch memory is owned by the
+// library, one set per device and stream, and grown on demand outside captures.
 #include <algorithm>
 #include <atomic>
 #include <cmath>

@@ -279,8 +279,9 @@ struct TbPartPlan {
 };
 
 // Traceback scratch of one launch: per-warp slots from var_slot_offset on
-// (words; the launches run one after another and each has everything the
-// row checkpoints leave).
+// (words).  The 16-bit launches run at once, each in its part of what the row
+// checkpoints leave; the int32 launches follow one after another, each with all
+// of it.
 struct DevTbPlan {
     int32_t var_n[N_TB_VARIANTS];
     int32_t var_warps[N_TB_VARIANTS];     // warps with a slot (the others exit)
