@@ -66,9 +66,9 @@ def test_long_reads_and_wide_windows():
     assert_parity(wl, run_gpu(wl, DEFAULT), DEFAULT)
 
 
-@pytest.mark.parametrize("n_pairs", [500, 12_000, 25_000, 45_000])
+@pytest.mark.parametrize("n_pairs", [500, 12_000, 45_000, 120_000, 400_000])
 def test_lanes_per_pair(n_pairs):
-    """8, 4, 2 and 1 lanes per two pairs (chosen by the batch's size)."""
+    """16, 8, 4, 2 and 1 lanes per two pairs (chosen by the batch's size)."""
     wl = synth.random_pairs(n_pairs, (30, 130), (20, 190), seed=n_pairs, alphabet=3)
     got = run_gpu(wl, DEFAULT)
     sample = np.random.default_rng(3).choice(n_pairs, 500, replace=False)
