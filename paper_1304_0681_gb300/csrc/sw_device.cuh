@@ -66,6 +66,15 @@ __device__ __forceinline__ KeyGroup key_group(int32_t key)
     return g;
 }
 
+// A converged warp moves on an index that it keeps in shared memory: one lane
+// stores (of lanes that store different values to one word, any may stay).
+__device__ __forceinline__ void next_index(volatile int32_t &index, int lane)
+{
+    __syncwarp();
+    if (lane == 0) index = index + 1;
+    __syncwarp();
+}
+
 // 64-bit best-cell key: larger H first, then smaller j, then smaller i.
 __device__ __forceinline__ uint64_t cell_key(uint32_t h, int32_t j, int32_t i)
 {

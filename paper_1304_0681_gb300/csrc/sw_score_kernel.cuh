@@ -323,7 +323,7 @@ __device__ __forceinline__ void score_body(const ScoreLaunch &L, const int varia
         cc->n_cls = planned ? L.dp->var_n[variant] : 1;
     }
     __syncwarp();
-    for (; cc->ci < cc->n_cls; __syncwarp(), cc->ci = cc->ci + (lane == 0 ? 1 : 0), __syncwarp()) {
+    for (; cc->ci < cc->n_cls; next_index(cc->ci, lane)) {
     const int ci = cc->ci;
     int T = L.lanes, cls = L.cls;
     const int32_t *order = L.order;

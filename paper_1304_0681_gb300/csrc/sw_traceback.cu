@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(128, 4) k_traceback16(const TracebackLaunch L)
     __syncwarp();
     if (lane == 0) pc->pi = 0;
     __syncwarp();
-    for (; pc->pi < dp.var_n[v]; __syncwarp(), pc->pi = pc->pi + (lane == 0 ? 1 : 0), __syncwarp()) {
+    for (; pc->pi < dp.var_n[v]; next_index(pc->pi, lane)) {
     if (lane == 0) {
         const TbPartPlan &pp = dp.part[dp.var_part[v][pc->pi]];
         const int32_t s4 = (pp.wcap + T - 1 + 3) >> 2;
