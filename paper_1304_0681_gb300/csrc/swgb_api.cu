@@ -32,7 +32,8 @@ namespace {
 
 constexpr int kThreads = 128;
 constexpr int kMaxDevices = 64;
-constexpr int kAuxStreams = 4;
+constexpr int kTbStreams = 4;                  // streams of the 16-bit traceback launches
+constexpr int kAuxStreams = kScoreStreams - 1; // beside the caller's
 constexpr int kHostChunks = 2;                 // sw_batch_align_host pipelines a batch in this many chunks
 constexpr int64_t kHostChunkMin = 65536;       // ... of at least this many pairs
 // Scratch budgets of a call, from its pair count (the only size the host
@@ -130,20 +131,22 @@ std::vector<PlanOverride> g_plans;
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Fork: the first n auxiliary streams wait for everything enqueued on st so
-// far.  Join: st waits for all of their work.  (The pattern is legal under
-// stream capture.)
+// Fork: work goes on over n streams, the caller's (number 0) and n - 1 auxiliary
+// ones, which wait for everything enqueued on st so far.  Join: st waits for all
+// of their work.  (The pattern is legal under stream capture.)
+cudaStream_t stream_at(const ExecCtx &x, cudaStream_t st, int k) { return k ? x.aux[k - 1] : st; }
+
 int fork_streams(const ExecCtx &x, cudaStream_t st, int n)
 {
     if (cuda_failed(cudaEventRecord(x.fork_ev, st))) return SW_ERR_CUDA;
-    for (int k = 0; k < n; ++k)
+    for (int k = 0; k < n - 1; ++k)
         if (cuda_failed(cudaStreamWaitEvent(x.aux[k], x.fork_ev, 0))) return SW_ERR_CUDA;
     return SW_OK;
 }
 
 int join_streams(const ExecCtx &x, cudaStream_t st, int n)
 {
-    for (int k = 0; k < n; ++k) {
+    for (int k = 0; k < n - 1; ++k) {
         if (cuda_failed(cudaEventRecord(x.join_ev[k], x.aux[k]))) return SW_ERR_CUDA;
         if (cuda_failed(cudaStreamWaitEvent(st, x.join_ev[k], 0))) return SW_ERR_CUDA;
     }
@@ -438,11 +441,11 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
         if (cuda_failed(cudaMemsetAsync(S.tb_keys, 0xFF, sizeof(int32_t) * n_pairs, st))) return SW_ERR_CUDA;
     }
     if (timing && cuda_failed(cudaEventRecord(x.phase[1], st))) return SW_ERR_CUDA;
-    if ((rc = fork_streams(x, st, kAuxStreams))) return rc;
+    if ((rc = fork_streams(x, st, kScoreStreams))) return rc;
     const ScoreLaunch L = score_launch(ps, sc, out_score, out_end, cig != nullptr, S);
-    for (int v = 0; v < N_SCORE_VARIANTS; ++v)
-        if ((rc = launch_score_variant(v, L, x.score_blocks[v], x.aux[v % kAuxStreams]))) return rc;
-    if ((rc = join_streams(x, st, kAuxStreams))) return rc;
+    for (int v = N_SCORE_VARIANTS - 1; v >= 0; --v)
+        if ((rc = launch_score_variant(v, L, x.score_blocks[v], stream_at(x, st, score_variant_stream(v))))) return rc;
+    if ((rc = join_streams(x, st, kScoreStreams))) return rc;
     if (timing && cuda_failed(cudaEventRecord(x.phase[2], st))) return SW_ERR_CUDA;
     if (cig) {
         if ((rc = launch_scan_scatter(S.tb_keys, n_pairs, S.info->count, S.hist, S.bstart, S.cursor, S.tb_order,
@@ -454,11 +457,11 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
         // the 16-bit launches at once, each in its part of the scratch, those
         // with the longest tasks first; then the int32 launches, each with
         // all of it
-        if ((rc = fork_streams(x, st, kAuxStreams))) return rc;
+        if ((rc = fork_streams(x, st, kTbStreams))) return rc;
         int k = 0;
         for (int v = 0; v < N_TB16_VARIANTS; v += tb_launch_variants(v), ++k)
-            if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], x.aux[k % kAuxStreams]))) return rc;
-        if ((rc = join_streams(x, st, kAuxStreams))) return rc;
+            if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], stream_at(x, st, k % kTbStreams)))) return rc;
+        if ((rc = join_streams(x, st, kTbStreams))) return rc;
         for (int v = N_TB16_VARIANTS; v < N_TB_VARIANTS; ++v)
             if ((rc = launch_traceback_variant(v, fma, B, x.tb_blocks[v], st))) return rc;
     }

@@ -193,6 +193,21 @@ constexpr int N_TB16_VARIANTS = 7;                        // 16-bit traceback: T
 constexpr int TB_VAR_TILED = 7;                           // int32 traceback, one lane per pair, warp tiles
 constexpr int TB_VAR_GROUPED = 8;                         // int32 traceback, T lanes per pair
 constexpr int N_TB_VARIANTS = 9;
+// The score launches of the general sequence fork over kScoreStreams streams,
+// the most rows first (they serve the longest reads).  The row counts of a mode
+// that a batch's longer reads take (25, 32 and 50) go to streams of their own, the
+// wide modes' apart from the others': launches on one stream wait for one
+// another, and a few long reads keep a launch busy for milliseconds.  Calls
+// without a CIGAR, with every row count of a mode on one of four streams, and so:
+// 200 reads of 1,000 to 4,000 bases 15.5 and 6.6 ms, 5,000 of 750 to 3,000 24.3
+// and 12.5, 20,000 of 75 to 800 0.95 and 0.81.  (Where the last tasks fall decides
+// a few batches the other way: 34,000 pairs of 4,000 such reads 0.90 and 1.12 ms.)
+constexpr int kScoreStreams = 8;
+inline int score_variant_stream(int v)
+{
+    const int rows = v / N_VMODES, mode = v % N_VMODES;
+    return (rows + (mode == MODE_I16S)) % 4 + (mode >= MODE_I16W ? 4 : 0);
+}
 __host__ __device__ inline int tb16_variant_lanes(int v) { return v < 2 ? 16 : v < 4 ? 8 : 64 >> v; }
 // Rows per lane of the 16-bit kernel: with 16 lanes per two pairs, taken where
 // there are too few pairs to fill the GPU, four -- a lone warp's step then

@@ -1,0 +1,41 @@
+"""Which stream each score launch of the general sequence goes to: launches on
+one stream run one after another, so the row counts that the long reads of a
+batch take must not share one (score_variant_stream in swgb_internal.h)."""
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SRC = r"""
+#include <cstdio>
+#include "swgb_internal.h"
+using namespace swgb;
+int main()
+{
+    int used[kScoreStreams] = {};
+    for (int mode = 0; mode < N_VMODES; ++mode)
+        for (int a = 0; a < N_SCORE_ROWS; ++a) {
+            const int s = score_variant_stream(a * N_VMODES + mode);
+            if (s < 0 || s >= kScoreStreams) { printf("stream %d\n", s); return 1; }
+            ++used[s];
+            for (int b = a + 1; b < N_SCORE_ROWS && b < a + 4; ++b)
+                if (s == score_variant_stream(b * N_VMODES + mode)) {
+                    printf("mode %d: %d and %d rows on stream %d\n", mode, score_rows_at(a), score_rows_at(b), s);
+                    return 1;
+                }
+        }
+    for (int s = 0; s < kScoreStreams; ++s)
+        if (!used[s]) { printf("stream %d is not used\n", s); return 1; }
+    return 0;
+}
+"""
+
+
+def test_long_reads_row_counts_run_side_by_side(tmp_path):
+    src = tmp_path / "streams.cpp"
+    src.write_text(SRC)
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-I", os.path.join(ROOT, "paper_1304_0681_gb300", "csrc"),
+                           "-I", os.path.join(ROOT, "include"), "-I", "/usr/local/cuda/include", str(src), "-o",
+                           str(tmp_path / "streams")])
+    r = subprocess.run([str(tmp_path / "streams")], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
