@@ -55,9 +55,9 @@ __device__ __forceinline__ bool plan_class(const PlanParams &pp, int mode, int32
     vmode = score_vmode(mode, hmax, pp.sc);
     for (int i = 0; i < pp.n_overrides; ++i)
         if (mm <= pp.ov[i].max_read_len) return true;
-    if (pp.small && !small_rows(ri)) {
-        // a small batch's one launch holds every other row count: the next
-        // larger one (its lanes then cover the read in no more chunks)
+    if (pp.small && !small_body(ri, vmode)) {
+        // not in a small batch's one launch: the next larger row count (its
+        // lanes then cover the read in no more chunks)
         ++ri;
         lanes = min(32, (mm + score_rows_at(ri) - 1) / score_rows_at(ri));
     }

@@ -1,7 +1,8 @@
 // sw_score_any.cu -- the score pass of a small batch in one launch: the bodies
-// of four row counts in every mode, run for the variants that have classes.
-// (255 registers, so 8 warps per SM whatever runs: a small batch has no more
-// tasks than that.)
+// that small_body() lists, run for the variants that have classes.  255 registers,
+// so 8 warps per SM whatever runs.  Most small batches have no more tasks; one
+// with more (thousands of long reads, up to 2,048 tasks of a warp) takes the plans
+// with the fewest steps, of 20 rows or more, whose own launches hold 8 to 12.
 #include "sw_score_kernel.cuh"
 
 namespace swgb {
@@ -9,11 +10,15 @@ namespace swgb {
 template <int R, bool FMA_ADD>
 __device__ __forceinline__ void score_rows_any(const ScoreLaunch &L, int v)
 {
+    if constexpr (R == 20 || R == 32) {
+        score_body<R, MODE_I16W, FMA_ADD, true>(L, v);
+        return;
+    }
     switch (v % N_VMODES) {
     case MODE_I32: score_body<R, MODE_I32, true, false>(L, v); break;
     case MODE_I16: score_body<R, MODE_I16, FMA_ADD, true>(L, v); break;
     case MODE_I16W:
-        if constexpr (R < 50) {
+        if constexpr (R == 8 || R == 16 || R == 25) {  // pipe_rows_idx
             score_body<R, MODE_I16W, FMA_ADD, true, SCORE_WARP_TASKS>(L, v);
             __syncthreads();
             score_body<R, MODE_I16W, FMA_ADD, true, SCORE_BLOCK_TASKS>(L, v);
@@ -38,7 +43,9 @@ __global__ void __launch_bounds__(128) k_score_any(const __grid_constant__ Score
         switch (v / N_VMODES) {
         case 0: score_rows_any<8, FMA_ADD>(L, v); break;
         case 1: score_rows_any<16, FMA_ADD>(L, v); break;
+        case 2: score_rows_any<20, FMA_ADD>(L, v); break;
         case 3: score_rows_any<25, FMA_ADD>(L, v); break;
+        case 4: score_rows_any<32, FMA_ADD>(L, v); break;
         case 5: score_rows_any<50, FMA_ADD>(L, v); break;
         default: break;
         }

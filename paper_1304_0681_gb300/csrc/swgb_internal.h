@@ -234,8 +234,14 @@ constexpr int kPlanThreads = 384;                         // >= N_CLASS
 // Batches of up to this many pairs (without plan overrides) take the few
 // launches of sw_small.cu.
 constexpr int kSmallPairs = 4096;
-// Row counts in the one score launch of a small batch (8, 16, 25, 50).
+// Row counts that a small batch steps down through (8, 16, 25, 50), and the bodies
+// in its one score launch: those, and the wide mode's 20 and 32 rows, the plans of
+// most reads of 500 to 640, 800 to 1,024 and 1,600 to 2,048 bases.  (With 25 and
+// 50 rows in their place 4,096 reads of 1,000 bases took 2.15 ms without a CIGAR,
+// of 2,000 bases 8.1 ms; so 1.52 and 5.3.  In the int32 mode 50 rows are the
+// faster: 300 reads of 7,000 bases 39.0 ms, 42.6 with 32.)
 __host__ __device__ inline bool small_rows(int rows_idx) { return rows_idx != 2 && rows_idx != 4; }
+__host__ __device__ inline bool small_body(int rows_idx, int vmode) { return small_rows(rows_idx) || vmode == MODE_I16W; }
 
 // Block tasks.  A long read's two pairs in one warp take a row chunk after
 // another, and a few of them leave the SMs empty: 200 reads of 1000 to 4000

@@ -41,6 +41,17 @@ def test_both_sides_of_the_limit(n, cigar):
     assert_parity(wl, got, DEFAULT, pairs=pick, cigar=cigar)
 
 
+@pytest.mark.parametrize("m", [513, 601, 640, 801, 1000, 1024, 1601, 2048])
+def test_plans_of_20_and_32_rows(m):
+    """Reads whose plan has 20 or 32 rows per lane, in one row chunk and in two,
+    in a small batch of too many pairs for block tasks."""
+    wl = synth.random_pairs(700, (m - 20, m), (m - 10, m + 90), seed=m, alphabet=3)
+    for cigar in (False, True):
+        got = run_gpu(wl, DEFAULT, cigar=cigar)
+        pick = np.sort(np.random.default_rng(m).choice(wl.n_pairs, 40, replace=False))
+        assert_parity(wl, got, DEFAULT, pairs=pick, cigar=cigar)
+
+
 @pytest.mark.parametrize("n", [300, 6000])
 def test_masked_and_empty_pairs(n):
     """Unselected pairs and empty windows are finished by the classification

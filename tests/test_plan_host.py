@@ -57,6 +57,11 @@ int main()
     PlanOverride ov3[1] = {{100, 2, 50}};
     score_plan_of(MODE_I16, 100, 1000, ov3, 1, l, r);
     if (l == 2 && score_rows_at(r) == 50) { printf("override 3 taken\n"); ++bad; }
+    // a small batch's one launch holds the plan of every read that runs in the wide mode
+    for (int m = 103; m <= 6400; ++m) {
+        score_plan_of(MODE_I16W, m, 5L * m, nullptr, 0, l, r);
+        if (!small_body(r, MODE_I16W)) { if (bad++ < 5) printf("no small body of %d rows (m=%d)\n", score_rows_at(r), m); }
+    }
     printf("mismatches %d\n", bad);
     return bad != 0;
 }
