@@ -52,7 +52,7 @@ __device__ __forceinline__ bool plan_class(const PlanParams &pp, int mode, int32
 {
     const int64_t hmax = (int64_t)pp.sc.ma * min(mm, mn);
     score_plan_of(mode, mm, hmax, pp.ov, pp.n_overrides, lanes, ri);
-    vmode = score_vmode(mode, hmax, pp.sc);
+    vmode = score_vmode(mode, hmax, pp.sc, mm > lanes * score_rows_at(ri));
     for (int i = 0; i < pp.n_overrides; ++i)
         if (mm <= pp.ov[i].max_read_len) return true;
     if (pp.small && !small_body(ri, vmode)) {

@@ -572,7 +572,7 @@ void plan_budgets(const ClassInfo &ci, const PlanParams &pp, bool cigar, int64_t
         score_plan_of(mode, mm, (int64_t)pp.sc.ma * std::min(mm, mn), pp.ov, pp.n_overrides, lanes, ri);
         const int rows = score_rows_at(ri);
         if ((mm + lanes * rows - 1) / (lanes * rows) > 1) {
-            const int v = ri * N_VMODES + score_vmode(mode, (int64_t)pp.sc.ma * std::min(mm, mn), pp.sc);
+            const int v = ri * N_VMODES + score_vmode(mode, (int64_t)pp.sc.ma * std::min(mm, mn), pp.sc, true);
             slot_s[v] = std::max<int64_t>(slot_s[v], (int64_t)(32 / lanes) * 16 * mn);
         }
     }

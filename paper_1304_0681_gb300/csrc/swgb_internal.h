@@ -362,10 +362,13 @@ __host__ __device__ inline int score_mode_for(int64_t hmax, int setting)
 // largest value is the score bound hmax less gap_open.
 __host__ __device__ inline bool half_exact(int64_t hmax, const Scoring &sc) { return hmax - sc.go <= 2047; }
 
-// The kernel mode of a class of `mode` with score bound hmax.
-__host__ __device__ inline int score_vmode(int mode, int64_t hmax, const Scoring &sc)
+// The kernel mode of a class of `mode` with score bound hmax.  Reads in several
+// row chunks stay in the class's mode: the variants that need boundary rows each
+// take an equal part of that scratch, and one more would leave the others too
+// little for the longest windows.
+__host__ __device__ inline int score_vmode(int mode, int64_t hmax, const Scoring &sc, bool chunked)
 {
-    return mode == MODE_I16W && half_exact(hmax, sc) ? (int)MODE_I16S : mode;
+    return mode == MODE_I16W && !chunked && half_exact(hmax, sc) ? (int)MODE_I16S : mode;
 }
 
 // Score-pass plan of a length class: lanes per group and rows per lane

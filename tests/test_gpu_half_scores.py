@@ -41,3 +41,35 @@ def test_bounds_of_the_fp16_add(scoring, cigar):
             wins.append(w[:max(1, m - 1)])
     wl = _batch(reads, wins)
     assert_parity(wl, run_gpu(wl, scoring, cigar=cigar), scoring, cigar=cigar)
+
+
+def test_long_reads_of_three_modes_share_the_boundary_scratch():
+    """A 1,700-base read on a short window has scores the fp16 add could take,
+    but runs in row chunks: a launch of its own would take a third part of the
+    boundary rows' scratch, and the rows of the two 700,000-base windows, at
+    most half of it each, would no longer fit theirs."""
+    import torch
+    from paper_1304_0681_gb300 import DeviceBatch, _swgb, align
+    rng = np.random.default_rng(31)
+    reads = [rng.integers(0, 4, 40).astype(np.uint8) for _ in range(4100)]
+    wins = [rng.integers(0, 4, 60).astype(np.uint8) for _ in range(4100)]
+    r = rng.integers(0, 4, 1700).astype(np.uint8)
+    reads.append(r)
+    wins.append(r[200:500].copy())
+    for m in (2000, 6500):     # 16-bit cells and 32-bit cells; the read's copy starts at column 1000
+        r = rng.integers(0, 4, m).astype(np.uint8)
+        w = rng.integers(0, 4, 700_000).astype(np.uint8)
+        w[1000:1000 + m] = r
+        reads.append(r)
+        wins.append(w)
+    wl = _batch(reads, wins)
+    b = DeviceBatch.from_packed(wl.packed_reads(), wl.read_offsets, wl.packed_windows(), wl.window_offsets, cigar=False)
+    align(b, (5, -4, -10, -1), cigar=False)
+    _swgb.sw_sync_status()
+    end = b.end.cpu().numpy().reshape(-1, 2).astype(np.int64)
+    score = b.score.cpu().numpy().astype(np.int64)
+    torch.cuda.synchronize()
+    assert score[-2:].tolist() == [5 * 2000, 5 * 6500]
+    assert end[-2:].tolist() == [[1999, 2999], [6499, 7499]]
+    assert_parity(wl, {"score": score, "i_end": end[:, 0], "j_end": end[:, 1]}, (5, -4, -10, -1),
+                  pairs=np.arange(4000, 4101), cigar=False)
