@@ -142,12 +142,12 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
         s_slots = 0;
     }
     __syncthreads();
-    auto long_class = [&](int c) { return pp.small && c >= N_MCLASS && info->max_m[c] > kPipeMinRead; };
+    auto long_class = [&](int c) { return pp.small && block_task_class(c, info->max_m[c]); };
     auto mean_n = [&](int c) { return (int32_t)__fdividef((float)info->sum_n[c], (float)info->count[c]); };
     for (int c = threadIdx.x; c < N_CLASS; c += blockDim.x) {
         const int32_t cnt = info->count[c];
         if (cnt == 0) continue;
-        if (long_class(c)) atomicAdd(&s_pipe_tasks, (cnt + 1) / 2);
+        if (long_class(c)) atomicAdd(&s_pipe_tasks, (int32_t)block_task_tasks(cnt));
         const int mode = c / N_MCLASS;
         int lanes = 1, ri = 0, vmode = 0;
         const bool fixed = plan_class(pp, mode, info->max_m[c], info->max_n[c], lanes, ri, vmode);
@@ -167,10 +167,9 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
             const int mode = c / N_MCLASS;
             const int32_t mm = info->max_m[c], mn = info->max_n[c];
             int ri = 0, vmode = mode;
-            // per group: two buffers x longest window x (H, F) x 4 bytes
             int64_t pipe = -1;
             if (long_class(c) && s_pipe_tasks <= pp.score_warps[0] / kPipeWarps) {
-                const unsigned long long need = 16ull * mn * ((cnt + 1) / 2);
+                const unsigned long long need = (unsigned long long)block_task_need(cnt, mn);
                 const unsigned long long at = atomicAdd(&s_pipe_bytes, need);
                 if (at + need <= (unsigned long long)pp.pipe_bytes) pipe = (int64_t)at;
             }
@@ -189,6 +188,7 @@ __device__ __forceinline__ void plan_score(const ClassInfo *info, const PlanPara
             }
             const int rows = score_rows_at(ri);
             const int chunks = (mm + lanes * rows - 1) / (lanes * rows);
+            // per group: two buffers x longest window x (H, F) x 4 bytes
             bnd = chunks > 1 && pipe < 0 ? 16 * mn : 0;
             var = ri * N_VMODES + vmode;
             if (pp.ck_bytes > 0 && mode != MODE_I32) ck = ck_block_rows(rows);

@@ -105,6 +105,8 @@ struct DeviceState {
     ExecCtx x;                       // grids, auxiliary streams, fork and join events
     int64_t tb_cap = 0;              // largest traceback budget (set at the first traceback)
     Buffer fixed, dyn;
+    Buffer pipe;             // boundary rows of small batches' block tasks
+    bool pipe_tried = false;
     Buffer stage;            // sw_batch_align_host device staging
     int32_t *last_status = nullptr;  // device status word of the last call
     const DevTbPlan *last_tplan = nullptr;  // traceback plan of the last call with a CIGAR
@@ -163,7 +165,7 @@ bool capturing(cudaStream_t st)
     return cs != cudaStreamCaptureStatusNone;
 }
 
-int ensure(Buffer &b, size_t bytes)
+int ensure(Buffer &b, size_t bytes, bool slack = true)
 {
     if (b.bytes >= bytes) return SW_OK;
     // pending work may still use the old buffer
@@ -171,7 +173,7 @@ int ensure(Buffer &b, size_t bytes)
     if (b.ptr) cudaFree(b.ptr);
     b.ptr = nullptr;
     b.bytes = 0;
-    const size_t want = align_up(bytes + std::min<size_t>(bytes / 4, (size_t)256 << 20), 1 << 20);
+    const size_t want = align_up(bytes + (slack ? std::min<size_t>(bytes / 4, (size_t)256 << 20) : 0), 1 << 20);
     if (cuda_failed(cudaMalloc(&b.ptr, want))) {
         cudaGetLastError();
         return SW_ERR_CUDA;
@@ -229,7 +231,7 @@ int device_state(DeviceState **out, cudaStream_t st)
 
 void free_state(DeviceState *s)
 {
-    for (Buffer *b : {&s->fixed, &s->dyn, &s->stage, &s->misc, &s->filt, &s->grad})
+    for (Buffer *b : {&s->fixed, &s->dyn, &s->pipe, &s->stage, &s->misc, &s->filt, &s->grad})
         if (b->ptr) {
             cudaFree(b->ptr);
             b->ptr = nullptr;
@@ -279,7 +281,8 @@ struct Scratch {
     TbClassInfo *tbinfo;
     DevScorePlan *splan;
     DevTbPlan *tplan;
-    uint8_t *pipe;  // boundary rows of a small batch's block tasks
+    uint8_t *pipe;  // boundary rows of a small batch's block tasks (0 bytes: it runs without them)
+    int64_t pipe_bytes;
     uint8_t *score_bnd;
     int64_t score_bnd_bytes;
     uint32_t *tb;
@@ -288,7 +291,7 @@ struct Scratch {
 
 // Lays out the pair-count-sized part at base (nullptr: sizes only); returns
 // its bytes.
-size_t fixed_layout(int64_t n_pairs, int64_t pipe_bytes, uint8_t *base, Scratch &S)
+size_t fixed_layout(int64_t n_pairs, uint8_t *base, Scratch &S)
 {
     const size_t nh = (size_t)N_CLASS * N_NBUCKET;
     size_t off = 0;
@@ -311,8 +314,13 @@ size_t fixed_layout(int64_t n_pairs, int64_t pipe_bytes, uint8_t *base, Scratch 
     S.expect = (int32_t *)take(sizeof(int32_t) * 3 * N_CLASS);
     S.splan = (DevScorePlan *)take(sizeof(DevScorePlan));
     S.tplan = (DevTbPlan *)take(sizeof(DevTbPlan));
-    S.pipe = take(pipe_bytes);
     return off;
+}
+
+bool plan_overrides()
+{
+    std::lock_guard<std::mutex> lk(g_plan_mu);
+    return !g_plans.empty();
 }
 
 PlanParams plan_params(const ExecCtx &x, const Scoring &sc, bool allow16, int64_t score_bnd_bytes,
@@ -382,7 +390,7 @@ int enqueue_small(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Sco
     int rc = SW_OK;
     const bool timing = x.timing && x.phase;
     pp.small = 1;
-    pp.pipe_bytes = kPipeBytes;
+    pp.pipe_bytes = S.pipe_bytes;
     for (int v = 0; v < N_SCORE_VARIANTS; ++v) pp.score_warps[v] = x.any_blocks * (kThreads / 32);
     auto blocks = [&](int full) { return (int)std::min<int64_t>(full, n_pairs); };
     if (timing && cuda_failed(cudaEventRecord(x.phase[0], st))) return SW_ERR_CUDA;
@@ -478,9 +486,7 @@ int run_batch(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const sw_scor
     std::lock_guard<std::mutex> lk(ds->mu);
     const Scoring sc{scoring->match, scoring->mismatch, scoring->gap_open, scoring->gap_extend};
     Scratch S{};
-    // (the block tasks' rows are taken for every size: a small call captured on
-    // a stream of larger ones finds them there)
-    const size_t fixed_bytes = fixed_layout(n_pairs, kPipeBytes, nullptr, S);
+    const size_t fixed_bytes = fixed_layout(n_pairs, nullptr, S);
     const int64_t bnd_bytes = std::min(kScoreBndMax, std::max(kScoreBndMin, n_pairs * kScoreBndPerPair));
     int64_t tb_bytes = 0;
     if (cig) {
@@ -495,7 +501,15 @@ int run_batch(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const sw_scor
     }
     if ((rc = ensure_on(ds->fixed, fixed_bytes, st))) return rc;
     if ((rc = ensure_on(ds->dyn, (size_t)(bnd_bytes + tb_bytes), st))) return rc;
-    fixed_layout(n_pairs, kPipeBytes, (uint8_t *)ds->fixed.ptr, S);
+    // the block tasks' rows, with the stream's first small batch (one that is
+    // captured before, or that finds the card full, runs without block tasks)
+    if (n_pairs <= kSmallPairs && !ds->pipe_tried && !plan_overrides() && !capturing(st)) {
+        ds->pipe_tried = true;
+        ensure(ds->pipe, kPipeBytes, false);
+    }
+    fixed_layout(n_pairs, (uint8_t *)ds->fixed.ptr, S);
+    S.pipe = (uint8_t *)ds->pipe.ptr;
+    S.pipe_bytes = (int64_t)ds->pipe.bytes;
     S.score_bnd = (uint8_t *)ds->dyn.ptr;
     S.score_bnd_bytes = bnd_bytes;
     S.tb = (uint32_t *)((uint8_t *)ds->dyn.ptr + bnd_bytes);
@@ -550,7 +564,7 @@ struct sw_plan {
     bool cigar = false;
     int score_setting = SW_SCORE_AUTO;  // the score mode setting at creation
     bool allow16 = true;      // the traceback mode setting at creation
-    swgb::Buffer fixed, dyn;  // owned: a captured graph keeps pointing here
+    swgb::Buffer fixed, dyn, pipe;  // owned: a captured graph keeps pointing here
     swgb::Scratch S{};
     swgb::ExecCtx x;          // owned auxiliary streams and events (a capture creates nothing)
 };
@@ -627,9 +641,8 @@ int plan_build(sw_plan *pl, DeviceState *ds, cudaStream_t st)
     int rc = SW_OK;
     const int64_t n_pairs = pl->n_pairs;
     Scratch &S = pl->S;
-    const int64_t pipe_bytes = n_pairs <= kSmallPairs ? kPipeBytes : 0;
-    if ((rc = ensure(pl->fixed, fixed_layout(n_pairs, pipe_bytes, nullptr, S)))) return rc;
-    fixed_layout(n_pairs, pipe_bytes, (uint8_t *)pl->fixed.ptr, S);
+    if ((rc = ensure(pl->fixed, fixed_layout(n_pairs, nullptr, S)))) return rc;
+    fixed_layout(n_pairs, (uint8_t *)pl->fixed.ptr, S);
     // classify once (it reads offsets only) and read the class table back
     const size_t nh = (size_t)N_CLASS * N_NBUCKET;
     if (cuda_failed(cudaMemsetAsync(S.hist, 0, sizeof(int32_t) * nh, st))) return SW_ERR_CUDA;
@@ -658,6 +671,10 @@ int plan_build(sw_plan *pl, DeviceState *ds, cudaStream_t st)
     int64_t bnd_bytes = 0, tb_bytes = 0;
     plan_budgets(ci, pp, pl->cigar, bnd_bytes, tb_bytes);
     if ((rc = ensure(pl->dyn, (size_t)(bnd_bytes + tb_bytes)))) return rc;
+    const int64_t pipe_bytes = n_pairs <= kSmallPairs ? block_task_bytes(ci, pl->x.any_blocks) : 0;
+    if (pipe_bytes && (rc = ensure(pl->pipe, (size_t)pipe_bytes, false))) return rc;
+    S.pipe = (uint8_t *)pl->pipe.ptr;
+    S.pipe_bytes = pipe_bytes;
     S.score_bnd = (uint8_t *)pl->dyn.ptr;
     S.score_bnd_bytes = bnd_bytes;
     S.tb = (uint32_t *)((uint8_t *)pl->dyn.ptr + bnd_bytes);
@@ -1065,6 +1082,7 @@ int sw_plan_destroy(sw_plan_t *plan)
     cudaDeviceSynchronize();
     if (plan->fixed.ptr) cudaFree(plan->fixed.ptr);
     if (plan->dyn.ptr) cudaFree(plan->dyn.ptr);
+    if (plan->pipe.ptr) cudaFree(plan->pipe.ptr);
     exec_ctx_free(plan->x);
     if (prev >= 0) cudaSetDevice(prev);
     delete plan;

@@ -245,12 +245,29 @@ __host__ __device__ inline bool small_body(int rows_idx, int vmode) { return sma
 
 // Block tasks.  A long read's two pairs in one warp take a row chunk after
 // another, and a few of them leave the SMs empty: 200 reads of 1000 to 4000
-// bases took 8.9 ms.  While there are at most kPipeTasks such tasks the four
-// warps of a block take a task's chunks side by side, each one wavefront
-// behind the other, with as few rows per lane as keep it at four chunks.
-// Classes of reads of up to 256 bases (one chunk of the fewest rows) never do.
+// bases took 8.9 ms.  While a small batch has no more such tasks than its score
+// launch has blocks, the four warps of a block take a task's chunks side by side,
+// each one wavefront behind the other, with as few rows per lane as keep it at
+// four chunks, 25 at most (reads over 3200 bases take more chunks).  Reads of up
+// to 512 bases never do: up to there one warp takes the read in one chunk of 16
+// rows or fewer.  The boundary rows of all tasks (two buffers of two values a
+// column) have kPipeBytes; a class that finds no room runs as warp tasks.
 constexpr int kPipeMinRead = 512, kPipeWarps = 4;
 constexpr int64_t kPipeBytes = (int64_t)64 << 20;
+__host__ __device__ inline bool block_task_class(int c, int32_t m_max) { return c >= N_MCLASS && m_max > kPipeMinRead; }
+__host__ __device__ inline int64_t block_task_tasks(int32_t cnt) { return (cnt + 1) / 2; }
+__host__ __device__ inline int64_t block_task_need(int32_t cnt, int32_t n_max) { return 16 * (int64_t)n_max * block_task_tasks(cnt); }
+// Bytes of boundary rows that the block tasks of a batch take at most.
+inline int64_t block_task_bytes(const ClassInfo &ci, int blocks)
+{
+    int64_t tasks = 0, bytes = 0;
+    for (int c = 0; c < N_CLASS; ++c)
+        if (ci.count[c] && block_task_class(c, ci.max_m[c])) {
+            tasks += block_task_tasks(ci.count[c]);
+            bytes += block_task_need(ci.count[c], ci.max_n[c]);
+        }
+    return tasks > blocks ? 0 : bytes < kPipeBytes ? bytes : kPipeBytes;
+}
 __host__ __device__ inline int pipe_rows_idx(int32_t m_max)
 {
     return m_max <= kPipeWarps * 32 * 8 ? 0 : m_max <= kPipeWarps * 32 * 16 ? 1 : 3;  // 8, 16, 25 rows

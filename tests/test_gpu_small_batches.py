@@ -108,3 +108,42 @@ def test_a_small_plan_checks_its_shape_and_replays():
     with pytest.raises(SwError):
         plan.status()
     plan.close()
+
+
+def test_block_tasks_rows_come_with_the_first_small_batch():
+    """A stream of larger batches holds no boundary rows of block tasks (64 MB);
+    a small batch captured there runs without them, and the first one outside a
+    capture brings them."""
+    import torch
+    from paper_1304_0681_gb300 import DeviceBatch, align
+    s = torch.cuda.Stream()
+
+    def batch(wl, cigar):
+        return DeviceBatch.from_packed(wl.packed_reads(), wl.read_offsets, wl.packed_windows(), wl.window_offsets,
+                                       cigar=cigar)
+
+    large = batch(synth.random_pairs(5000, (90, 100), (150, 160), seed=1), False)
+    wl = synth.random_pairs(24, (600, 2000), (700, 2100), seed=3, alphabet=3)
+    small = batch(wl, False)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    align(large, DEFAULT, cigar=False, stream=s)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 100 << 20
+
+    def check(run):
+        small.score.fill_(-7)
+        small.end.fill_(-7)
+        torch.cuda.synchronize()
+        run()
+        torch.cuda.synchronize()
+        end = small.end.cpu().numpy().reshape(-1, 2).astype(np.int64)
+        got = {"score": small.score.cpu().numpy().astype(np.int64), "i_end": end[:, 0], "j_end": end[:, 1]}
+        assert_parity(wl, got, DEFAULT, cigar=False)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=s):
+        align(small, DEFAULT, cigar=False, stream=s, sync=False)
+    check(graph.replay)
+    check(lambda: align(small, DEFAULT, cigar=False, stream=s))
+    check(graph.replay)
