@@ -405,9 +405,10 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
             }
         }
         if (lane >= N_TB16_VARIANTS && lane < N_TB_VARIANTS) {
-            // int32: as many warps as fit all of the scratch
-            w = n ? min((int64_t)pp.tb_warps[lane], total / max(words, (int64_t)1)) : 0;
-            at = 0;
+            // int32: as many warps as fit all of the scratch (the checkpoints
+            // have been read by then)
+            w = n ? min((int64_t)pp.tb_warps[lane], pp.tb_bytes / 4 / max(words, (int64_t)1)) : 0;
+            at = -ck_words;
             if (n && w < 1) atomicOr(status, ST_UNSUPPORTED);  // one warp's slot does not fit the scratch
         }
         if (lane == 0) {

@@ -87,3 +87,29 @@ def test_block_doubling_when_the_pool_is_small():
         pairs.append((r, np.where(flip, (w + rng.integers(1, 4, len(w))) & 3, w).astype(np.uint8)))
     wl = _batch(pairs)
     assert_parity(wl, run_gpu(wl, DEFAULT), DEFAULT, pairs=np.arange(0, 40, 8))
+
+
+def test_32_bit_pairs_have_all_of_the_scratch():
+    """An 8,192-base read that matches with its last 200 bases only: its band
+    takes most of a small batch's scratch, which the row checkpoints of the other
+    pairs fill before.  Both fit, one after the other."""
+    from paper_1304_0681_gb300 import DeviceBatch, _swgb, align
+    rng = np.random.default_rng(20)
+    r = rng.integers(0, 4, 8192).astype(np.uint8)
+    w = np.concatenate([rng.integers(0, 4, 45_000).astype(np.uint8), r[-200:]])
+    pairs = [(r, w)]
+    for _ in range(70):
+        r = rng.integers(0, 4, 6000).astype(np.uint8)
+        pairs.append((r, np.concatenate([rng.integers(0, 4, 8000).astype(np.uint8), r])))
+    got = []
+    for wl in (_batch(pairs[:1]), _batch(pairs)):
+        b = DeviceBatch.from_packed(wl.packed_reads(), wl.read_offsets, wl.packed_windows(), wl.window_offsets)
+        align(b, DEFAULT)
+        _swgb.sw_sync_status()
+        n = b.cigar_n.cpu().numpy()
+        got.append((int(b.score[0]), b.end[:2].tolist(), b.cigar_ops[:n[0]].tolist()))
+        score, ops = b.score.cpu().numpy(), b.cigar_ops.cpu().numpy().view(np.uint32)
+    assert got[0] == got[1] and got[0][0] >= 1000
+    # the others: exact copies, one run of 6,000 bases
+    assert (score[1:] == 30_000).all() and (n[1:] == 1).all()
+    assert (ops[b.cigar_offsets.cpu().numpy()[1:-1]] == 6000 << 4).all()
