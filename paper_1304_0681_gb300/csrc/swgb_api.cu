@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "sw_device.cuh"
+#include "sw_budgets.h"
 #include "swgb_internal.h"
 #include "swgb_seed.h"
 
@@ -36,18 +37,10 @@ constexpr int kTbStreams = 4;                  // streams of the 16-bit tracebac
 constexpr int kAuxStreams = kScoreStreams - 1; // beside the caller's
 constexpr int kHostChunks = 2;                 // sw_batch_align_host pipelines a batch in this many chunks
 constexpr int64_t kHostChunkMin = 65536;       // ... of at least this many pairs
-// Scratch budgets of a call, from its pair count (the only size the host
-// knows without reading the device): chunk-boundary rows of the score pass,
-// and the per-warp slots of the traceback.  A warp's slot is sized on the
-// device for its launch's largest part; launches use as many warps as fit.
-constexpr int64_t kScoreBndMin = (int64_t)32 << 20, kScoreBndMax = (int64_t)1 << 30, kScoreBndPerPair = 1024;
-constexpr int64_t kTbMin = (int64_t)256 << 20, kTbPerPair = (int64_t)160 << 10;
-constexpr int64_t kTbCapMax = (int64_t)16 << 30, kTbCapMin = (int64_t)1 << 30;
-constexpr double kTbFreeShare = 0.3;
-
 struct Buffer {
     void *ptr = nullptr;
     size_t bytes = 0;
+    size_t refused = 0;  // the size asked for when it got less (the card had no more)
 };
 
 // What an execution needs besides scratch: the full-occupancy grid of every
@@ -165,30 +158,40 @@ bool capturing(cudaStream_t st)
     return cs != cudaStreamCaptureStatusNone;
 }
 
-int ensure(Buffer &b, size_t bytes, bool slack = true)
+// least: on a card that has no more, this many bytes or more will do (0: it has
+// to be all of them).
+int ensure(Buffer &b, size_t bytes, bool slack = true, size_t least = 0)
 {
     if (b.bytes >= bytes) return SW_OK;
     // pending work may still use the old buffer
     if (cuda_failed(cudaDeviceSynchronize())) return SW_ERR_CUDA;
     if (b.ptr) cudaFree(b.ptr);
-    b.ptr = nullptr;
-    b.bytes = 0;
-    const size_t want = align_up(bytes + (slack ? std::min<size_t>(bytes / 4, (size_t)256 << 20) : 0), 1 << 20);
-    if (cuda_failed(cudaMalloc(&b.ptr, want))) {
-        cudaGetLastError();
-        return SW_ERR_CUDA;
-    }
-    b.bytes = want;
+    b = Buffer{};
+    auto take = [&](size_t want) {
+        if (cuda_failed(cudaMalloc(&b.ptr, want))) {
+            cudaGetLastError();
+            b.ptr = nullptr;
+            return false;
+        }
+        b.bytes = want;
+        return true;
+    };
+    if (take(align_up(bytes + (slack ? std::min<size_t>(bytes / 4, (size_t)256 << 20) : 0), 1 << 20))) return SW_OK;
+    if (!least || !alloc_between(bytes, least, take)) return SW_ERR_CUDA;
+    if (b.bytes < bytes) b.refused = bytes;
     return SW_OK;
 }
 
 // As ensure, for a call that may be captured: a buffer cannot grow while
 // the stream is capturing (the first call of a size on a stream allocates).
-int ensure_on(Buffer &b, size_t bytes, cudaStream_t st)
+// One that got less than it asked for asks again only for a smaller size, or
+// when it is too small.
+int ensure_on(Buffer &b, size_t bytes, cudaStream_t st, size_t least = 0)
 {
     if (b.bytes >= bytes) return SW_OK;
+    if (least && b.bytes >= least && b.refused && bytes >= b.refused) return SW_OK;
     if (capturing(st)) return SW_ERR_UNSUPPORTED;
-    return ensure(b, bytes);
+    return ensure(b, bytes, true, least);
 }
 
 int device_state(DeviceState **out, cudaStream_t st)
@@ -488,7 +491,7 @@ int run_batch(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const sw_scor
     Scratch S{};
     const size_t fixed_bytes = fixed_layout(n_pairs, nullptr, S);
     const int64_t bnd_bytes = std::min(kScoreBndMax, std::max(kScoreBndMin, n_pairs * kScoreBndPerPair));
-    int64_t tb_bytes = 0;
+    int64_t tb_bytes = 0, tb_least = 0;
     if (cig) {
         if (!ds->tb_cap) {
             // once per stream: a share of the memory free at its first traceback
@@ -498,9 +501,11 @@ int run_batch(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const sw_scor
                 ds->tb_cap = std::max(kTbCapMin, std::min(kTbCapMax, (int64_t)(kTbFreeShare * (double)free_b)));
         }
         tb_bytes = std::min(ds->tb_cap, std::max(kTbMin, n_pairs * kTbPerPair));
+        tb_least = std::min(ds->tb_cap, std::max(kTbLeastMin, n_pairs * kTbLeastPerPair));
     }
     if ((rc = ensure_on(ds->fixed, fixed_bytes, st))) return rc;
-    if ((rc = ensure_on(ds->dyn, (size_t)(bnd_bytes + tb_bytes), st))) return rc;
+    if ((rc = ensure_on(ds->dyn, (size_t)(bnd_bytes + tb_bytes), st, (size_t)(bnd_bytes + tb_least)))) return rc;
+    tb_bytes = std::min(tb_bytes, ((int64_t)ds->dyn.bytes - bnd_bytes) & ~(int64_t)255);
     // the block tasks' rows, with the stream's first small batch (one that is
     // captured before, or that finds the card full, runs without block tasks)
     if (n_pairs <= kSmallPairs && !ds->pipe_tried && !plan_overrides() && !capturing(st)) {
