@@ -321,23 +321,9 @@ __device__ __forceinline__ void plan_tb(const ClassInfo *info, const TbClassInfo
             int64_t slot = 0;
             if (t.count > 0) {
                 const int64_t need = ti->max_need[c] > 1 ? ti->max_need[c] : 1;
-                // Lanes per two pairs.  A batch too small to give a wave of
-                // warps tasks of 64 / T pairs spreads each two pairs over
-                // more lanes: its tasks (several blocks one after another)
-                // then finish sooner, which is what the call waits for.  The
-                // smallest run with 16 lanes in one launch; else a part takes
-                // lanes until its pairs make a wave, the narrow windows four at
-                // most unless that leaves three quarters of the warps idle
-                // (60,000 pairs of 100 x 200: 1 lane 0.58 ms, 4 lanes 0.44;
-                // 120,000: 1 lane 0.81, 2 lanes 0.63; 16,384: 4 lanes 0.16, 16
-                // lanes 0.20), and long reads follow their class's count.
-                const int64_t wave = (int64_t)pp.tb_warps[0] * 64;
-                const int64_t all = s_n16[2], same = part < 2 ? s_n16[part] : all;
-                auto enough = [&](int lanes) { return part < 2 || lanes < 4 ? wave : wave / 4; };
-                int lanes = one_launch || 16 * all < wave ? 16 : part == 0 ? 8 : 1;  // (wide windows: see kTbWide)
-                while (lanes < 16 &&
-                       (same * lanes < enough(lanes) || (info->max_m[c] > 512 && (int64_t)cnt * lanes < wave / 4)))
-                    lanes *= 2;
+                const int64_t all = s_n16[2];
+                const int lanes = tb_part_lanes(one_launch, part, all, part < 2 ? s_n16[part] : all, cnt, info->max_m[c],
+                                                pp.tb_warps[0]);
                 slot = tb_part_shape(c / N_MCLASS, pp.allow16 != 0, sp->cls_ck[c], info->max_m[c], need,
                                      ti->max_wcap[part][c], part, pp.sc, lanes, t);
                 out->part[kTbParts * c + part] = t;

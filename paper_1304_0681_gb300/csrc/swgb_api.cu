@@ -577,70 +577,6 @@ struct sw_plan {
 namespace swgb {
 namespace {
 
-// Worst-case scratch of a shape: every window may lie inside the band, so
-// a chunk window is at most the class's longest window (and smaller ones may
-// pick other traceback kernels, whose slots are bounded too).
-void plan_budgets(const ClassInfo &ci, const PlanParams &pp, bool cigar, int64_t &bnd_bytes, int64_t &tb_bytes)
-{
-    int64_t slot_s[N_SCORE_VARIANTS] = {};
-    for (int c = 0; c < N_CLASS; ++c) {
-        if (!ci.count[c]) continue;
-        const int mode = c / N_MCLASS;
-        const int32_t mm = ci.max_m[c], mn = ci.max_n[c];
-        int lanes = 1, ri = 0;
-        score_plan_of(mode, mm, (int64_t)pp.sc.ma * std::min(mm, mn), pp.ov, pp.n_overrides, lanes, ri);
-        const int rows = score_rows_at(ri);
-        if ((mm + lanes * rows - 1) / (lanes * rows) > 1) {
-            const int v = ri * N_VMODES + score_vmode(mode, (int64_t)pp.sc.ma * std::min(mm, mn), pp.sc, true);
-            slot_s[v] = std::max<int64_t>(slot_s[v], (int64_t)(32 / lanes) * 16 * mn);
-        }
-    }
-    int nb = 0;
-    int64_t per = 0;
-    for (int v = 0; v < N_SCORE_VARIANTS; ++v)
-        if (slot_s[v]) {
-            ++nb;
-            per = std::max(per, slot_s[v] * pp.score_warps[v]);
-        }
-    bnd_bytes = std::max<int64_t>(nb * (int64_t)align_up(per, 256), 256);
-    tb_bytes = 0;
-    if (!cigar) return;
-    // the row checkpoints of every class, and per traceback launch the widest
-    // slot over the classes it may serve
-    int64_t slot_v[N_TB_VARIANTS] = {}, ck = 0;
-    for (int c = 0; c < N_CLASS; ++c) {
-        if (!ci.count[c]) continue;
-        const int mode = c / N_MCLASS;
-        const int32_t mm = ci.max_m[c], mn = std::max(ci.max_n[c], 1);
-        const int64_t chunks = (mm + TB_ROWS - 1) / TB_ROWS;
-        if (pp.allow16 && mode != MODE_I32)
-            ck += 16 * std::max(ck_class_units(ci.count[c], (int64_t)ci.sum_n[c], mm, mn, 1, 40),
-                                ck_class_units(ci.count[c], (int64_t)ci.sum_n[c], mm, mn, 32, 40));
-        // the widest window, the widest of the narrow part, and the widest
-        // one-lane tile of the int32 kernels
-        const int64_t cand[3] = {mn, std::min<int64_t>(mn, kTbWide), std::min<int64_t>(mn, kTiledLaneWords / chunks)};
-        for (int64_t w : cand) {
-            if (w < 1) continue;
-            for (int lanes = w > kTbWide ? 8 : 1; lanes <= 16; lanes *= 2) {
-                TbPartPlan t{};
-                const int64_t slot = tb_part_shape(mode, pp.allow16 != 0, 64, mm, chunks * w, (int32_t)w,
-                                                   tb_part_of((int32_t)w), pp.sc, lanes, t);
-                slot_v[t.variant] = std::max(slot_v[t.variant], (slot + 63) & ~(int64_t)63);
-            }
-        }
-    }
-    const int64_t cap = kTbCapMax / 4;  // words
-    int64_t all16 = 0;  // the 16-bit launches run at once
-    for (int v = 0; v < N_TB_VARIANTS; ++v) {
-        const int64_t words = std::max(std::min(pp.tb_warps[v] * slot_v[v], cap), 4 * slot_v[v]);
-        if (v < N_TB16_VARIANTS) all16 += words;
-        else tb_bytes = std::max(tb_bytes, 4 * words);
-    }
-    tb_bytes = std::max(tb_bytes, 4 * std::min(all16, 2 * cap));
-    // the planner lets checkpoints take three quarters of the scratch
-    tb_bytes = std::max(tb_bytes + std::min(ck, kTbCapMax), (std::min(ck, kTbCapMax) + 2) / 3 * 4);
-}
-
 int plan_build(sw_plan *pl, DeviceState *ds, cudaStream_t st)
 {
     int rc = SW_OK;

@@ -163,6 +163,7 @@ struct TracebackLaunch {
 // A launch serves the variants of one kernel: those of 16 lanes, of 8 lanes,
 // then one each.
 __host__ __device__ inline int tb_launch_variants(int v) { return v == 0 || v == 2 ? 2 : 1; }
+__host__ __device__ inline int tb_launch_first(int v) { return v == 1 || v == 3 ? v - 1 : v; }
 
 // Row counts compiled for the score kernels.
 constexpr int N_SCORE_ROWS = 6;
@@ -227,6 +228,27 @@ __host__ __device__ constexpr int tb16_rows(int T) { return T == 16 ? 4 : 8; }
 constexpr int kTbWide = 256, kTbMid = 64;
 constexpr int kTbParts = 3;
 __host__ __device__ inline int tb_part_of(int32_t wc) { return wc > kTbWide ? 0 : wc > kTbMid ? 1 : 2; }
+
+// Lanes per two pairs of a part of a 16-bit class.  A batch too small to give a
+// wave of warps tasks of 64 / T pairs spreads each two pairs over more lanes: its
+// tasks (several blocks one after another) then finish sooner, which is what the
+// call waits for.  The smallest run with 16 lanes in one launch; else a part takes
+// lanes until its pairs make a wave, the narrow windows four at most unless that
+// leaves three quarters of the warps idle (60,000 pairs of 100 x 200: 1 lane 0.58
+// ms, 4 lanes 0.44; 120,000: 1 lane 0.81, 2 lanes 0.63; 16,384: 4 lanes 0.16, 16
+// lanes 0.20), and long reads follow their class's count.  all, same, cnt: pairs
+// of the 16-bit classes, of the part over all of them (of the last part: all),
+// and of the class.
+__host__ __device__ inline int tb_part_lanes(bool one_launch, int part, int64_t all, int64_t same, int64_t cnt,
+                                             int32_t m_max, int32_t warps)
+{
+    const int64_t wave = (int64_t)warps * 64;
+    int lanes = one_launch || 16 * all < wave ? 16 : part == 0 ? 8 : 1;  // (wide windows: see kTbWide)
+    while (lanes < 16 && (same * lanes < (part < 2 || lanes < 4 ? wave : wave / 4) ||
+                          (m_max > 512 && cnt * lanes < wave / 4)))
+        lanes *= 2;
+    return lanes;
+}
 constexpr int N_TB_PARTS = kTbParts * N_CLASS;
 constexpr int kMaxPlanOverrides = 16;
 constexpr int kPlanThreads = 384;                         // >= N_CLASS
