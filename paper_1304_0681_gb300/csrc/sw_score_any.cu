@@ -1,8 +1,9 @@
 // sw_score_any.cu -- the score pass of a small batch in one launch: the bodies
 // that small_body() lists, run for the variants that have classes.  255 registers,
-// so 8 warps per SM whatever runs.  Most small batches have no more tasks; one
-// with more (thousands of long reads, up to 2,048 tasks of a warp) takes the plans
-// with the fewest steps, of 20 rows or more, whose own launches hold 8 to 12.
+// so 8 warps per SM whatever runs.  Most small batches have no more tasks; one of
+// thousands of long reads (a task of a warp each, or two) does, and loses little:
+// its plans have 20 rows or more, whose own launches hold 8 to 12 warps (4,096
+// reads of 1,000 bases without a CIGAR 1.52 ms, through those launches 1.49).
 #include "sw_score_kernel.cuh"
 
 namespace swgb {

@@ -1,8 +1,8 @@
-"""The 16-bit traceback recomputes a read in blocks of 40 to 64 rows from the
-score pass's checkpoints: reads whose length, end row, gaps or start fall on
-and around the block edges, windows on both sides of the wide-window split,
-every number of lanes per two pairs, and several scorings, bit-exact against
-the oracle."""
+"""The 16-bit traceback recomputes a read in blocks of 50, 60 or 64 rows (by the
+score plan's rows per lane) from the score pass's checkpoints: reads whose
+length, end row, gaps or start fall on and around the block edges under every
+plan, windows on both sides of the wide-window split, every number of lanes per
+two pairs, and several scorings, bit-exact against the oracle."""
 import numpy as np
 import pytest
 
@@ -29,7 +29,7 @@ def _edge_pairs(rng, lengths, alphabet=4):
     out = []
     base = lambda n: rng.integers(0, alphabet, n).astype(np.uint8)  # noqa: E731
     for m in lengths:
-        for at in sorted({1, m // 2} | {e + d for e in (40, 50, 64, 100, 128) for d in (-1, 0, 1) if 0 < e + d < m - 1}):
+        for at in sorted({1, m // 2} | {e + d for e in (50, 60, 64, 100, 120, 128) for d in (-1, 0, 1) if 0 < e + d < m - 1}):
             read = base(m)
             for gap in (0, 1, 7, -1, -6, 40, 300):
                 if gap >= 0:   # window bases the read lacks
@@ -42,12 +42,29 @@ def _edge_pairs(rng, lengths, alphabet=4):
     return out
 
 
+EDGES = (39, 40, 41, 49, 50, 51, 59, 60, 61, 63, 64, 65, 81, 101, 121, 129, 151)
+
+
 @pytest.mark.parametrize("scoring", [DEFAULT, (2, -3, -5, -2), (2, -9, -4, -1), (5, -4, -10, 0), (1, -1, -2, -2)])
 def test_gaps_around_block_edges(scoring):
     rng = np.random.default_rng(17)
-    wl = _batch(_edge_pairs(rng, (39, 40, 41, 49, 50, 51, 63, 64, 65, 81, 101, 129, 151)) +
-                _edge_pairs(rng, (66, 102), alphabet=2))
+    wl = _batch(_edge_pairs(rng, EDGES) + _edge_pairs(rng, (66, 102), alphabet=2))
     assert_parity(wl, run_gpu(wl, scoring), scoring)
+
+
+@pytest.mark.parametrize("rows,block", [(8, 64), (16, 64), (20, 60), (25, 50), (32, 64), (50, 50)])
+def test_every_block_height_at_its_edges(rows, block):
+    """Each rows-per-lane choice for every read: blocks of its height."""
+    import paper_1304_0681_gb300 as sw
+    rng = np.random.default_rng(rows)
+    lengths = sorted({e + d for e in (block, 2 * block) for d in (-1, 0, 1)} | {block + 20, 2 * block + 23})
+    wl = _batch(_edge_pairs(rng, lengths) + _edge_pairs(rng, (block + 1,), alphabet=2))
+    sw.sw_set_plan(160, -(-160 // rows), rows)
+    try:
+        for scoring in (DEFAULT, (2, -3, -5, -2)):
+            assert_parity(wl, run_gpu(wl, scoring), scoring)
+    finally:
+        sw.sw_set_plan(0, 1, 8)
 
 
 def test_long_reads_and_wide_windows():
