@@ -454,8 +454,10 @@ int enqueue_core(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Scor
     if (timing && cuda_failed(cudaEventRecord(x.phase[1], st))) return SW_ERR_CUDA;
     if ((rc = fork_streams(x, st, kScoreStreams))) return rc;
     const ScoreLaunch L = score_launch(ps, sc, out_score, out_end, cig != nullptr, S);
-    for (int v = N_SCORE_VARIANTS - 1; v >= 0; --v)
+    for (int q = 0; q < N_SCORE_VARIANTS; ++q) {
+        const int v = score_launch_order(q);
         if ((rc = launch_score_variant(v, L, x.score_blocks[v], stream_at(x, st, score_variant_stream(v))))) return rc;
+    }
     if ((rc = join_streams(x, st, kScoreStreams))) return rc;
     if (timing && cuda_failed(cudaEventRecord(x.phase[2], st))) return SW_ERR_CUDA;
     if (cig) {

@@ -1,6 +1,6 @@
-"""Which stream each score launch of the general sequence goes to: launches on
-one stream run one after another, so the row counts that the long reads of a
-batch take must not share one (score_variant_stream in swgb_internal.h)."""
+"""Order and streams of the score launches of the general sequence
+(swgb_internal.h): launches on one stream run one after another, so the row
+counts that the long reads of a batch take must not share one."""
 import os
 import subprocess
 
@@ -19,11 +19,17 @@ int main()
             if (s < 0 || s >= kScoreStreams) { printf("stream %d\n", s); return 1; }
             ++used[s];
             for (int b = a + 1; b < N_SCORE_ROWS && b < a + 4; ++b)
-                if (s == score_variant_stream(b * N_VMODES + mode)) {
+                if (mode != MODE_I16 && s == score_variant_stream(b * N_VMODES + mode)) {
                     printf("mode %d: %d and %d rows on stream %d\n", mode, score_rows_at(a), score_rows_at(b), s);
                     return 1;
                 }
         }
+    bool seen[N_SCORE_VARIANTS] = {};
+    for (int q = 0; q < N_SCORE_VARIANTS; ++q) {
+        const int v = score_launch_order(q);
+        if (v < 0 || v >= N_SCORE_VARIANTS || seen[v]) { printf("launch %d: variant %d\n", q, v); return 1; }
+        seen[v] = true;
+    }
     for (int s = 0; s < kScoreStreams; ++s)
         if (!used[s]) { printf("stream %d is not used\n", s); return 1; }
     return 0;
