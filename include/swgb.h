@@ -131,7 +131,9 @@ int64_t sw_packed_bytes(int64_t n_bases);
  * would have to grow scratch during a capture returns SW_ERR_UNSUPPORTED.
  * Replays use the bases, offsets and outputs the captured call named.
  * sw_sync_status waits and reports what the kernels found (invalid device
- * input, an overflowing CIGAR slot, ...).  Scratch is bounded per call: a
+ * input, an overflowing CIGAR slot, ...).  On a card with less free memory
+ * than a call would take for its traceback it takes what there is, down to a
+ * fifth (long reads are then slower).  Scratch is bounded per call: a
  * batch whose longest pair needs more than the call's scratch for one warp
  * (far beyond the workloads of the paper, e.g. an 8,000-base read against a
  * window of a million bases) is reported as SW_ERR_UNSUPPORTED.
@@ -565,8 +567,8 @@ int sw_set_plan(int32_t max_read_len, int32_t lanes, int32_t r_rows);
  * cost model.  Without an override, a class with too few tasks for its
  * launch's warps runs with fewer rows per lane on more lanes; the query
  * reports the plan before that adjustment, which depends on the batch's pair
- * counts.  Host-only;
- * SW_ERR_INVALID_ARG for null outputs or values out of range.
+ * counts (small batches also run long reads over the warps of a block).
+ * Host-only; SW_ERR_INVALID_ARG for null outputs or values out of range.
  */
 int sw_plan_query(int32_t max_read_len, int32_t max_window_len, int32_t match, int32_t *lanes, int32_t *r_rows);
 
