@@ -421,7 +421,7 @@ int enqueue_small(const PairSet &ps, int64_t n_reads, int64_t n_pairs, const Sco
 }
 
 // Enqueues one whole batch on st: classification, the device planners,
-// every score variant (forked over the auxiliary streams), and with a CIGAR
+// every score variant (over the caller's and the auxiliary streams), and with a CIGAR
 // the traceback sort, its planner and every traceback variant.  A fixed
 // sequence of memsets and launches: no host synchronisation, no allocation.
 // expect (or nullptr): per-class counts and maxima a plan was made for.
