@@ -197,22 +197,23 @@ constexpr int N_TB_VARIANTS = 9;
 // The score launches of the general sequence fork over kScoreStreams streams.
 // Launches on one stream wait for one another, and a few long reads keep a launch
 // busy for milliseconds, so the row counts of the modes that long reads run in
-// take turns on four of them.  The fifth has the two plans of most short reads,
-// 50 and 25 rows of the 16-bit keys: nothing waits before a batch of one length,
-// and few empty launches after it.  The wide modes start first, and the most rows
-// first.  Calls without a CIGAR, with every row count of a mode on one stream, and
-// so: 200 reads of 1,000 to 4,000 bases 15.5 and 6.5 to 8.6 ms, 5,000 of 750 to
-// 3,000 24.2 and 12.3 to 14.1, 20,000 of 75 to 800 0.95 and 0.81.  (Where the last
-// tasks fall decides a few batches the other way: 34,000 pairs of 4,000 such reads
-// 0.90 and 1.12 ms, 35,000 such reads with introns 1.5 and 1.8 to 2.0.)  On eight
-// streams the kernels take as long, but the device has eight queues in all, and
-// host batches on two worker streams lost 6 % (14.6 to 13.7M reads/s).
+// take turns on four of them, and the plans that reads of 75 to 800 bases get at
+// one batch size (fewer rows the smaller it is) lie apart.  The fifth has the 50,
+// 32 and 25 rows of the 16-bit keys: nothing waits before a batch of one length of
+// short reads, and few empty launches after it.  The wide modes start first, and
+// the most rows first.  Calls without a CIGAR, with every row count of a mode on
+// one stream, and so: 200 reads of 1,000 to 4,000 bases 15.5 and 6.5 to 8.6 ms,
+// 5,000 of 750 to 3,000 24.3 and 12.3 to 14.0, 20,000 of 75 to 800 0.95 and 0.81.
+// (Where the last tasks fall decides a few batches the other way: 35,000 such
+// reads with introns 1.5 and 2.1 ms.)  On eight streams the kernels take as long,
+// but the device has eight queues in all, and host batches on two worker streams
+// lost 6 % (14.6 to 13.7M reads/s).
 constexpr int kScoreStreams = 5;
 inline int score_variant_stream(int v)
 {
-    const int rows = v / N_VMODES, mode = v % N_VMODES;
-    if (mode == MODE_I16) return rows == 3 || rows == 5 ? 4 : rows % 4;
-    return (rows + (mode == MODE_I16S) + 2 * (mode == MODE_I32)) % 4;
+    constexpr int8_t stream[N_SCORE_ROWS][N_VMODES] = {  // by rows; int32, 16-bit keys, wide, wide with the fp16 add
+        {2, 2, 0, 0}, {3, 1, 1, 1}, {0, 3, 2, 0}, {1, 4, 3, 2}, {2, 4, 0, 1}, {3, 4, 1, 2}};
+    return stream[v / N_VMODES][v % N_VMODES];
 }
 // The variant that is launched as number q.
 inline int score_launch_order(int q)
@@ -220,7 +221,7 @@ inline int score_launch_order(int q)
     constexpr int W = MODE_I16W, S = MODE_I16S, K = MODE_I16, I = MODE_I32;
     constexpr struct { int8_t rows, mode; } order[N_SCORE_VARIANTS] = {
         {5, W}, {4, W}, {3, W}, {2, W}, {1, W}, {0, W}, {5, S}, {4, S}, {3, S}, {2, S}, {1, S}, {0, S},
-        {5, K}, {3, K}, {5, I}, {4, I}, {3, I}, {2, I}, {1, I}, {0, I}, {4, K}, {2, K}, {1, K}, {0, K}};
+        {5, K}, {3, K}, {4, K}, {2, K}, {1, K}, {0, K}, {5, I}, {4, I}, {3, I}, {2, I}, {1, I}, {0, I}};
     return order[q].rows * N_VMODES + order[q].mode;
 }
 __host__ __device__ inline int tb16_variant_lanes(int v) { return v < 2 ? 16 : v < 4 ? 8 : 64 >> v; }

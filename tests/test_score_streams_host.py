@@ -18,7 +18,7 @@ int main()
             const int s = score_variant_stream(a * N_VMODES + mode);
             if (s < 0 || s >= kScoreStreams) { printf("stream %d\n", s); return 1; }
             ++used[s];
-            for (int b = a + 1; b < N_SCORE_ROWS && b < a + 4; ++b)
+            for (int b = a + 1; b < N_SCORE_ROWS && b < a + (mode == MODE_I16S ? 2 : 4); ++b)
                 if (mode != MODE_I16 && s == score_variant_stream(b * N_VMODES + mode)) {
                     printf("mode %d: %d and %d rows on stream %d\n", mode, score_rows_at(a), score_rows_at(b), s);
                     return 1;
